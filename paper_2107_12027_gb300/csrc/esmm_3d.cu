@@ -232,16 +232,11 @@ __global__ void k3_cfl(Geom3 g, double gam, const double *__restrict__ q, const 
             double m[3];
             for (int a = 0; a < 3; ++a) m[a] = q[(F_M + 3 * d + a) * g.P + c];
             double Lk = sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
-            double nn[3] = {m[0] / Lk, m[1] / Lk, m[2] / Lk}, T[3][3], wr[8], lam[8], R[8][8];
+            double nn[3] = {m[0] / Lk, m[1] / Lk, m[2] / Lk}, T[3][3], wr[8], lo, hi;
             frame3(nn, T);
             rot3(T, w, wr);
-            eigen_mhd(gam, wr, lam, R, false);
-            double a = 0.0, lo = lam[0], hi = lam[0];
-            for (int mm = 0; mm < 8; ++mm) {
-                a = fmax(a, fabs(lam[mm]));
-                lo = fmin(lo, lam[mm]);
-                hi = fmax(hi, lam[mm]);
-            }
+            mhd_speed_range<double>(gam, wr, lo, hi);
+            const double a = fmax(fabs(lo), fabs(hi));
             r[d] = Lk * a * iJ;
             if (cflb) {
                 cflb[(3 + d) * g.N + id] = Lk * lo * iJ;

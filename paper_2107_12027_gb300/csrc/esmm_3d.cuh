@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(128) k3_iface(Geom3 g, Phys ph, const double *
         align3(T, wm);
         rot3(T, wm, wrot);
         double lam[8], R[8][8];
-        eigen_mhd(ph.gamma, wrot, lam, R, true);
+        eigen_mhd<double>(ph.gamma, wrot, lam, R);
         double lhat = 0.0;
 #pragma unroll
         for (int m = 0; m < 8; ++m) lhat = fmax(lhat, fabs(jt + Lk * lam[m]));

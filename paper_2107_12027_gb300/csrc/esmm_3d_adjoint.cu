@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(128) k3_iface_vjp(Geom3 g, Phys ph, const doub
     }
     rot3(T, wm, wrot);
     double lam[8], R[8][8];
-    eigen_mhd<double>(ph.gamma, wrot, lam, R, true);
+    eigen_mhd_gram<double>(ph.gamma, wrot, lam, R, true);
     double lhat = 0.0;
     int msel = 0;
     for (int m = 0; m < 8; ++m) {
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(128) k3_iface_vjp(Geom3 g, Phys ph, const doub
     for (int a = 0; a < 8; ++a) {
         dual wd[8], lamd[8], Rd[8][8];
         for (int k = 0; k < 8; ++k) wd[k] = dual(wrot[k], k == a ? 1.0 : 0.0);
-        eigen_mhd<dual>(ph.gamma, wd, lamd, Rd, true);
+        eigen_mhd_gram<dual>(ph.gamma, wd, lamd, Rd, true);
         double acc = -0.5 * sg * Lk * lamd[msel].d * zeta;
         for (int b = 0; b < 8; ++b)
             for (int m = 0; m < 8; ++m) acc += Rbar[b][m] * Rd[b][m].d;

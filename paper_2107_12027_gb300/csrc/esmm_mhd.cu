@@ -26,9 +26,9 @@ __global__ void k_prim_out_mhd(ProbArg pa, double gam, const double *__restrict_
 
 
 // Spectral radius of the 8-wave system per node and direction (eq. cfl),
-// with the speeds from the eigen-system in the working precision R (FP32 in
-// the mixed form: the step carries ~1e-6 relative rounding, harmless for a
-// stability bound).
+// the fast speeds in the working precision R (FP32 in the mixed form: the step
+// carries ~1e-6 relative rounding, harmless for a stability bound).  The roots
+// of their quartic replace a whole eigen-system per node and direction.
 // With cflb (the moving-mesh step) also the speed bounds L_k lambda_min/J and
 // L_k lambda_max/J of every node into its rows 2 + k and 4 + k.
 template <typename R>
@@ -55,14 +55,9 @@ __global__ void k_cfl_mhd(ProbArg pa, double gam, const double *__restrict__ q, 
             double nx = mx / Lk, ny = my / Lk;
             R wr[8] = {(R)w[0], (R)(nx * w[1] + ny * w[2]), (R)(-ny * w[1] + nx * w[2]), (R)w[3],
                        (R)w[4], (R)(nx * w[5] + ny * w[6]), (R)(-ny * w[5] + nx * w[6]), (R)w[7]};
-            R lam[8], Rm[8][8];
-            eigen_mhd<R>(gam, wr, lam, Rm, false);
-            double a = 0.0, lo = (double)lam[0], hi = (double)lam[0];
-            for (int m = 0; m < 8; ++m) {
-                a = fmax(a, fabs((double)lam[m]));
-                lo = fmin(lo, (double)lam[m]);
-                hi = fmax(hi, (double)lam[m]);
-            }
+            R l0, l1;
+            mhd_speed_range<R>(gam, wr, l0, l1);
+            const double lo = (double)l0, hi = (double)l1, a = fmax(fabs(lo), fabs(hi));
             r[k] = owned_row(g, j) ? Lk * a * iJ : 0.0;
             if (cflb) {
                 cflb[6 * D.on + (2 + k) * g.N + id] = Lk * lo * iJ;

@@ -273,7 +273,7 @@ __device__ __forceinline__ void jacobi6(S C[6][6], S Q[6][6], bool want_vectors)
 }
 
 template <typename R>
-static __device__ __noinline__ void eigen_mhd(double gam, const R w[8], R lam[8], R Rv[8][8], bool want_vectors)
+static __device__ __noinline__ void eigen_mhd_gram(double gam, const R w[8], R lam[8], R Rv[8][8], bool want_vectors)
 {
     R Pp[8];
     mhd_phiprime(w, Pp);
@@ -469,6 +469,210 @@ static __device__ __noinline__ void eigen_mhd(double gam, const R w[8], R lam[8]
             Rv[r][2 + m] = acc;
         }
     });
+}
+
+}  // namespace esmm
+
+#include "esmm_mhd_waves.cuh"
+
+namespace esmm {
+
+// The canonical basis of the clusters (consecutive speeds closer than
+// MHD_CLUSTER_TOL) among the six waves, whose columns of Rv it replaces: with
+// G = L L^T the Gram matrix of the y_a of eigen_mhd_gram and S[a][m] the wave
+// m's coefficients in them, E = L^T S are the waves in C-space; the basis is the
+// Gram-Schmidt of the unit vectors projected on the cluster's span, as there.
+template <typename R>
+static __device__ __noinline__ void mhd_canonical(double gam, const R w[8], const R lam[8], R S[6][6], R Rv[8][8])
+{
+    R Pp[8];
+    mhd_phiprime(w, Pp);
+    const R v1 = w[1];
+    R a_rho[8] = {(R)1, (R)0, (R)0, (R)0, (R)0, (R)0, (R)0, (R)0};
+    R a_div[8] = {(R)0, (R)0, (R)0, (R)0, (R)0, (R)1 - v1 * v1, -v1 * w[2], -v1 * w[3]};
+    R Ur[8], Vr[8], Ud[8], Vd[8], Fx[8];
+    mhd_images(gam, w, a_rho, Pp, Ur, Vr, Fx);
+    mhd_images(gam, w, a_div, Pp, Ud, Vd, Fx);
+    const R in_rho = rcp<R>(dot8(Ur, Vr)), in_div = rcp<R>(dot8(Ud, Vd));
+    const int comp[6] = {1, 2, 3, 4, 6, 7};
+    R Uy[6][8], Vy[6][8], Gm[6][6], idg[6];
+#pragma unroll 1
+    for (int a = 0; a < 6; ++a) {
+        R e[8] = {(R)0, (R)0, (R)0, (R)0, (R)0, (R)0, (R)0, (R)0};
+        e[comp[a]] = (R)1;
+        R Ue[8], Ve[8];
+        mhd_images(gam, w, e, Pp, Ue, Ve, Fx);
+        const R cr = dot8(Ue, Vr) * in_rho, cd = dot8(Ue, Vd) * in_div;
+        for (int r = 0; r < 8; ++r) {
+            Uy[a][r] = Ue[r] - cr * Ur[r] - cd * Ud[r];
+            Vy[a][r] = Ve[r] - cr * Vr[r] - cd * Vd[r];
+        }
+        // y_a of unit <y_a, y_a> (E is unchanged by the scaling)
+        const R sa = rsq<R>(dot8(Uy[a], Vy[a])), isa = rcp<R>(sa);
+        for (int r = 0; r < 8; ++r) {
+            Uy[a][r] *= sa;
+            Vy[a][r] *= sa;
+        }
+        for (int m = 0; m < 6; ++m) S[a][m] *= isa;
+    }
+    for (int a = 0; a < 6; ++a)
+        for (int b = 0; b <= a; ++b) Gm[a][b] = (R)0.5 * (dot8(Uy[a], Vy[b]) + dot8(Uy[b], Vy[a]));
+    for (int j = 0; j < 6; ++j) {
+        R d = Gm[j][j];
+        for (int k = 0; k < j; ++k) d -= Gm[j][k] * Gm[j][k];
+        if constexpr (sizeof(R) == 4)
+            if (!(d > (R)1.0e-12)) d = (R)1.0e-12;   // FP32: keep the factor finite
+        idg[j] = rsq<R>(d);
+        Gm[j][j] = d * idg[j];
+        for (int i = j + 1; i < 6; ++i) {
+            R s = Gm[i][j];
+            for (int k = 0; k < j; ++k) s -= Gm[i][k] * Gm[j][k];
+            Gm[i][j] = s * idg[j];
+        }
+    }
+    int start = 0;
+    while (start < 6) {
+        int end = start + 1;
+        while (end < 6 && lam[2 + end] - lam[1 + end] < (R)MHD_CLUSTER_TOL) ++end;
+        const int k = end - start;
+        if (k > 1) {
+            // E = L^T S, orthonormalized (twice: the waves of a cluster may be
+            // oblique at rounding level over their gap)
+            R E[6][6], z[6][6];
+            for (int c = 0; c < k; ++c) {
+                for (int i = 0; i < 6; ++i) {
+                    R acc = (R)0;
+                    for (int j = i; j < 6; ++j) acc += Gm[j][i] * S[j][start + c];
+                    E[i][c] = acc;
+                }
+                for (int pass = 0; pass < 2; ++pass)
+                    for (int b = 0; b < c; ++b) {
+                        R pr = (R)0;
+                        for (int i = 0; i < 6; ++i) pr += E[i][b] * E[i][c];
+                        for (int i = 0; i < 6; ++i) E[i][c] -= pr * E[i][b];
+                    }
+                R n2 = (R)0;
+                for (int i = 0; i < 6; ++i) n2 += E[i][c] * E[i][c];
+                const R inr = rsq<R>(n2);
+                for (int i = 0; i < 6; ++i) E[i][c] *= inr;
+            }
+            R basis[6][6];
+            for (int i = 0; i < 6; ++i)
+                for (int c = 0; c < k; ++c) z[i][c] = E[i][c];
+            int nt = 0;
+            for (int i = 0; i < 6 && nt < k; ++i) {
+                R n2 = (R)0;
+                for (int c = 0; c < k; ++c) n2 += z[i][c] * z[i][c];
+                if (!(n2 >= (R)0.125)) continue;
+                const R inr = rsq<R>(n2);
+                for (int c = 0; c < k; ++c) basis[nt][c] = z[i][c] * inr;
+                for (int ii = i + 1; ii < 6; ++ii) {
+                    R pr = (R)0;
+                    for (int c = 0; c < k; ++c) pr += z[ii][c] * basis[nt][c];
+                    for (int c = 0; c < k; ++c) z[ii][c] -= pr * basis[nt][c];
+                }
+                ++nt;
+            }
+            for (int t = 0; t < nt && nt == k; ++t) {   // (nt < k: non-finite input)
+                R s[6];
+                for (int i = 5; i >= 0; --i) {
+                    R acc = (R)0;
+                    for (int c = 0; c < k; ++c) acc += E[i][c] * basis[t][c];
+                    for (int j = i + 1; j < 6; ++j) acc -= Gm[j][i] * s[j];
+                    s[i] = acc * idg[i];
+                }
+                for (int r = 0; r < 8; ++r) {
+                    R acc = (R)0;
+                    for (int a = 0; a < 6; ++a) acc += s[a] * Uy[a][r];
+                    Rv[r][2 + start + t] = acc;
+                }
+            }
+        }
+        start = end;
+    }
+}
+
+// The eigen-system of eigen_mhd_gram from the waves in closed form
+// (esmm_mhd_waves.cuh); clusters get their canonical basis, and states whose
+// coefficients leave the FP32 range of the root estimates take the Gram path.
+template <typename R>
+static __device__ __noinline__ void eigen_mhd(double gam, const R w[8], R lam[8], R Rv[8][8])
+{
+    const R gg = (R)(gam / (gam - 1.0));
+    MhdBase<R> s;
+    mhd_base<R>((R)gam, gg, w, s);
+    const R lim = (R)(sizeof(R) == 4 ? 1.0e-12 : 1.0e-25);
+    if (!(s.gp > lim && s.e < (R)1 / lim)) {
+        eigen_mhd_gram<R>(gam, w, lam, Rv, true);
+        return;
+    }
+    MhdSix<R> x;
+    lam[0] = lam[1] = s.v1;
+    mhd_six<R>(s, x, lam + 2);
+    bool cluster = false;
+#pragma unroll
+    for (int m = 0; m < 5; ++m) cluster = cluster || lam[3 + m] - lam[2 + m] < (R)MHD_CLUSTER_TOL;
+    // the entropy wave d rho = 1 and the divergence wave dB = e_1 - v_1 v
+    {
+        const R sr = rsq<R>(gg * s.W * rcp<R>(s.rho));
+        Rv[0][0] = s.W * sr;
+        for (int k = 0; k < 3; ++k) Rv[1 + k][0] = s.W * s.u[1 + k] * sr;
+        Rv[4][0] = s.W * s.W * sr;
+        for (int k = 5; k < 8; ++k) Rv[k][0] = (R)0;
+        MhdWave<R> q;
+        const R dB[3] = {(R)1 - s.v1 * s.v1, -s.v1 * w[2], -s.v1 * w[3]};
+        q.rho = q.p = (R)0;
+        q.b[0] = s.v1 * s.iW;
+        q.u[0] = (R)0;
+        for (int k = 0; k < 3; ++k) {
+            q.u[1 + k] = (R)0;
+            q.b[1 + k] = (dB[k] + q.b[0] * s.u[1 + k]) * s.iW;
+        }
+        const R sd = rsq<R>(s.beta * s.W * mdot<R>(q.b, q.b));
+        for (int k = 0; k < 4; ++k) q.b[k] *= sd;
+        R dU[8];
+        mhd_wave_dU<R>(s, gg, q, dU);
+        for (int r = 0; r < 8; ++r) Rv[r][1] = dU[r];
+    }
+    R S[6][6];
+#pragma unroll 1
+    for (int m = 0; m < 6; ++m) {
+        MhdWave<R> q;
+        mhd_six_wave<R>(s, x, m, q);
+        R dU[8];
+        mhd_wave_dU<R>(s, gg, q, dU);
+        for (int r = 0; r < 8; ++r) Rv[r][2 + m] = dU[r];
+        if (cluster) {   // the wave's coefficients in the y_a
+            for (int k = 0; k < 3; ++k) S[k][m] = (q.u[1 + k] - w[1 + k] * q.u[0]) * s.iW;
+            S[3][m] = q.p;
+            const R ga = -dU[5] * rcp<R>((R)1 - s.v1 * s.v1);
+            S[4][m] = dU[6] - ga * s.v1 * w[2];
+            S[5][m] = dU[7] - ga * s.v1 * w[3];
+        }
+    }
+    if (cluster) mhd_canonical<R>(gam, w, lam, S, Rv);
+}
+// the smallest and largest speed (the fast waves) at the rotated state w: the
+// CFL radius needs no vectors
+template <typename R>
+static __device__ __noinline__ void mhd_speed_range(double gam, const R w[8], R &lo, R &hi)
+{
+    MhdBase<R> s;
+    mhd_base<R>((R)gam, (R)(gam / (gam - 1.0)), w, s);
+    const R lim = (R)(sizeof(R) == 4 ? 1.0e-12 : 1.0e-25);
+    if (!(s.gp > lim && s.e < (R)1 / lim)) {
+        R lam[8], Rm[8][8];
+        eigen_mhd_gram<R>(gam, w, lam, Rm, false);
+        lo = lam[2];
+        hi = lam[7];
+        return;
+    }
+    const R sqe = sq_rt<R>(s.e);
+    R tA, ts, tf;
+    mhd_side<R>(s, sqe, 1, false, tA, ts, tf);
+    lo = s.v1 - tf * s.iW;
+    mhd_side<R>(s, sqe, -1, false, tA, ts, tf);
+    hi = s.v1 + tf * s.iW;
 }
 
 // ---------------------------------------------------------------------------
@@ -795,7 +999,7 @@ __global__ void __launch_bounds__(128) k_iface_mhd(ProbArg pa, Phys ph, const do
             wrot[7] = wm[7];
         }
         R lam[8], Rm[8][8];
-        eigen_mhd<R>(ph.gamma, wrot, lam, Rm, true);
+        eigen_mhd<R>(ph.gamma, wrot, lam, Rm);
         R lhat = (R)0;
 #pragma unroll
         for (int m = 0; m < 8; ++m) lhat = vmax(lhat, fab<R>(jt + Lk * lam[m]));

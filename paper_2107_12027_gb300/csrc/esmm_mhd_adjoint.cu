@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(128) k_iface_vjp_mhd(ProbArg pa, Phys ph, cons
         wrot[7] = wm[7];
     }
     double lam[8], R[8][8];
-    eigen_mhd<double>(ph.gamma, wrot, lam, R, true);
+    eigen_mhd_gram<double>(ph.gamma, wrot, lam, R, true);
     double lhat = 0.0;
     int msel = 0;
     for (int m = 0; m < 8; ++m) {
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(128) k_iface_vjp_mhd(ProbArg pa, Phys ph, cons
     for (int a = 0; a < 8; ++a) {
         dual wd[8], lamd[8], Rd[8][8];
         for (int k = 0; k < 8; ++k) wd[k] = dual(wrot[k], k == a ? 1.0 : 0.0);
-        eigen_mhd<dual>(ph.gamma, wd, lamd, Rd, true);
+        eigen_mhd_gram<dual>(ph.gamma, wd, lamd, Rd, true);
         double acc = -0.5 * sg * Lk * lamd[msel].d * zeta;
         for (int b = 0; b < 8; ++b)
             for (int m = 0; m < 8; ++m) acc += Rbar[b][m] * Rd[b][m].d;
@@ -515,7 +515,7 @@ __global__ void k_eigen_mhd(double gam, int n, const double *__restrict__ w, con
     if (!dw) {
         double wk[8], l[8], Rk[8][8];
         for (int a = 0; a < 8; ++a) wk[a] = w[8 * k + a];
-        eigen_mhd<double>(gam, wk, l, Rk, true);
+        eigen_mhd_gram<double>(gam, wk, l, Rk, true);
         for (int a = 0; a < 8; ++a) {
             lam[8 * k + a] = l[a];
             for (int b = 0; b < 8; ++b) R[64 * k + 8 * a + b] = Rk[a][b];
@@ -524,7 +524,7 @@ __global__ void k_eigen_mhd(double gam, int n, const double *__restrict__ w, con
     }
     dual wk[8], l[8], Rk[8][8];
     for (int a = 0; a < 8; ++a) wk[a] = dual(w[8 * k + a], dw[8 * k + a]);
-    eigen_mhd<dual>(gam, wk, l, Rk, true);
+    eigen_mhd_gram<dual>(gam, wk, l, Rk, true);
     for (int a = 0; a < 8; ++a) {
         lam[8 * k + a] = l[a].v;
         dlam[8 * k + a] = l[a].d;
