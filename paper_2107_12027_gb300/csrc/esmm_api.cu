@@ -1354,8 +1354,7 @@ int rhs_vjp_core(esmm_grid *g, const double *cons, const double *J, const double
         CK(cudaGetLastError());
         return ESMM_OK;
     }
-    CK(cudaMemsetAsync(g->adjG, 0, ADJ_G_PER_NODE * P * d, g->st));
-    CK(cudaMemsetAsync(g->adjGp, 0, ADJ_GP_PER_NODE * P * d, g->st));
+    // (the pair and interface passes write every contribution the node pass reads)
     CK(cudaMemsetAsync(lam, 0, 4 * N * d, g->st));
     Phys ph = phys(g);
     for (int dir = 0; dir < 2; ++dir) {

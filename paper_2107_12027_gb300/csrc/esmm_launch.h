@@ -119,7 +119,7 @@ int mhd_eigen_host(double gam, int n, const double *w, const double *dw, double 
                    double *dR);
 
 // sizes of the adjoint's contribution buffers, in doubles per padded node
-constexpr long long ADJ_G_PER_NODE = 2 * 6 * 7;
+constexpr long long ADJ_G_PER_NODE = 2 * (6 * 4 + 7);
 constexpr long long ADJ_GP_PER_NODE = 2 * PMAX * 2 * 7;
 
 }  // namespace esmm
