@@ -786,11 +786,14 @@ int rhs_vjp_core3(esmm3 *g, const double *cons, const double *J, const double *x
 {
     size_t N = (size_t)g->g.N, P = (size_t)g->g.P, d = sizeof(double);
     node3(g, cons, J, x, xdot, nullptr, nullptr);
-    fluxes3(g);   // the Powell term's div B~
     CK3(cudaMemsetAsync(g->lamq, 0, 11 * P * d, g->st));
     CK3(cudaMemsetAsync(lam, 0, 8 * N * d, g->st));
     Phys ph = phys3(g);
     for (int dir = 0; dir < 3; ++dir) {
+        {
+            Prof3 pr_(g, ESMM_KIND_IFACE);   // the Powell term's div B~
+            launch3_bflux(g->g, ph, g->q, g->iflux, dir, g->st);
+        }
         {
             Prof3 pr_(g, ESMM_KIND_PAIRS);
             launch3_pairs_vjp(g->g, ph, g->q, mu, g->lamq, dir, g->st);

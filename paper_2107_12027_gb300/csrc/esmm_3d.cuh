@@ -349,6 +349,7 @@ void launch3_pairs_vjp(const Geom3 &g, const Phys &ph, const double *q, const do
                        cudaStream_t st);
 void launch3_iface_vjp(const Geom3 &g, const Phys &ph, const double *q, const double *mu, double *lamq, int dir,
                        cudaStream_t st);
+void launch3_bflux(const Geom3 &g, const Phys &ph, const double *q, double *iflux, int dir, cudaStream_t st);
 void launch3_node_vjp(const Geom3 &g, double gam, const double *q, const double *lamq, const double *iflux,
                       const double *mu, const double *J, double *lam, cudaStream_t st);
 void launch3_prim_grad(const Geom3 &g, double gam, const double *cons, const double *J, const double *lam,

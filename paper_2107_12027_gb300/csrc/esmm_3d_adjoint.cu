@@ -12,13 +12,12 @@
 //   phi = atan2(t2.B, t1.B) with (t1, t2) the rows before the turn,
 // and the adjoint adds d(objective)/d(phi) d(phi)/d(interface state).
 #include "esmm_3d.cuh"
+#include "esmm_mhd_vjp.cuh"
 
 namespace esmm {
 namespace d3 {
 
 namespace {
-
-enum { A_RHO = 0, A_BETA, A_LNR, A_LNB, A_W, A_U0, A_U1, A_U2, A_B0, A_B1, A_B2, NQN };
 
 __device__ __forceinline__ bool inside3(const Geom3 &g, const int c[3])
 {
@@ -59,36 +58,6 @@ __device__ void lambda_face3(const Geom3 &g, const double *__restrict__ q, const
     lb = mu_phi3(g, q, mu, c1) - mu_phi3(g, q, mu, c);
 }
 
-__device__ __forceinline__ NodeMT<dual> load3_dual(const double *__restrict__ q, long long P, long long c)
-{
-    NodeMT<dual> v;
-    v.rho = dual(q[F_RHO * P + c]);
-    v.beta = dual(q[F_BETA * P + c]);
-    v.lnr = dual(q[F_LNR * P + c]);
-    v.lnb = dual(q[F_LNB * P + c]);
-    v.r = v.rho;
-    v.b = v.beta;
-    v.W = dual(q[F_W * P + c]);
-    for (int a = 0; a < 3; ++a) {
-        v.u[a] = dual(q[(F_U0 + a) * P + c]);
-        v.B[a] = dual(q[(F_B0 + a) * P + c]);
-    }
-    return v;
-}
-
-__device__ __forceinline__ void seed3(NodeMT<dual> &v, int k)
-{
-    switch (k) {
-    case A_RHO: v.rho.d = 1.0; v.r.d = 1.0; break;
-    case A_BETA: v.beta.d = 1.0; v.b.d = 1.0; break;
-    case A_LNR: v.lnr.d = 1.0; break;
-    case A_LNB: v.lnb.d = 1.0; break;
-    case A_W: v.W.d = 1.0; break;
-    case A_U0: case A_U1: case A_U2: v.u[k - A_U0].d = 1.0; break;
-    default: v.B[k - A_B0].d = 1.0; break;
-    }
-}
-
 __device__ __forceinline__ void addq(double *lamq, long long P, int k, long long c, double v)
 {
     if (v != 0.0) atomicAdd(lamq + k * P + c, v);
@@ -118,7 +87,7 @@ __global__ void __launch_bounds__(128) k3_pairs_vjp(Geom3 g, Phys ph, const doub
     const long long sd = dir == 0 ? 1 : (dir == 1 ? (long long)g.pd[0] : (long long)g.pd[0] * g.pd[1]);
     const double *Mt = q + (F_MT + dir) * g.P;
     const double *Md = q + (F_M + 3 * dir) * g.P;
-    const dual gm1inv = dual(1.0 / (ph.gamma - 1.0));
+    const double gm1inv = 1.0 / (ph.gamma - 1.0);
     const int A = c3[dir];
     for (int n = 1; n <= P; ++n) {
         double lp[8] = {0, 0, 0, 0, 0, 0, 0, 0}, lbs = 0.0;
@@ -145,25 +114,13 @@ __global__ void __launch_bounds__(128) k3_pairs_vjp(Geom3 g, Phys ph, const doub
         double mmv[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) mmv[a] = 0.5 * (Md[a * g.P + c0] + Md[a * g.P + cr]);
-        // B~ of the pair: 1/2 sum_a mm_a (B_a,l + B_a,r)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            addq(lamq, g.P, A_B0 + a, c0, lbs * 0.5 * mmv[a]);
-            addq(lamq, g.P, A_B0 + a, cr, lbs * 0.5 * mmv[a]);
+        double gl[NQN], gr[NQN];
+        mhd_pair_vjp(load3(q, g.P, c0), load3(q, g.P, cr), gm1inv, ph.ln_thr, 0.5 * (Mt[c0] + Mt[cr]), mmv, lp, lbs,
+                     gl, gr);
+        for (int k = 0; k < NQN; ++k) {
+            addq(lamq, g.P, k, c0, gl[k]);
+            addq(lamq, g.P, k, cr, gr[k]);
         }
-        const dual mt = dual(0.5 * (Mt[c0] + Mt[cr]));
-        const dual mm[3] = {dual(mmv[0]), dual(mmv[1]), dual(mmv[2])};
-        for (int side = 0; side < 2; ++side)
-            for (int k = 0; k < NQN; ++k) {
-                NodeMT<dual> l = load3_dual(q, g.P, c0), r = load3_dual(q, g.P, cr);
-                seed3(side ? r : l, k);
-                dual out[8];
-                ec_pair_mhd<3, dual>(l, r, gm1inv, ph.ln_thr, mt, mm, out);
-                double gsum = 0.0;
-#pragma unroll
-                for (int a = 0; a < 8; ++a) gsum += lp[a] * out[a].d;
-                addq(lamq, g.P, k, side ? cr : c0, gsum);
-            }
     }
 }
 
@@ -180,10 +137,10 @@ __global__ void __launch_bounds__(128) k3_iface_vjp(Geom3 g, Phys ph, const doub
                                                     const double *__restrict__ mu, double *__restrict__ lamq, int dir)
 {
     constexpr int NS = WW + 1, OFF = (WW - 1) / 2;
-    const int nd = g.n[dir];
     const int oa = dir == 0 ? 1 : 0, ob = dir == 2 ? 1 : 2;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)(nd + 1) * g.n[oa] * g.n[ob]) return;
+    if (idx >= (long long)(g.n[dir] + 1) * g.n[oa] * g.n[ob]) return;
+    const int nd = g.n[dir];
     int c3[3];
     sweep_index(g, dir, nd, 1, idx, c3);
     double lf[8], lbdummy;
@@ -244,85 +201,19 @@ __global__ void __launch_bounds__(128) k3_iface_vjp(Geom3 g, Phys ph, const doub
         }
     }
     rot3(T, wm, wrot);
-    double lam[8], R[8][8];
-    eigen_mhd_gram<double>(ph.gamma, wrot, lam, R, true);
-    double lhat = 0.0;
-    int msel = 0;
-    for (int m = 0; m < 8; ++m) {
-        const double v = fabs(jt + Lk * lam[m]);
-        if (v > lhat) { lhat = v; msel = m; }
-    }
-    const double sg = (jt + Lk * lam[msel]) >= 0.0 ? 1.0 : -1.0;
     const double ig = 1.0 / (ph.gamma - 1.0), c1g = ph.gamma * ig;
-    double TV[NS][8], Vt[NS][8], scale[8];
-    for (int m = 0; m < 8; ++m) scale[m] = 0.0;
+    double TV[NS][8], lrot[8], gTV[NS][8], gw[8], Rz[8], hl;
     for (int k = 0; k < NS; ++k) {
         double V[8];
         node_V3(q, g.P, c0 + (k - OFF) * sd, c1g, ig, V);
         rot3(T, V, TV[k]);
-        for (int m = 0; m < 8; ++m) {
-            double acc = 0.0;
-            for (int a = 0; a < 8; ++a) {
-                const double t = R[a][m] * TV[k][a];
-                acc += t;
-                if (k == OFF || k == OFF + 1) scale[m] += fabs(t);
-            }
-            Vt[k][m] = acc;
-        }
     }
-    double z[8];
-    bool ym[8];
-    for (int m = 0; m < 8; ++m) {
-        double vminus, vplus;
-        if (WW == 5)
-            weno5_lr<double>(Vt[0][m], Vt[1][m], Vt[2][m], Vt[3][m], Vt[4][m], Vt[5][m], ph.eps, vminus, vplus);
-        else
-            weno3_lr<double>(Vt[0][m], Vt[1][m], Vt[2][m], Vt[3][m], ph.eps, vminus, vplus);
-        const double jw = vplus - vminus;
-        const double jump = Vt[OFF + 1][m] - Vt[OFF][m];
-        const int sj = fabs(jump) <= ph.sign_tol * scale[m] ? 0 : sgn_d(jump);
-        ym[m] = sgn_d(jw) == sj;
-        z[m] = ym[m] ? jw : 0.0;
-    }
-    // reverse: objective contribution -hl lrot . (R z), lrot = rot3(T, lambda_F)
-    double lrot[8];
     rot3(T, lf, lrot);
-    const double hl = 0.5 * lhat;
-    double zeta = 0.0, qm[8], Rz[8];
-    for (int b = 0; b < 8; ++b) {
-        double a = 0.0;
-        for (int m = 0; m < 8; ++m) a += R[b][m] * z[m];
-        Rz[b] = a;
-    }
-    for (int m = 0; m < 8; ++m) {
-        double a = 0.0;
-        for (int b = 0; b < 8; ++b) a += R[b][m] * lrot[b];
-        qm[m] = -hl * a;
-        zeta += a * z[m];
-    }
-    double lVt[NS][8];
-    const dual epsd = dual(ph.eps);
-    for (int k = 0; k < NS; ++k) {
-        dual s[NS];
-        for (int m = 0; m < 8; ++m) {
-            for (int kk = 0; kk < NS; ++kk) s[kk] = dual(Vt[kk][m], kk == k ? 1.0 : 0.0);
-            dual vminus, vplus;
-            if (WW == 5)
-                weno5_lr<dual>(s[0], s[1], s[2], s[3], s[4], s[5], epsd, vminus, vplus);
-            else
-                weno3_lr<dual>(s[0], s[1], s[2], s[3], epsd, vminus, vplus);
-            lVt[k][m] = ym[m] ? qm[m] * (vplus.d - vminus.d) : 0.0;
-        }
-    }
+    mhd_diss_vjp<WW>(ph, wrot, Lk, jt, lrot, TV, gTV, gw, Rz, hl);
     // stencil nodes
     for (int k = 0; k < NS; ++k) {
-        double lT[8], lV[8];
-        for (int b = 0; b < 8; ++b) {
-            double a = 0.0;
-            for (int m = 0; m < 8; ++m) a += R[b][m] * lVt[k][m];
-            lT[b] = a;
-        }
-        unrot3(T, lT, lV);
+        double lV[8];
+        unrot3(T, gTV[k], lV);
         const long long ck = c0 + (k - OFF) * sd;
         const double beta = q[F_BETA * g.P + ck], W = q[F_W * g.P + ck];
         const double u[3] = {q[F_U0 * g.P + ck], q[F_U1 * g.P + ck], q[F_U2 * g.P + ck]};
@@ -350,24 +241,6 @@ __global__ void __launch_bounds__(128) k3_iface_vjp(Geom3 g, Phys ph, const doub
             addq(lamq, g.P, A_B0 + l, ck, lB[l]);
         }
     }
-    // interface state, through the eigen-system
-    double Rbar[8][8];
-    for (int b = 0; b < 8; ++b)
-        for (int m = 0; m < 8; ++m) {
-            double a = -hl * lrot[b] * z[m];
-            for (int k = 0; k < NS; ++k) a += lVt[k][m] * TV[k][b];
-            Rbar[b][m] = a;
-        }
-    double gw[8];
-    for (int a = 0; a < 8; ++a) {
-        dual wd[8], lamd[8], Rd[8][8];
-        for (int k = 0; k < 8; ++k) wd[k] = dual(wrot[k], k == a ? 1.0 : 0.0);
-        eigen_mhd_gram<dual>(ph.gamma, wd, lamd, Rd, true);
-        double acc = -0.5 * sg * Lk * lamd[msel].d * zeta;
-        for (int b = 0; b < 8; ++b)
-            for (int m = 0; m < 8; ++m) acc += Rbar[b][m] * Rd[b][m].d;
-        gw[a] = acc;
-    }
     double gwm[8];
     unrot3(T, gw, gwm);
     // ... and through the frame's angle
@@ -379,11 +252,7 @@ __global__ void __launch_bounds__(128) k3_iface_vjp(Geom3 g, Phys ph, const doub
         for (int a = 0; a < 8; ++a) gphi += gw[a] * d8[a];
         for (int k = 0; k < NS; ++k) {
             dphi8(TV[k], d8);
-            for (int m = 0; m < 8; ++m) {
-                double dv = 0.0;
-                for (int b = 0; b < 8; ++b) dv += R[b][m] * d8[b];
-                gphi += lVt[k][m] * dv;
-            }
+            for (int b = 0; b < 8; ++b) gphi += gTV[k][b] * d8[b];
         }
         // phi = atan2(tb2, tb1), tb_i = (row i of the unturned frame) . (B or v)
         for (int qq = 0; qq < 3; ++qq) gwm[fo + qq] += gphi * (tb1 * T0[2][qq] - tb2 * T0[1][qq]) / tt2;
@@ -418,6 +287,35 @@ __global__ void __launch_bounds__(128) k3_iface_vjp(Geom3 g, Phys ph, const doub
             addq(lamq, g.P, A_B0 + k, c1, 0.5 * gwm[5 + k]);
         }
     }
+}
+
+// B~ alone (row 9 of a direction's interface values), for the Powell term's div B~
+template <int P>
+__global__ void k3_bflux(Geom3 g, Phys ph, const double *__restrict__ q, double *__restrict__ iflux, int dir)
+{
+    const int nd = g.n[dir];
+    const int oa = dir == 0 ? 1 : 0, ob = dir == 2 ? 1 : 2;
+    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (long long)(nd + 1) * g.n[oa] * g.n[ob]) return;
+    int c3[3];
+    sweep_index(g, dir, nd, 1, idx, c3);
+    const long long c0 = pidx3(g, c3[0], c3[1], c3[2]);
+    const long long sd = dir == 0 ? 1 : (dir == 1 ? (long long)g.pd[0] : (long long)g.pd[0] * g.pd[1]);
+    const double *Md = q + (F_M + 3 * dir) * g.P, *B = q + F_B0 * g.P;
+    double Bt = 0.0;
+#pragma unroll
+    for (int n = 1; n <= P; ++n) {
+        double Bts = 0.0;
+#pragma unroll
+        for (int s = 0; s < n; ++s) {
+            const long long cl = c0 - s * sd, cr = cl + n * sd;
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+                Bts += 0.25 * (Md[a * g.P + cl] + Md[a * g.P + cr]) * (B[a * g.P + cl] + B[a * g.P + cr]);
+        }
+        Bt += ph.alpha[n - 1] * Bts;
+    }
+    iflux[(long long)(dir * NF3 + 9) * g.P + c0] = Bt;
 }
 
 __device__ void dUdw3(double gam, const double w[8], double A[8][8])
@@ -564,6 +462,15 @@ void launch3_iface_vjp(const Geom3 &g, const Phys &ph, const double *q, const do
     const unsigned nb = nbk((long long)(g.n[dir] + 1) * g.n[oa] * g.n[ob]);
     if (ph.w == 5) k3_iface_vjp<5><<<nb, 128, 0, st>>>(g, ph, q, mu, lamq, dir);
     else if (ph.w == 3) k3_iface_vjp<3><<<nb, 128, 0, st>>>(g, ph, q, mu, lamq, dir);
+}
+
+void launch3_bflux(const Geom3 &g, const Phys &ph, const double *q, double *iflux, int dir, cudaStream_t st)
+{
+    const int oa = dir == 0 ? 1 : 0, ob = dir == 2 ? 1 : 2;
+    const unsigned nb = nbk((long long)(g.n[dir] + 1) * g.n[oa] * g.n[ob]);
+    if (ph.p == 1) k3_bflux<1><<<nb, 128, 0, st>>>(g, ph, q, iflux, dir);
+    else if (ph.p == 2) k3_bflux<2><<<nb, 128, 0, st>>>(g, ph, q, iflux, dir);
+    else k3_bflux<3><<<nb, 128, 0, st>>>(g, ph, q, iflux, dir);
 }
 
 void launch3_node_vjp(const Geom3 &g, double gam, const double *q, const double *lamq, const double *iflux,

@@ -1331,19 +1331,22 @@ int rhs_vjp_core(esmm_grid *g, const double *cons, const double *J, const double
     size_t P = (size_t)g->Ptot, N = (size_t)g->Ntot, d = sizeof(double);
     node(g, cons, J, x, xdot, nullptr, nullptr);
     if (g->phys == ESMM_RMHD) {
-        // forward interface fluxes first: the Powell term needs div B~
-        fluxes(g);
         CK(cudaMemsetAsync(g->adjG, 0, ADJ_LAMQ_PER_NODE * P * d, g->st));
         CK(cudaMemsetAsync(lam, 0, 8 * N * d, g->st));
         Phys ph = phys(g);
         for (int dir = 0; dir < 2; ++dir) {
+            const LaunchDom Li = dom(g, dir ? D_IFACE1 : D_IFACE0);
+            {
+                Prof pr_(g, ESMM_KIND_IFACE);   // the Powell term needs div B~
+                launch_bflux_mhd(Li, ph, g->q, (double *)g->iflux, dir, g->st);
+            }
             {
                 Prof pr_(g, ESMM_KIND_PAIRS);
                 launch_pairs_vjp_mhd(dom(g, dir ? D_PAIR1 : D_PAIR0), ph, g->q, mu, g->adjG, dir, g->st);
             }
             if (g->w > 0) {
                 Prof pr_(g, ESMM_KIND_IFACE);
-                launch_iface_vjp_mhd(dom(g, dir ? D_IFACE1 : D_IFACE0), ph, g->q, mu, g->adjG, dir, g->st);
+                launch_iface_vjp_mhd(Li, ph, g->q, mu, g->adjG, dir, g->st);
             }
         }
         {

@@ -109,6 +109,8 @@ void launch_pairs_vjp_mhd(const LaunchDom &L, const Phys &ph, const double *q, c
                           int dir, cudaStream_t st);
 void launch_iface_vjp_mhd(const LaunchDom &L, const Phys &ph, const double *q, const double *mu, double *lamq,
                           int dir, cudaStream_t st);
+// the magnetic flux B~ alone into row 9 of the direction's interface values
+void launch_bflux_mhd(const LaunchDom &L, const Phys &ph, const double *q, double *iflux, int dir, cudaStream_t st);
 void launch_node_vjp_mhd(const LaunchDom &L, double gam, const double *q, const double *lamq, const double *iflux,
                          const double *mu, const double *J, double *lam, cudaStream_t st);
 void launch_prim_grad_mhd(const LaunchDom &L, double gam, const double *cons, const double *J, const double *lam,

@@ -10,12 +10,10 @@
 //   lambda_F = mu_{L+1} - mu_L for the interface fluxes, and
 //   lambda_B = mu_{L+1}.Phi'_{L+1} - mu_L.Phi'_L for the magnetic flux B~ of
 //   the Powell source;
-//   per node pair: dual numbers seeded at one of 11 node quantities give the
-//   two-point flux's Jacobian-vector products;
-//   per interface: a reverse sweep of the dissipation (WENO weights through
-//   dual numbers per stencil position, Y frozen), and the eigen-system's
-//   tangent along each of the 8 interface-state directions (eigen_mhd<dual>:
-//   perturbation theory on the Jacobi result, cluster spans kept);
+//   per node pair: a reverse sweep of the two-point flux (esmm_mhd_vjp.cuh);
+//   per interface: a reverse sweep of the dissipation (Y frozen) with first-order
+//   perturbation theory on the waves, the rotation of the canonical basis of
+//   clustered speeds included;
 //   per node: the Powell term's own dependence on v and B, the chain rule to
 //   the primitives w, and the implicit-function adjoint of the Newton
 //   recovery, lambda_U = (dU/dw)^-T lambda_w; lambda_cons += lambda_U / J.
@@ -23,12 +21,11 @@
 // padded grid; ghost nodes fold into their source node in the node pass.
 #include "esmm_launch.h"
 #include "esmm_mhd.cuh"
+#include "esmm_mhd_vjp.cuh"
 
 namespace esmm {
 
 namespace {
-
-enum { A_RHO = 0, A_BETA, A_LNR, A_LNB, A_W, A_U0, A_U1, A_U2, A_B0, A_B1, A_B2, NQN };
 
 __device__ __forceinline__ bool inside(const Geom &g, int i, int j)
 {
@@ -63,19 +60,6 @@ __device__ void lambda_face_mhd(const Geom &g, const double *__restrict__ q, con
     lb = mu_phi(g, q, mu, i1, j1) - mu_phi(g, q, mu, i, j);
 }
 
-__device__ __forceinline__ void seed_m(NodeMT<dual> &v, int k)
-{
-    switch (k) {
-    case A_RHO: v.rho.d = 1.0; v.r.d = 1.0; break;
-    case A_BETA: v.beta.d = 1.0; v.b.d = 1.0; break;
-    case A_LNR: v.lnr.d = 1.0; break;
-    case A_LNB: v.lnb.d = 1.0; break;
-    case A_W: v.W.d = 1.0; break;
-    case A_U0: case A_U1: case A_U2: v.u[k - A_U0].d = 1.0; break;
-    default: v.B[k - A_B0].d = 1.0; break;
-    }
-}
-
 __device__ __forceinline__ void add_q(double *lamq, long long P, int k, long long c, double v)
 {
     if (v != 0.0) atomicAdd(lamq + k * P + c, v);
@@ -103,7 +87,7 @@ __global__ void __launch_bounds__(128) k_pairs_vjp_mhd(ProbArg pa, Phys ph, cons
     const double *Mt = q + (Q_MT0 + dir) * g.P;
     const double *Mx = q + (Q_M00 + 2 * dir) * g.P;
     const double *My = q + (Q_M01 + 2 * dir) * g.P;
-    const dual gm1inv = dual(1.0 / (ph.gamma - 1.0));
+    const double gm1inv = 1.0 / (ph.gamma - 1.0);
     const int A = dir == 0 ? i : j;
     for (int n = 1; n <= P; ++n) {
         double lp[8] = {0, 0, 0, 0, 0, 0, 0, 0}, lbs = 0.0;
@@ -126,31 +110,20 @@ __global__ void __launch_bounds__(128) k_pairs_vjp_mhd(ProbArg pa, Phys ph, cons
         lbs *= an;
         if (!any) continue;
         const long long cr = c0 + n * sd;
-        // B~ of the pair: 1/4 (Mx_l + Mx_r)(B1_l + B1_r) + 1/4 (My_l + My_r)(B2_l + B2_r)
-        const double bx = 0.25 * (Mx[c0] + Mx[cr]), by = 0.25 * (My[c0] + My[cr]);
-        add_q(lamq, g.P, A_B0, c0, lbs * bx);
-        add_q(lamq, g.P, A_B0, cr, lbs * bx);
-        add_q(lamq, g.P, A_B1, c0, lbs * by);
-        add_q(lamq, g.P, A_B1, cr, lbs * by);
-        const dual mt = dual(0.5 * (Mt[c0] + Mt[cr]));
-        const dual mm[3] = {dual(0.5 * (Mx[c0] + Mx[cr])), dual(0.5 * (My[c0] + My[cr])), dual(0.0)};
-        for (int side = 0; side < 2; ++side)
-            for (int k = 0; k < NQN; ++k) {
-                NodeMT<dual> l = load_node_m<dual>(q, g.P, c0), r = load_node_m<dual>(q, g.P, cr);
-                seed_m(side ? r : l, k);
-                dual out[8];
-                ec_pair_mhd<2, dual>(l, r, gm1inv, ph.ln_thr, mt, mm, out);
-                double gsum = 0.0;
-#pragma unroll
-                for (int a = 0; a < 8; ++a) gsum += lp[a] * out[a].d;
-                add_q(lamq, g.P, k, side ? cr : c0, gsum);
-            }
+        const double mm[3] = {0.5 * (Mx[c0] + Mx[cr]), 0.5 * (My[c0] + My[cr]), 0.0};
+        double gl[NQN], gr[NQN];
+        mhd_pair_vjp(load_node_m<double>(q, g.P, c0), load_node_m<double>(q, g.P, cr), gm1inv, ph.ln_thr,
+                     0.5 * (Mt[c0] + Mt[cr]), mm, lp, lbs, gl, gr);
+        for (int k = 0; k < NQN; ++k) {
+            add_q(lamq, g.P, k, c0, gl[k]);
+            add_q(lamq, g.P, k, cr, gr[k]);
+        }
     }
 }
 
 // The ES dissipation of one interface (eq. ESFlux_HO; F = F_EC - diss), in
 // reverse: its adjoint with respect to the stencil nodes' entropy variables
-// and to the interface state (through the eigen-system's tangents).
+// and to the interface state (mhd_diss_vjp).
 template <int WW>
 __global__ void __launch_bounds__(128) k_iface_vjp_mhd(ProbArg pa, Phys ph, const double *__restrict__ q,
                                                        const double *__restrict__ mu, double *__restrict__ lamq,
@@ -210,18 +183,8 @@ __global__ void __launch_bounds__(128) k_iface_vjp_mhd(ProbArg pa, Phys ph, cons
         wrot[6] = -ny * wm[5] + nx * wm[6];
         wrot[7] = wm[7];
     }
-    double lam[8], R[8][8];
-    eigen_mhd_gram<double>(ph.gamma, wrot, lam, R, true);
-    double lhat = 0.0;
-    int msel = 0;
-    for (int m = 0; m < 8; ++m) {
-        const double v = fabs(jt + Lk * lam[m]);
-        if (v > lhat) { lhat = v; msel = m; }
-    }
-    const double sg = (jt + Lk * lam[msel]) >= 0.0 ? 1.0 : -1.0;
     const double ig = 1.0 / (ph.gamma - 1.0), c1g = ph.gamma * ig;
-    double TV[NS][8], Vt[NS][8], scale[8];
-    for (int m = 0; m < 8; ++m) scale[m] = 0.0;
+    double TV[NS][8];
     for (int k = 0; k < NS; ++k) {
         double V[8];
         node_V_mhd<double>(q, g.P, c0 + (k - OFF) * sd, c1g, ig, V);
@@ -233,65 +196,14 @@ __global__ void __launch_bounds__(128) k_iface_vjp_mhd(ProbArg pa, Phys ph, cons
         TV[k][5] = nx * V[5] + ny * V[6];
         TV[k][6] = -ny * V[5] + nx * V[6];
         TV[k][7] = V[7];
-        for (int m = 0; m < 8; ++m) {
-            double acc = 0.0;
-            for (int a = 0; a < 8; ++a) {
-                const double t = R[a][m] * TV[k][a];
-                acc += t;
-                if (k == OFF || k == OFF + 1) scale[m] += fabs(t);
-            }
-            Vt[k][m] = acc;
-        }
     }
-    double z[8];
-    bool ym[8];
-    for (int m = 0; m < 8; ++m) {
-        double vminus, vplus;
-        if (WW == 5)
-            weno5_lr<double>(Vt[0][m], Vt[1][m], Vt[2][m], Vt[3][m], Vt[4][m], Vt[5][m], ph.eps, vminus, vplus);
-        else
-            weno3_lr<double>(Vt[0][m], Vt[1][m], Vt[2][m], Vt[3][m], ph.eps, vminus, vplus);
-        const double jw = vplus - vminus;
-        const double jump = Vt[OFF + 1][m] - Vt[OFF][m];
-        const int sj = fabs(jump) <= ph.sign_tol * scale[m] ? 0 : sgn_d(jump);
-        ym[m] = sgn_d(jw) == sj;
-        z[m] = ym[m] ? jw : 0.0;
-    }
-    // reverse: objective contribution -hl lrot . (R z), lrot = T lambda_F
-    double lrot[8] = {lf[0], nx * lf[1] + ny * lf[2], -ny * lf[1] + nx * lf[2], lf[3],
-                      lf[4], nx * lf[5] + ny * lf[6], -ny * lf[5] + nx * lf[6], lf[7]};
-    const double hl = 0.5 * lhat;
-    double zeta = 0.0, qm[8];
-    for (int m = 0; m < 8; ++m) {
-        double a = 0.0;
-        for (int b = 0; b < 8; ++b) a += R[b][m] * lrot[b];
-        qm[m] = -hl * a;
-        zeta += a * z[m];
-    }
-    // WENO partials d z_m / d Vt[k][m] (the fields are independent, so one
-    // dual pass per stencil position serves all eight)
-    double lVt[NS][8];
-    const dual epsd = dual(ph.eps);
-    for (int k = 0; k < NS; ++k) {
-        dual s[NS];
-        for (int m = 0; m < 8; ++m) {
-            for (int kk = 0; kk < NS; ++kk) s[kk] = dual(Vt[kk][m], kk == k ? 1.0 : 0.0);
-            dual vminus, vplus;
-            if (WW == 5)
-                weno5_lr<dual>(s[0], s[1], s[2], s[3], s[4], s[5], epsd, vminus, vplus);
-            else
-                weno3_lr<dual>(s[0], s[1], s[2], s[3], epsd, vminus, vplus);
-            lVt[k][m] = ym[m] ? qm[m] * (vplus.d - vminus.d) : 0.0;
-        }
-    }
+    const double lrot[8] = {lf[0], nx * lf[1] + ny * lf[2], -ny * lf[1] + nx * lf[2], lf[3],
+                            lf[4], nx * lf[5] + ny * lf[6], -ny * lf[5] + nx * lf[6], lf[7]};
+    double gTV[NS][8], gw[8], Rz[8], hl;
+    mhd_diss_vjp<WW>(ph, wrot, Lk, jt, lrot, TV, gTV, gw, Rz, hl);
     // stencil nodes: lambda of V_k, then of the node quantities V depends on
     for (int k = 0; k < NS; ++k) {
-        double lT[8];
-        for (int b = 0; b < 8; ++b) {
-            double a = 0.0;
-            for (int m = 0; m < 8; ++m) a += R[b][m] * lVt[k][m];
-            lT[b] = a;
-        }
+        const double *lT = gTV[k];
         const double lV[8] = {lT[0], nx * lT[1] - ny * lT[2], ny * lT[1] + nx * lT[2], lT[3],
                               lT[4], nx * lT[5] - ny * lT[6], ny * lT[5] + nx * lT[6], lT[7]};
         const long long ck = c0 + (k - OFF) * sd;
@@ -322,24 +234,6 @@ __global__ void __launch_bounds__(128) k_iface_vjp_mhd(ProbArg pa, Phys ph, cons
             add_q(lamq, g.P, A_U0 + l, ck, lu[l]);
             add_q(lamq, g.P, A_B0 + l, ck, lB[l]);
         }
-    }
-    // interface state: tangents of (lam, R) along each rotated-state direction
-    double Rbar[8][8];
-    for (int b = 0; b < 8; ++b)
-        for (int m = 0; m < 8; ++m) {
-            double a = -hl * lrot[b] * z[m];
-            for (int k = 0; k < NS; ++k) a += lVt[k][m] * TV[k][b];
-            Rbar[b][m] = a;
-        }
-    double gw[8];
-    for (int a = 0; a < 8; ++a) {
-        dual wd[8], lamd[8], Rd[8][8];
-        for (int k = 0; k < 8; ++k) wd[k] = dual(wrot[k], k == a ? 1.0 : 0.0);
-        eigen_mhd_gram<dual>(ph.gamma, wd, lamd, Rd, true);
-        double acc = -0.5 * sg * Lk * lamd[msel].d * zeta;
-        for (int b = 0; b < 8; ++b)
-            for (int m = 0; m < 8; ++m) acc += Rbar[b][m] * Rd[b][m].d;
-        gw[a] = acc;
     }
     // wrot = T wm
     const double gm_[8] = {gw[0], nx * gw[1] - ny * gw[2], ny * gw[1] + nx * gw[2], gw[3],
@@ -378,6 +272,38 @@ __global__ void __launch_bounds__(128) k_iface_vjp_mhd(ProbArg pa, Phys ph, cons
             add_q(lamq, g.P, A_B0 + k, c1, 0.5 * gm_[5 + k]);
         }
     }
+}
+
+// The magnetic flux B~ alone (eqs. BFlux_O2p / BFlux_O2), row 9 of a direction's
+// interface values: the Powell term's div B~ needs no other flux.
+template <int P>
+__global__ void k_bflux_mhd(ProbArg pa, Phys ph, const double *__restrict__ q, double *__restrict__ iflux, int dir)
+{
+    ProbDesc D;
+    long long lb_;
+    locate(pa, D, lb_);
+    const Geom &g = D.g;
+    const int nd = dir == 0 ? g.nx : g.ny, no = dir == 0 ? g.ny : g.nx;
+    const long long idx = lb_ * blockDim.x + threadIdx.x;
+    if (idx >= (long long)(nd + 1) * no) return;
+    int i, j;
+    if (dir == 0) { j = (int)(idx / (nd + 1)); i = (int)(idx % (nd + 1)) - 1; }
+    else { i = (int)(idx % no); j = (int)(idx / no) - 1; }
+    const long long c0 = pidx(g, i, j), sd = dir == 0 ? 1 : g.px;
+    const double *Mx = q + (Q_M00 + 2 * dir) * g.P, *My = q + (Q_M01 + 2 * dir) * g.P;
+    const double *B1 = q + QM_B1 * g.P, *B2 = q + QM_B2 * g.P;
+    double Bt = 0.0;
+#pragma unroll
+    for (int n = 1; n <= P; ++n) {
+        double Bts = 0.0;
+#pragma unroll
+        for (int s = 0; s < n; ++s) {
+            const long long cl = c0 - s * sd, cr = cl + n * sd;
+            Bts += 0.25 * (Mx[cl] + Mx[cr]) * (B1[cl] + B1[cr]) + 0.25 * (My[cl] + My[cr]) * (B2[cl] + B2[cr]);
+        }
+        Bt += ph.alpha[n - 1] * Bts;
+    }
+    iflux[(long long)(dir * NFM + 9) * g.P + c0] = Bt;
 }
 
 // dU/dw at the primitive state w (column c = derivative along w_c)
@@ -572,6 +498,13 @@ void launch_iface_vjp_mhd(const LaunchDom &L, const Phys &ph, const double *q, c
 {
     if (ph.w == 5) k_iface_vjp_mhd<5><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, mu, lamq, dir);
     else if (ph.w == 3) k_iface_vjp_mhd<3><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, mu, lamq, dir);
+}
+
+void launch_bflux_mhd(const LaunchDom &L, const Phys &ph, const double *q, double *iflux, int dir, cudaStream_t st)
+{
+    if (ph.p == 1) k_bflux_mhd<1><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, iflux, dir);
+    else if (ph.p == 2) k_bflux_mhd<2><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, iflux, dir);
+    else k_bflux_mhd<3><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, iflux, dir);
 }
 
 void launch_node_vjp_mhd(const LaunchDom &L, double gam, const double *q, const double *lamq, const double *iflux,
