@@ -57,9 +57,9 @@ __device__ __forceinline__ void ec_pair_vjp(const NodeV<double> &l, const NodeV<
                                             double gr[NQA])
 {
     double rln, irln, bln, ibln;
-    logmean<double, double>(l.rho, r.rho, l.lnr, r.lnr, thr, rln, irln);
-    logmean<double, double>(l.beta, r.beta, l.lnb, r.lnb, thr, bln, ibln);
-    const double rm = 0.5 * (l.r + r.r), bm = 0.5 * (l.b + r.b), W = 0.5 * (l.W + r.W);
+    logmean2<double>(l.rho, r.rho, thr, rln, irln);
+    logmean2<double>(l.beta, r.beta, thr, bln, ibln);
+    const double rm = 0.5 * (l.rho.v + r.rho.v), bm = 0.5 * (l.beta.v + r.beta.v), W = 0.5 * (l.W + r.W);
     const double ux = 0.5 * (l.ux + r.ux), uy = 0.5 * (l.uy + r.uy);
     const double usq = ux * ux + uy * uy, Lam = W * W - usq, alpha0 = 1.0 + gm1inv * ibln;
     const double ibm = __drcp_rn(bm), pm = rm * ibm, rinv = __drcp_rn(Lam * W), iLam = rinv * W, iW = rinv * Lam;
@@ -91,8 +91,8 @@ __device__ __forceinline__ void ec_pair_vjp(const NodeV<double> &l, const NodeV<
     gl[3] = gr[3] = 0.5 * gW;
     gl[4] = gr[4] = gl[5] = gr[5] = 0.0;
     gl[6] = gr[6] = hr;
-    logmean_vjp(l.rho, r.rho, l.lnr, r.lnr, thr, grln, gl[6], gr[6], gl[4], gr[4]);
-    logmean_vjp(l.beta, r.beta, l.lnb, r.lnb, thr, -gA * rln * gm1inv * ibln * ibln, gl[0], gr[0], gl[5], gr[5]);
+    logmean_vjp(l.rho.v, r.rho.v, l.rho.l, r.rho.l, thr, grln, gl[6], gr[6], gl[4], gr[4]);
+    logmean_vjp(l.beta.v, r.beta.v, l.beta.l, r.beta.l, thr, -gA * rln * gm1inv * ibln * ibln, gl[0], gr[0], gl[5], gr[5]);
 }
 
 // Adjoint contributions of the pair fluxes anchored at A: the pair (A, A+n)
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(128) k_iface_vjp(ProbArg pa, Phys ph, const do
         a_[side] = a; dvn_[side] = dvn; dvt_[side] = dvt; vdv_[side] = vdv; drho_[side] = drho;
     }
     // projections and jumps; then their adjoints
-    QStencil<double> st{q, g.P, c0, sd, OFF};
+    NodeStencil<double, QGet> st{{q, g.P, c0, sd, OFF}};
     double TV[NS][4], aT[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
     for (int k = 0; k < NS; ++k) {

@@ -67,12 +67,10 @@ __device__ void node_state(double rho, double vx, double vy, double p, cnt st[6]
     st[3] = cnt(W);
     st[4] = cnt(log(rho));
     st[5] = cnt(log(beta));
-    nv.rho = cnt(rho);
-    nv.beta = cnt(beta);
-    nv.lnr = st[4];
-    nv.lnb = st[5];
-    nv.r = cnt(rho);
-    nv.b = cnt(beta);
+    nv.rho.v = cnt(rho);
+    nv.rho.l = st[4];
+    nv.beta.v = cnt(beta);
+    nv.beta.l = st[5];
     nv.ux = st[1];
     nv.uy = st[2];
     nv.W = st[3];
@@ -84,6 +82,7 @@ __global__ void k_count_rhd(double gamma, int w, unsigned long long *out)
     Phys ph;
     ph.gamma = gamma;
     ph.gm1i = 1.0 / (gamma - 1.0);
+    ph.igg = (gamma - 1.0) / gamma;
     ph.eps = 1e-6;
     ph.ln_thr = 1e-4;
     ph.sign_tol = 1e-10;
@@ -96,18 +95,16 @@ __global__ void k_count_rhd(double gamma, int w, unsigned long long *out)
     g_nops = 0;
     ec_pair<cnt>(nv[2], nv[3], cnt(0.05), cnt(1.1), cnt(0.1), cnt(ph.gm1i), ph.ln_thr, f);
     out[0] = g_nops;
-    cnt diss[4];
+    cnt diss[4] = {cnt(0.0), cnt(0.0), cnt(0.0), cnt(0.0)};
     g_nops = 0;
     if (w == 5) {
-        ArrStencil<cnt, 6> s{st};
-        es_dissipation<cnt, cnt, 5>(cnt(1.1), cnt(0.1), cnt(0.05), nv[2].rho, nv[3].rho, nv[2].lnr, nv[3].lnr,
-                                    nv[2].r, nv[3].r, s, ph, diss);
+        NodeStencil<cnt, ArrGet<cnt>> s{{st}};
+        es_dissipation<cnt, 5>(cnt(1.1), cnt(0.1), cnt(0.05), nv[2].rho, nv[3].rho, s, ph, diss);
     } else {
-        ArrStencil<cnt, 4> s{st + 1};
-        es_dissipation<cnt, cnt, 3>(cnt(1.1), cnt(0.1), cnt(0.05), nv[2].rho, nv[3].rho, nv[2].lnr, nv[3].lnr,
-                                    nv[2].r, nv[3].r, s, ph, diss);
+        NodeStencil<cnt, ArrGet<cnt>> s{{st + 1}};
+        es_dissipation<cnt, 3>(cnt(1.1), cnt(0.1), cnt(0.05), nv[2].rho, nv[3].rho, s, ph, diss);
     }
-    out[1] = g_nops;
+    out[1] = g_nops - 4;   // (its subtraction from the flux counts in ops[2])
 }
 
 }  // namespace

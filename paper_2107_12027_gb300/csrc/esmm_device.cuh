@@ -8,6 +8,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "esmm_conv.h"
 
 namespace esmm {
@@ -125,6 +127,7 @@ __device__ __forceinline__ double to_f64(float x) { return f2d_int(x); }
 struct Phys {
     double gamma;
     double gm1i;      // 1 / (Gamma - 1), once per launch
+    double igg;       // (Gamma - 1) / Gamma
     double eps;       // WENO epsilon
     double ln_thr;    // log-mean series switch on ((b-a)/(b+a))^2
     double sign_tol;  // relative size below which [[V~]] counts as zero
@@ -427,6 +430,49 @@ template <> __device__ __forceinline__ hdual rsq<hdual>(hdual x)
     return hchain(x, r, -0.5 * r * ir, 0.75 * r * ir * ir);
 }
 template <typename R> __device__ __forceinline__ R sqrt_pos(R x) { return x * rsq<R>(x); }
+
+// a b + c in one rounding, and a - b not contracted with what forms or uses them (left to
+// itself the compiler contracts by what it sees in a basic block, so that two kernels
+// inlining one function may round differently)
+template <typename R> __device__ __forceinline__ R fma_(R a, R b, R c) { return a * b + c; }
+template <> __device__ __forceinline__ double fma_<double>(double a, double b, double c) { return __fma_rn(a, b, c); }
+template <> __device__ __forceinline__ float fma_<float>(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
+template <typename R> __device__ __forceinline__ R sub_(R a, R b) { return a - b; }
+template <> __device__ __forceinline__ double sub_<double>(double a, double b) { return __dsub_rn(a, b); }
+template <> __device__ __forceinline__ float sub_<float>(float a, float b) { return __fsub_rn(a, b); }
+
+// Reciprocal of a non-zero and reciprocal square root of a positive normal finite
+// number, within about an ulp: the hardware's first approximation (error below 2^-20
+// in FP64, 2^-22 in FP32) and one correction by the series of 1/(1-e) and
+// (1-e)^-1/2 in its residual e (Householder's iteration of third order in FP64, of
+// second order in FP32).  In FP64 that is 3 and 5 FP64 instructions, against about 7
+// and 10 of the correctly rounded reciprocal and of rsqrt, whose special cases (zero,
+// infinite, subnormal arguments) these leave out: here they give a NaN.
+template <typename R> __device__ __forceinline__ R qrcp(R x) { return rcp<R>(x); }
+template <typename R> __device__ __forceinline__ R qrsq(R x) { return rsq<R>(x); }
+#if defined(__CUDA_ARCH__)
+template <> __device__ __forceinline__ double qrcp<double>(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = __fma_rn(-x, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+template <> __device__ __forceinline__ float qrcp<float>(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return __fmaf_rn(r, __fmaf_rn(-x, r, 1.0f), r);
+}
+template <> __device__ __forceinline__ double qrsq<double>(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+    return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
+}
+#endif
 template <typename R> __device__ __forceinline__ R fab(R x);
 template <> __device__ __forceinline__ double fab<double>(double x) { return fabs(x); }
 template <> __device__ __forceinline__ float fab<float>(float x) { return fabsf(x); }
@@ -487,11 +533,63 @@ __device__ __forceinline__ void lmean<float, double>(double a, double b, double 
     }
 }
 
+// An argument of the RHD log means: the value and its logarithm, in FP32 with the
+// rest of the FP64 value, so that the jump of two near-equal values keeps FP32
+// relative precision without FP64 arithmetic: (b.v - a.v) is exact within a factor 2
+// of each other, and v + lo carries 48 bits.
+template <typename R> struct LmV { R v, l; };
+template <> struct LmV<float> { float v, lo, l; };
+__device__ __forceinline__ LmV<float> lmv_f32(double x, float v, float l)
+{
+    LmV<float> a;
+    a.v = v;
+    a.lo = d2f_int(x - f2d_int(v));
+    a.l = l;
+    return a;
+}
+__device__ __forceinline__ float to_f32(double x) { return d2f_int(x); }
+__device__ __forceinline__ float to_f32(float x) { return x; }
+
+// Logarithmic mean (b - a)/(ln b - ln a) and its reciprocal; near-equal arguments,
+// |b - a| < sqrt(thr) (a + b), by the Ismail-Roe series F = 1 + u/3 + u^2/5 + u^3/7 in
+// u = ((b-a)/(b+a))^2: inverse 2F/(a+b), mean (a+b)/2 times the series of 1/F (their
+// dropped terms are below u^4/9).  The switch is taken in FP32 (both branches hold
+// there; FP64 compares cost FP64-pipe slots).
+template <typename R>
+__device__ __forceinline__ void logmean2(const LmV<R> &a, const LmV<R> &b, double thr, R &mean, R &inv_mean)
+{
+    R d, s;
+    bool near;
+    if constexpr (std::is_same<R, float>::value) {
+        d = (b.v - a.v) + (b.lo - a.lo);
+        s = b.v + a.v;
+        near = d * d < (float)thr * (s * s);
+    } else {
+        d = b.v - a.v;
+        s = b.v + a.v;
+        if constexpr (std::is_same<R, double>::value) {
+            const float d32 = d2f_int(d), s32 = d2f_int(s);
+            near = s32 > 1.0e-30f ? fabsf(d32) < sqrtf((float)thr) * s32 : d * d < thr * s * s;
+        } else {
+            near = val(d * d) < val(thr * s * s);
+        }
+    }
+    if (near) {
+        const R is = qrcp<R>(s), r = d * is, u = r * r;
+        mean = (R)0.5 * s * ((R)1 + u * ((R)(-1.0 / 3.0) + u * ((R)(-4.0 / 45.0) + u * (R)(-44.0 / 945.0))));
+        inv_mean = (R)2 * is * ((R)1 + u * ((R)(1.0 / 3.0) + u * ((R)(1.0 / 5.0) + u * (R)(1.0 / 7.0))));
+    } else {
+        const R dl = b.l - a.l;
+        mean = d * qrcp<R>(dl);
+        inv_mean = dl * qrcp<R>(d);
+    }
+}
+
 // Node values of one two-point flux argument (the parameter variables).
 template <typename R>
 struct NodeV {
-    typename LogT<R>::type rho, beta, lnr, lnb;  // log-mean arguments (FP64 unless dual)
-    R r, b, ux, uy, W;
+    LmV<R> rho, beta;
+    R ux, uy, W;
 };
 
 // Curvilinear two-point EC flux of Sec. 3.1 for one node pair in direction k:
@@ -511,19 +609,17 @@ __device__ __forceinline__ void ec_pair(const NodeV<R> &l, const NodeV<R> &r, R 
                                         R gm1inv, double thr, R out[4])
 {
     R rln, irln, bln, ibln;
-    lmean<R, typename LogT<R>::type>(l.rho, r.rho, l.lnr, r.lnr, l.r, r.r, thr, rln, irln);
-    lmean<R, typename LogT<R>::type>(l.beta, r.beta, l.lnb, r.lnb, l.b, r.b, thr, bln, ibln);
+    logmean2<R>(l.rho, r.rho, thr, rln, irln);
+    logmean2<R>(l.beta, r.beta, thr, bln, ibln);
     R half = (R)0.5;
-    R rm = half * (l.r + r.r);
-    R bm = half * (l.b + r.b);
     R Wm = half * (l.W + r.W);
     R uxm = half * (l.ux + r.ux);
     R uym = half * (l.uy + r.uy);
     R usq = uxm * uxm + uym * uym;
     R Lam = Wm * Wm - usq;
     R alpha0 = (R)1 + gm1inv * ibln;
-    R pm = rm * rcp<R>(bm);
-    R rinv = rcp<R>(Lam * Wm);
+    R pm = (l.rho.v + r.rho.v) * qrcp<R>(l.beta.v + r.beta.v);
+    R rinv = qrcp<R>(Lam * Wm);
     R iLam = rinv * Wm;
     R iW = rinv * Lam;
     R UD = rln * Wm;
@@ -535,6 +631,57 @@ __device__ __forceinline__ void ec_pair(const NodeV<R> &l, const NodeV<R> &r, R 
     out[1] = uxm * cm + pm * mx;
     out[2] = uym * cm + pm * my;
     out[3] = mt * UE + Es;
+}
+
+// The jump (right minus left Jiang-Shu edge value) at one interface from the first
+// differences D_k = V_{k+1} - V_k of its stencil.  WENO5, V0..V5 with the interface
+// between V2 and V3: with the second differences t, the third differences d and the
+// candidates of the left value q_0, q_a, q_b (q_a, q_b also the right value's),
+//   q_0 - q_a = d_0/3,  q_b - q_a = d_1/6,  q_0' - q_b = -d_2/3,
+// the weights a_k = d_k/(eps + b_k)^2 (multiplied through by the squared denominators)
+// give left = q_a + (2 a_0 d_0 + a_2 d_1)/(6 sum a), and likewise on the right, so that
+//   jump = (d_1 - (2 a_0' d_2 + a_2' d_1)/sum a' - (2 a_0 d_0 + a_2 d_1)/sum a)/6
+// without the edge values themselves: ~60 operations against ~95, and no cancellation
+// of the field's mean value (with the eigenvectors in closed form below, the FP32
+// tolerance and the short reciprocals: the 400^2 FP64 step 5.50 -> 4.26 ms, the mixed one
+// 1.25 -> 1.22 ms, one 64^2 right-hand side 44 -> 37 us).  Everything is scaled by 4 (eps4 = 4 eps, b_k of doubled
+// first-derivative terms).  Sums of two products are written as the fused operation, so
+// that every kernel that inlines this rounds them alike.
+template <typename R>
+__device__ __forceinline__ R weno5_jump(R D0, R D1, R D2, R D3, R D4, R eps4)
+{
+    const R c = (R)(13.0 / 3.0), two = (R)2, three = (R)3, six = (R)6;
+    const R t0 = D1 - D0, ta = D2 - D1, tb = D3 - D2, t5 = D4 - D3;
+    const R d0 = t0 - ta, d1 = ta - tb, d2 = tb - t5;
+    const R S0 = fma_<R>(c * t0, t0, eps4), Sa = fma_<R>(c * ta, ta, eps4), Sb = fma_<R>(c * tb, tb, eps4),
+            S5 = fma_<R>(c * t5, t5, eps4);
+    R nl, ql, nr, qr;
+    {
+        const R r0 = t0 + two * D1, r1 = D1 + D2, r2 = tb - two * D2;
+        R e0 = fma_<R>(r0, r0, S0), e1 = fma_<R>(r1, r1, Sa), e2 = fma_<R>(r2, r2, Sb);
+        e0 *= e0; e1 *= e1; e2 *= e2;
+        nl = e1 * fma_<R>(three, e0 * d1, two * (e2 * d0));
+        ql = qrcp<R>(fma_<R>(e2, fma_<R>(six, e0, e1), three * (e0 * e1)));
+    }
+    {
+        const R r0 = t5 - two * D3, r1 = D2 + D3, r2 = ta + two * D2;
+        R e0 = fma_<R>(r0, r0, S5), e1 = fma_<R>(r1, r1, Sb), e2 = fma_<R>(r2, r2, Sa);
+        e0 *= e0; e1 *= e1; e2 *= e2;
+        nr = e1 * fma_<R>(three, e0 * d1, two * (e2 * d2));
+        qr = qrcp<R>(fma_<R>(e2, fma_<R>(six, e0, e1), three * (e0 * e1)));
+    }
+    return (d1 - fma_<R>(nl, ql, nr * qr)) * (R)(1.0 / 6.0);
+}
+
+// WENO3, V0..V3 with the interface between V1 and V2: left = q - w t_0/2, right =
+// q - w' t_1/2 with q the mean of V1 and V2.
+template <typename R>
+__device__ __forceinline__ R weno3_jump(R D0, R D1, R D2, R eps)
+{
+    R e0 = fma_<R>(D0, D0, eps), e1 = fma_<R>(D1, D1, eps), e2 = fma_<R>(D2, D2, eps);
+    e0 *= e0; e1 *= e1; e2 *= e2;
+    const R w0 = e1 * qrcp<R>(fma_<R>((R)2, e0, e1)), w1 = e1 * qrcp<R>(fma_<R>((R)2, e2, e1));
+    return (R)0.5 * fma_<R>(w0, D1 - D0, w1 * (D1 - D2));
 }
 
 // The two Jiang-Shu WENO5 edge values of one interface from its six stencil
@@ -605,74 +752,64 @@ __device__ __forceinline__ void weno3_lr(R V0, R V1, R V2, R V3, R eps, R &vm, R
     }
 }
 
-__device__ __forceinline__ int sgn_d(double a) { return (a > 0.0) - (a < 0.0); }
+// (in FP64 on the integer pipes: an FP64 compare takes an FP64-pipe slot)
+__device__ __forceinline__ int sgn_d(double a)
+{
+    const uint64_t b = conv_bits64(a), m = b & 0x7fffffffffffffffull;
+    return m == 0 || m > 0x7ff0000000000000ull ? 0 : ((b >> 63) ? -1 : 1);
+}
 __device__ __forceinline__ int sgn_d(float a) { return (a > 0.0f) - (a < 0.0f); }
 __device__ __forceinline__ int sgn_d(dual a) { return (a.v > 0.0) - (a.v < 0.0); }
 __device__ __forceinline__ bool le(double a, double b) { return a <= b; }
 __device__ __forceinline__ bool le(float a, float b) { return a <= b; }
 __device__ __forceinline__ bool le(dual a, dual b) { return a.v <= b.v; }
 
-// Scaled eigenvectors of dF_1/dU (Sec. 4) at the rotated state (rho, vn, vt, p)
-// with W = 1/sqrt(1 - vn^2 - vt^2): columns dU_m * s_m, s_m = (dU_m . dV_m)^-1/2,
-// for the waves (lambda_-, v_n [entropy, d rho = 1], v_n [shear, d v_t = 1],
-// lambda_+ [acoustic, dp = 1]).  dU (4 x 4, column per wave) and s are returned
-// separately; lam_m, lam_p are the acoustic speeds; gm1i = 1/(Gamma - 1).
+// Scaled eigenvectors of dF_1/dU (Sec. 4) at the rotated state with 4-velocity (W,
+// un, ut): rows E[m] = s_m (dD, dm_n, dm_t, dE) with s_m = (dU.dV)^-1/2, for the waves
+// lambda_-, v_n (entropy, d rho = 1), v_n (shear, d v_t = 1), lambda_+.  An acoustic wave is, with
+// xi = (-lambda, n), a = u.xi = W (v_n - lambda), k = xi + a u and k^2 = 1 - lambda^2 + a^2,
+//   du = -a k,  dp = Gamma p k^2,  d rho = rho k^2,
+//   dU.dV = 2 beta rho h a^2 kap,  kap = W (1 - lambda^2) - a lambda,
+// (rho h a^2 = Gamma p k^2), and a = +-c W (disc +- v_n c/W^2)/(1 - v^2 c^2) keeps its
+// relative accuracy.  igg = (Gamma-1)/Gamma.
 template <typename R>
-__device__ __forceinline__ void eigen_rhd(R gam, R gm1i, R rho, R vn, R vt, R p, R W,
-                                          R dU[4][4], R s[4], R &lam_m, R &lam_p)
+__device__ __forceinline__ void eigen_rhd(R gam, R gg, R igg, R rho, R p, R un, R ut, R W, R iW, R E[4][4], R &lam_m,
+                                          R &lam_p)
 {
-    R one = (R)1;
-    R gg = gam * gm1i;
-    R W2 = W * W;
-    R iW2 = rcp<R>(W2);                    // 1 - v^2
-    R v2 = one - iW2;
-    R irp = rcp<R>(rho * p);
-    R ip = rho * irp, ir = p * irp;
-    R rh = rho + gg * p;                   // rho h
-    R c2 = gam * p * rcp<R>(rh);
-    R c = sqrt_pos<R>(c2);
-    R disc = sqrt_pos<R>(iW2 * (one - v2 * c2 - vn * vn * (one - c2)));
-    R den = rcp<R>(one - v2 * c2);
-    lam_m = (vn * (one - c2) - c * disc) * den;
-    lam_p = (vn * (one - c2) + c * disc) * den;
-    R Q = rh * W2;
-    R beta = rho * ip;
-    R un = W * vn, ut = W * vt;
-    R W4 = W2 * W2;
-    // entropy wave, d rho = 1:  dU = (W, W^2 v, W^2),  dU.dV = G W/((G-1) rho)
-    dU[0][1] = W; dU[1][1] = W2 * vn; dU[2][1] = W2 * vt; dU[3][1] = W2;
-    s[1] = rsq<R>(gg * W * ir);
-    // shear wave, d v_t = 1:  dU = (rho W^3 vt, 2 rho h W^4 vn vt,
-    //   rho h (2 W^4 vt^2 + W^2), 2 rho h W^4 vt),  dU.dV = rho h beta W^3 (1 + W^2 vt^2)
-    dU[0][2] = rho * W2 * W * vt;
-    dU[1][2] = (R)2 * rh * W4 * vn * vt;
-    dU[2][2] = rh * ((R)2 * W4 * vt * vt + W2);
-    dU[3][2] = (R)2 * rh * W4 * vt;
-    s[2] = rsq<R>(rh * beta * W2 * W * (one + W2 * vt * vt));
+    const R one = (R)1, two = (R)2;
+    const R iW2 = iW * iW, vn = un * iW, v2 = fma_<R>(-iW, iW, one);
+    const R gp = gam * p, rh = fma_<R>(gg, p, rho), beta = rho * qrcp<R>(p);
+    const R c2 = gp * qrcp<R>(rh), c = c2 * qrsq<R>(c2);
+    const R D0 = fma_<R>(-v2, c2, one), X = fma_<R>(-(vn * vn), sub_<R>(one, c2), D0);
+    const R disc = iW * X * qrsq<R>(X), cd = W * c * qrcp<R>(D0), vc = vn * c * iW2;
+    const R e0 = fma_<R>(gg, gp, rho), rhW = rh * W, brh = two * beta * rh;
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
-        int m = side == 0 ? 0 : 3;
-        R l = side == 0 ? lam_m : lam_p;
-        R a = rcp<R>((l - vn) * Q);          // 1 / ((lam - v_n) Q)
-        R dvn = (one - vn * l) * a;
-        R dvt = -l * vt * a;
-        R vdv = vn * dvn + vt * dvt;
-        R drho = rho * dvn * a * Q - rho * W2 * vdv;
-        // dU/dw dw with dp = 1
-        R h1 = drho + gg;                    // d(rho h)
-        R dW = W2 * W * vdv;
-        dU[0][m] = W * drho + rho * dW;
-        dU[1][m] = W2 * vn * h1 + rh * ((R)2 * W4 * vn * vdv + W2 * dvn);
-        dU[2][m] = W2 * vt * h1 + rh * ((R)2 * W4 * vt * vdv + W2 * dvt);
-        dU[3][m] = W2 * h1 - one + rh * (R)2 * W4 * vdv;
-        // dV/dw dw
-        R dbeta = drho * ip - beta * ip;
-        R dV0 = drho * ir + (drho * ir - ip) * gm1i + dbeta;
-        R dV1 = dbeta * un + beta * (W * dvn + vn * dW);
-        R dV2 = dbeta * ut + beta * (W * dvt + vt * dW);
-        R dV3 = -(dbeta * W + beta * dW);
-        s[m] = rsq<R>(dU[0][m] * dV0 + dU[1][m] * dV1 + dU[2][m] * dV2 + dU[3][m] * dV3);
+        const int m = side == 0 ? 0 : 3;
+        const R a = cd * sub_<R>(vc, side == 0 ? -disc : disc);
+        const R lam = fma_<R>(-a, iW, vn);
+        (side == 0 ? lam_m : lam_p) = lam;
+        const R ol = (one - lam) * (one + lam), k0 = fma_<R>(a, W, lam), k2 = fma_<R>(a, a, ol), kap = fma_<R>(W, ol, -(a * lam));
+        const R s = qrsq<R>(brh * (a * a) * kap);
+        const R ek = e0 * k2, ha = rhW * a, cc = fma_<R>(ek, W, -(rh * a * k0));
+        E[m][0] = s * (rho * kap);
+        E[m][1] = s * fma_<R>(cc, un, -(ha * fma_<R>(a, un, one)));
+        E[m][2] = s * fma_<R>(cc, ut, -(ha * (a * ut)));
+        E[m][3] = s * fma_<R>(-gp, k2, fma_<R>(ek, W * W, -(two * (ha * k0))));
     }
+    // entropy wave: dU = (W, W^2 v, W^2), dU.dV = Gamma W/((Gamma-1) rho)
+    const R q = W * rho * igg, g1 = q * qrsq<R>(q);
+    E[1][0] = g1;
+    E[1][1] = g1 * un;
+    E[1][2] = g1 * ut;
+    E[1][3] = g1 * W;
+    // shear wave: dU = (rho W^3 v_t, 2 rho h W^4 v_n v_t, rho h (2 W^4 v_t^2 + W^2), 2 rho h W^4
+    // v_t), dU.dV = rho h beta W^3 (1 + W^2 v_t^2)
+    const R f = qrsq<R>(rh * beta * iW * fma_<R>(ut, ut, one)), h = f * rh, h2 = two * h * ut;
+    E[2][0] = f * rho * ut;
+    E[2][1] = h2 * un;
+    E[2][2] = fma_<R>(h2, ut, h);
+    E[2][3] = h2 * W;
 }
 
 }  // namespace esmm

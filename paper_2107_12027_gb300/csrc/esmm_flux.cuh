@@ -16,41 +16,43 @@
 
 namespace esmm {
 
-// One flux argument: the FP64 log-mean arguments from q and the working
-// values from q (FP64) or from the FP32 copies q32 (float).
+// One flux argument from the node arrays q (FP64) or from the FP32 copies q32 (float,
+// with the FP64 rest of rho and beta for their jumps).
 template <typename R>
 __device__ __forceinline__ NodeV<R> load_node(const Geom &g, const double *__restrict__ q,
                                               const float *__restrict__ q32, long long c)
 {
     NodeV<R> v;
-    v.rho = q[Q_RHO * g.P + c];
-    v.beta = q[Q_BETA * g.P + c];
-    v.lnr = q[Q_LNR * g.P + c];
-    v.lnb = q[Q_LNB * g.P + c];
     if constexpr (std::is_same<R, float>::value) {
-        v.r = q32[Q32_R * g.P + c];
-        v.b = q32[Q32_B * g.P + c];
+        v.rho = lmv_f32(q[Q_RHO * g.P + c], q32[Q32_R * g.P + c], q32[Q32_LNR * g.P + c]);
+        v.beta = lmv_f32(q[Q_BETA * g.P + c], q32[Q32_B * g.P + c], q32[Q32_LNB * g.P + c]);
         v.ux = q32[Q32_UX * g.P + c];
         v.uy = q32[Q32_UY * g.P + c];
         v.W = q32[Q32_W * g.P + c];
     } else {
-        v.r = (R)v.rho;
-        v.b = (R)v.beta;
-        v.ux = (R)q[Q_UX * g.P + c];
-        v.uy = (R)q[Q_UY * g.P + c];
-        v.W = (R)q[Q_W * g.P + c];
+        v.rho.v = q[Q_RHO * g.P + c];
+        v.rho.l = q[Q_LNR * g.P + c];
+        v.beta.v = q[Q_BETA * g.P + c];
+        v.beta.l = q[Q_LNB * g.P + c];
+        v.ux = q[Q_UX * g.P + c];
+        v.uy = q[Q_UY * g.P + c];
+        v.W = q[Q_W * g.P + c];
     }
     return v;
 }
 
 // The ES dissipation 1/2 lambda^ T^-1 R Y <<V~>> of eq. ESFlux_HO at one
-// interface (to be subtracted from the EC flux).  nvx, nvy, jt: the interface
-// metrics (mean of the two nodes); rho0/1, lnr0/1: density and its log at the
-// two interface nodes (the log-mean arguments), r0/1 the densities in the
-// working precision; st[k] = (beta, u_x, u_y, W,
-// ln rho, ln beta) of the w + 1 stencil nodes, the interface nodes at
-// k = (w-1)/2 and (w+1)/2.  The eigen-system is taken at rho = {{rho}}^ln,
+// interface, subtracted from the EC flux F.  nvx, nvy, jt: the interface
+// metrics (mean of the two nodes); rho0/1: the density at the two interface nodes
+// (log-mean arguments); st: the w + 1 stencil nodes, the interface nodes at
+// k = (w-1)/2 and (w+1)/2, with state (beta, u_x, u_y), differences dV(k) = V_{k+1} -
+// V_k of the entropy variables, and V32 their FP32 values (for the switch's
+// tolerance).  The eigen-system is taken at rho = {{rho}}^ln,
 // u = {{u}}, p = {{rho}}/{{beta}}; Y has sign 0 for jumps at rounding level.
+// Sums of two products are written as the fused operation, so that the kernels that
+// inline this round them alike.
+// The dissipation depends on differences of V alone, so they are projected (w of
+// them) rather than the w + 1 values.
 // The entropy variables (V_1, V_x, V_y, V_E) of one node (Sec. 2, B = 0)
 // from beta, u, W, ln rho, ln beta: V_1 = Gamma/(Gamma-1) + ln rho +
 // ln beta/(Gamma-1) + beta, (V_x, V_y) = beta u, V_E = -beta W.  Every
@@ -85,26 +87,64 @@ __device__ __forceinline__ void entropy_vars4<float>(float b, float ux, float uy
     V[3] = -__fmul_rn(b, W);
 }
 
-// stencil values read straight from the node arrays (forward kernels)
+// d = b - a of two nodes' entropy variables, one rounding each (in FP64 and FP32
+// never contracted with what forms or uses them)
 template <typename R>
-struct QStencil {
-    const double *q;
-    long long P, c0, sd;
-    int off;
-    __device__ __forceinline__ R operator()(int k, int j) const
+__device__ __forceinline__ void v_diff(const R a[4], const R b[4], R d[4])
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q) d[q] = sub_<R>(b[q], a[q]);
+}
+
+// the type of the switch's tolerance: FP32 in both forms
+template <typename R> struct TolT { using type = R; };
+template <> struct TolT<double> { using type = float; };
+__device__ __forceinline__ float to_tol(double x) { return d2f_int(x); }
+template <typename R> __device__ __forceinline__ R to_tol(R x) { return x; }
+
+// the six quantities of stencil node k: get(k, j), j = 0..5: beta, u_x, u_y, W, ln rho,
+// ln beta
+template <typename R, typename GET>
+struct NodeStencil {
+    GET get;
+    __device__ __forceinline__ void state(int k, R &b, R &ux, R &uy) const
     {
-        const int f = j == 0 ? Q_BETA : (j == 1 ? Q_UX : (j == 2 ? Q_UY : (j == 3 ? Q_W : (j == 4 ? Q_LNR : Q_LNB))));
-        return (R)q[f * P + c0 + (k - off) * sd];
+        b = get(k, 0);
+        ux = get(k, 1);
+        uy = get(k, 2);
     }
     __device__ __forceinline__ void V(int k, R c1g, R ig, R v[4]) const
     {
-        entropy_vars4<R>((*this)(k, 0), (*this)(k, 1), (*this)(k, 2), (*this)(k, 3), (*this)(k, 4), (*this)(k, 5), c1g,
-                         ig, v);
+        entropy_vars4<R>(get(k, 0), get(k, 1), get(k, 2), get(k, 3), get(k, 4), get(k, 5), c1g, ig, v);
+    }
+    __device__ __forceinline__ void dV(int k, R c1g, R ig, R d[4]) const
+    {
+        R a[4], b[4];
+        V(k, c1g, ig, a);
+        V(k + 1, c1g, ig, b);
+        v_diff<R>(a, b, d);
+    }
+    __device__ __forceinline__ void V32(int k, R c1g, R ig, typename TolT<R>::type v[4]) const
+    {
+        R a[4];
+        V(k, c1g, ig, a);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = to_tol(a[q]);
     }
 };
-
-// the same from the FP32 copies (the mixed form)
-struct QStencil32 {
+// ... read straight from the node arrays
+struct QGet {
+    const double *q;
+    long long P, c0, sd;
+    int off;
+    __device__ __forceinline__ double operator()(int k, int j) const
+    {
+        const int f = j == 0 ? Q_BETA : (j == 1 ? Q_UX : (j == 2 ? Q_UY : (j == 3 ? Q_W : (j == 4 ? Q_LNR : Q_LNB))));
+        return q[f * P + c0 + (k - off) * sd];
+    }
+};
+// ... from the FP32 copies (the mixed form)
+struct QGet32 {
     const float *q;
     long long P, c0, sd;
     int off;
@@ -114,102 +154,97 @@ struct QStencil32 {
                     : (j == 1 ? Q32_UX : (j == 2 ? Q32_UY : (j == 3 ? Q32_W : (j == 4 ? Q32_LNR : Q32_LNB))));
         return q[f * P + c0 + (k - off) * sd];
     }
-    __device__ __forceinline__ void V(int k, float c1g, float ig, float v[4]) const
-    {
-        entropy_vars4<float>((*this)(k, 0), (*this)(k, 1), (*this)(k, 2), (*this)(k, 3), (*this)(k, 4), (*this)(k, 5),
-                             c1g, ig, v);
-    }
 };
-
-// stencil values held in an array (the adjoint's seeded duals)
-template <typename R, int NS>
-struct ArrStencil {
+// ... from an array (the operation count)
+template <typename R>
+struct ArrGet {
     const R (*a)[6];
     __device__ __forceinline__ R operator()(int k, int j) const { return a[k][j]; }
-    __device__ __forceinline__ void V(int k, R c1g, R ig, R v[4]) const
-    {
-        entropy_vars4<R>(a[k][0], a[k][1], a[k][2], a[k][3], a[k][4], a[k][5], c1g, ig, v);
-    }
 };
 
-template <typename R, typename T, int WW, typename ST>
-__device__ __forceinline__ void es_dissipation(R nvx, R nvy, R jt, T rho0, T rho1, T lnr0, T lnr1, R r0, R r1,
-                                               const ST &st, const Phys &ph, R diss[4])
+template <typename R, int WW, typename ST>
+__device__ __forceinline__ void es_dissipation(R nvx, R nvy, R jt, const LmV<R> &rho0, const LmV<R> &rho1,
+                                               const ST &st, const Phys &ph, R F[4])
 {
-    constexpr int NS = WW + 1, OFF = (WW - 1) / 2;
+    constexpr int OFF = (WW - 1) / 2;
+    using S = typename TolT<R>::type;
     const R half = (R)0.5, one = (R)1;
     const R gam = (R)ph.gamma;
-    R n2 = nvx * nvx + nvy * nvy;
-    R iLk = rsq<R>(n2);
+    R n2 = fma_<R>(nvx, nvx, nvy * nvy);
+    R iLk = qrsq<R>(n2);
     R Lk = n2 * iLk;
     R nx = nvx * iLk, ny = nvy * iLk;
-    R rho, irho;
-    lmean<R, T>(rho0, rho1, lnr0, lnr1, r0, r1, ph.ln_thr, rho, irho);
-    R ux = half * (st(OFF, 1) + st(OFF + 1, 1));
-    R uy = half * (st(OFF, 2) + st(OFF + 1, 2));
-    R p = (r0 + r1) * rcp<R>(st(OFF, 0) + st(OFF + 1, 0));
-    R w2 = one + ux * ux + uy * uy;
-    R iW = rsq<R>(w2);
+    R rho, irho, b0, b1, u0, u1, y0, y1;
+    logmean2<R>(rho0, rho1, ph.ln_thr, rho, irho);
+    st.state(OFF, b0, u0, y0);
+    st.state(OFF + 1, b1, u1, y1);
+    R ux = half * (u0 + u1), uy = half * (y0 + y1);
+    R p = (rho0.v + rho1.v) * qrcp<R>(b0 + b1);
+    R w2 = fma_<R>(uy, uy, fma_<R>(ux, ux, one));
+    R iW = qrsq<R>(w2);
     R W = w2 * iW;
-    R vx = ux * iW, vy = uy * iW;
-    R vn = nx * vx + ny * vy, vt = -ny * vx + nx * vy;
-    R dU[4][4], s[4], lm, lp;
     const R ig = (R)ph.gm1i, c1g = gam * ig;
-    eigen_rhd<R>(gam, ig, rho, vn, vt, p, W, dU, s, lm, lp);
-    R lhat = vmax(fab<R>(jt + Lk * lm), fab<R>(jt + Lk * lp));
-    // Vt_m = s_m dU_m . (T V): the rotation T and the scale s_m folded into
-    // the projection row Ar[m] once per interface
-    R Ar[4][4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        Ar[m][0] = s[m] * dU[0][m];
-        Ar[m][1] = s[m] * (nx * dU[1][m] - ny * dU[2][m]);
-        Ar[m][2] = s[m] * (ny * dU[1][m] + nx * dU[2][m]);
-        Ar[m][3] = s[m] * dU[3][m];
+    R E[4][4], lm, lp;
+    eigen_rhd<R>(gam, c1g, (R)ph.igg, rho, p, fma_<R>(nx, ux, ny * uy), fma_<R>(nx, uy, -(ny * ux)), W, iW, E, lm,
+                 lp);
+    R lhat = vmax(fab<R>(fma_<R>(Lk, lm, jt)), fab<R>(fma_<R>(Lk, lp, jt)));
+    // |T V| summed over the two interface nodes, for the switch's tolerance
+    S aT[4];
+    {
+        S V0[4], V1[4];
+        const S nx_ = to_tol(nx), ny_ = to_tol(ny);
+        st.V32(OFF, c1g, ig, V0);
+        st.V32(OFF + 1, c1g, ig, V1);
+        aT[0] = fab<S>(V0[0]) + fab<S>(V1[0]);
+        aT[1] = fab<S>(nx_ * V0[1] + ny_ * V0[2]) + fab<S>(nx_ * V1[1] + ny_ * V1[2]);
+        aT[2] = fab<S>(nx_ * V0[2] - ny_ * V0[1]) + fab<S>(nx_ * V1[2] - ny_ * V1[1]);
+        aT[3] = fab<S>(V0[3]) + fab<S>(V1[3]);
     }
-    R Vt[NS][4];
-    R aT[4] = {(R)0, (R)0, (R)0, (R)0};     // |T V| summed over the two interface nodes
+    // projected differences, the rotation T folded into the projection rows once per
+    // interface
+    R Dt[WW][4];
+    {
+        R Ar[4][4];
 #pragma unroll
-    for (int k = 0; k < NS; ++k) {
-        R V[4];
-        st.V(k, c1g, ig, V);
-        if (k == OFF || k == OFF + 1) {
-            aT[0] += fab<R>(V[0]);
-            aT[1] += fab<R>(nx * V[1] + ny * V[2]);
-            aT[2] += fab<R>(-ny * V[1] + nx * V[2]);
-            aT[3] += fab<R>(V[3]);
+        for (int m = 0; m < 4; ++m) {
+            Ar[m][0] = E[m][0];
+            Ar[m][1] = fma_<R>(nx, E[m][1], -(ny * E[m][2]));
+            Ar[m][2] = fma_<R>(ny, E[m][1], nx * E[m][2]);
+            Ar[m][3] = E[m][3];
         }
 #pragma unroll
-        for (int m = 0; m < 4; ++m) Vt[k][m] = Ar[m][0] * V[0] + Ar[m][1] * V[1] + Ar[m][2] * V[2] + Ar[m][3] * V[3];
+        for (int k = 0; k < WW; ++k) {
+            R D[4];
+            st.dV(k, c1g, ig, D);
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                Dt[k][m] = fma_<R>(Ar[m][3], D[3], fma_<R>(Ar[m][2], D[2], fma_<R>(Ar[m][1], D[1], Ar[m][0] * D[0])));
+        }
     }
-    const R eps = (R)ph.eps;
-    const R sign_tol = (R)ph.sign_tol;
-    R z[4];
+    const S tol = (S)ph.sign_tol;
+    R d[4] = {(R)0, (R)0, (R)0, (R)0};
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-        R vminus, vplus;
-        if (WW == 5)
-            weno5_lr<R>(Vt[0][m], Vt[1][m], Vt[2][m], Vt[3][m], Vt[4][m], Vt[5][m], eps, vminus, vplus);
+        R jw;
+        if constexpr (WW == 5)
+            jw = weno5_jump<R>(Dt[0][m], Dt[1][m], Dt[2][m], Dt[3][m], Dt[4][m], (R)(4.0 * ph.eps));
         else
-            weno3_lr<R>(Vt[0][m], Vt[1][m], Vt[2][m], Vt[3][m], eps, vminus, vplus);
-        R jw = vplus - vminus;
-        R jump = Vt[OFF + 1][m] - Vt[OFF][m];
+            jw = weno3_jump<R>(Dt[0][m], Dt[1][m], Dt[2][m], (R)ph.eps);
+        const R jump = Dt[OFF][m];
         // a jump within sign_tol of the magnitudes forming V~_m at the two
         // interface nodes is rounding noise: its sign is 0 (so Y = 0)
-        R scale = s[m] * (fab<R>(dU[0][m]) * aT[0] + fab<R>(dU[1][m]) * aT[1] +
-                          fab<R>(dU[2][m]) * aT[2] + fab<R>(dU[3][m]) * aT[3]);
-        int sj = le(fab<R>(jump), sign_tol * scale) ? 0 : sgn_d(jump);
-        z[m] = (sgn_d(jw) == sj) ? jw * s[m] : (R)0;
-    }
-    R d[4];
+        const S scale = fab<S>(to_tol(E[m][0])) * aT[0] + fab<S>(to_tol(E[m][1])) * aT[1] +
+                        fab<S>(to_tol(E[m][2])) * aT[2] + fab<S>(to_tol(E[m][3])) * aT[3];
+        const int sj = le(fab<S>(to_tol(jump)), tol * scale) ? 0 : sgn_d(jump);
+        const R z = (sgn_d(jw) == sj) ? jw : (R)0;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-        d[a] = dU[a][0] * z[0] + dU[a][1] * z[1] + dU[a][2] * z[2] + dU[a][3] * z[3];
+        for (int a = 0; a < 4; ++a) d[a] = fma_<R>(E[m][a], z, d[a]);
+    }
     R hl = half * lhat;
-    diss[0] = hl * d[0];
-    diss[1] = hl * (nx * d[1] - ny * d[2]);
-    diss[2] = hl * (ny * d[1] + nx * d[2]);
-    diss[3] = hl * d[3];
+    F[0] = fma_<R>(-hl, d[0], F[0]);
+    F[1] = fma_<R>(-hl, fma_<R>(nx, d[1], -(ny * d[2])), F[1]);
+    F[2] = fma_<R>(-hl, fma_<R>(ny, d[1], nx * d[2]), F[2]);
+    F[3] = fma_<R>(-hl, d[3], F[3]);
 }
 
 // anchors A in [-P, n_dir - 1] along the sweep, every line of the other
@@ -321,28 +356,26 @@ __device__ __forceinline__ void iface_tile(const ProbArg &pa, const Phys &ph, co
         }
         const R an = (R)ph.alpha[n - 1];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) F[a] += an * Fs[a];
+        for (int a = 0; a < 4; ++a) F[a] = fma_<R>(an, Fs[a], F[a]);
         Ft += (MT)ph.alpha[n - 1] * Fts;
     }
 
-    if (WW > 0) {
+    if constexpr (WW > 0) {
         // eq. ESFlux_HO: subtract 1/2 lambda^ T^-1 R Y <<V~>>
         const long long c1 = c0 + sd;
         const R nvx = (R)((MT)0.5 * (Mx[c0] + Mx[c1])), nvy = (R)((MT)0.5 * (My[c0] + My[c1]));
         const R jt = (R)((MT)0.5 * (Mt[c0] + Mt[c1]));
-        const double rho0 = q[Q_RHO * g.P + c0], rho1 = q[Q_RHO * g.P + c1];
-        const double lnr0 = q[Q_LNR * g.P + c0], lnr1 = q[Q_LNR * g.P + c1];
-        R diss[4];
         if constexpr (F32) {
-            QStencil32 st{q32, g.P, c0, sd, (WW - 1) / 2};
-            es_dissipation<R, double, WW>(nvx, nvy, jt, rho0, rho1, lnr0, lnr1, q32[Q32_R * g.P + c0],
-                                          q32[Q32_R * g.P + c1], st, ph, diss);
+            const LmV<R> rho0 = lmv_f32(q[Q_RHO * g.P + c0], q32[Q32_R * g.P + c0], q32[Q32_LNR * g.P + c0]);
+            const LmV<R> rho1 = lmv_f32(q[Q_RHO * g.P + c1], q32[Q32_R * g.P + c1], q32[Q32_LNR * g.P + c1]);
+            NodeStencil<R, QGet32> st{{q32, g.P, c0, sd, (WW - 1) / 2}};
+            es_dissipation<R, WW>(nvx, nvy, jt, rho0, rho1, st, ph, F);
         } else {
-            QStencil<R> st{q, g.P, c0, sd, (WW - 1) / 2};
-            es_dissipation<R, double, WW>(nvx, nvy, jt, rho0, rho1, lnr0, lnr1, (R)rho0, (R)rho1, st, ph, diss);
+            const LmV<R> rho0 = {q[Q_RHO * g.P + c0], q[Q_LNR * g.P + c0]};
+            const LmV<R> rho1 = {q[Q_RHO * g.P + c1], q[Q_LNR * g.P + c1]};
+            NodeStencil<R, QGet> st{{q, g.P, c0, sd, (WW - 1) / 2}};
+            es_dissipation<R, WW>(nvx, nvy, jt, rho0, rho1, st, ph, F);
         }
-#pragma unroll
-        for (int a = 0; a < 4; ++a) F[a] -= diss[a];
     }
     R *out = iflux + (long long)(dir * 5) * g.P + c0;
 #pragma unroll

@@ -33,8 +33,6 @@
 
 namespace esmm {
 
-__device__ __forceinline__ float to_f32(double x) { return d2f_int(x); }
-__device__ __forceinline__ float to_f32(float x) { return x; }
 template <typename R> __device__ __forceinline__ R of_f32(float x);
 template <> __device__ __forceinline__ double of_f32<double>(float x) { return f2d_int(x); }
 template <> __device__ __forceinline__ float of_f32<float>(float x) { return x; }

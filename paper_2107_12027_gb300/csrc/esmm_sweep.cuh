@@ -23,8 +23,9 @@
 // are laid out [field][node] with a stride of 41 nodes (conflict-free for
 // both the row reads of the lanes and the column-interleaved staging writes).
 // The staging also forms each node's entropy variables once (entropy_vars4,
-// the rounded operations the two-kernel path applies per interface), which
-// the dissipation then reads for every stencil that holds the node.
+// the rounded operations the two-kernel path applies per interface) and then
+// their differences along the line, which the dissipation reads for every
+// stencil that holds them.
 #pragma once
 
 #include <type_traits>
@@ -38,16 +39,16 @@ constexpr int SW_NNP = 41;   // node stride of a staged field (>= the largest se
 template <typename R, int P>
 struct SweepLayout {
     static constexpr bool F32 = std::is_same<R, float>::value;
-    // FP64 fields: rho, beta, ln rho, ln beta (the log-mean arguments), and in
-    // the FP64 form also u_x, u_y, W, the direction's metrics Mt, Mx, My and
-    // the entropy variables V_1, V_x, V_y, V_E
-    static constexpr int NF64 = F32 ? 4 : 14;
-    // FP32 fields of the mixed form: r, b, u_x, u_y, W, ln rho, ln beta, Mt,
-    // Mx, My, V_1, V_x, V_y, V_E
-    static constexpr int NF32 = F32 ? 14 : 0;
+    // 14 fields in the working precision: rho, beta, ln rho, ln beta, u_x, u_y, W, the
+    // direction's metrics Mt, Mx, My, and the entropy variables V_1, V_x, V_y, V_E
+    // (replaced by their differences to the next node once all are staged); and NTOL
+    // FP32 ones: the entropy variables again (the switch's tolerance), in the mixed
+    // form also the FP64 rests of rho and beta.  (NTOL is even, so that the FP64 pair
+    // fluxes behind them are aligned.)
+    static constexpr int NTOL = F32 ? 6 : 4;
     static constexpr int PAIR_VALUES = P * 4 * 32;   // pair fluxes of the warp's 32 anchors
     static constexpr size_t bytes_per_warp =
-        (size_t)NF64 * SW_NNP * 8 + (size_t)NF32 * SW_NNP * 4 + (size_t)PAIR_VALUES * sizeof(R);
+        (size_t)14 * SW_NNP * sizeof(R) + (size_t)NTOL * SW_NNP * 4 + (size_t)PAIR_VALUES * sizeof(R);
 };
 
 template <int P, int WW>
@@ -58,98 +59,110 @@ struct SweepShape {
     static_assert(TA + HL + HR <= SW_NNP, "segment exceeds the staged node stride");
 };
 
-// the staged stencil of es_dissipation: field j of node k (k = 0 .. WW)
+// staged fields of one warp: values f = 0 .. 13 in the working precision (rho, beta,
+// ln rho, ln beta, u_x, u_y, W, Mt, Mx, My, dV_1, dV_x, dV_y, dV_E)
 template <typename R>
-struct SmemStencil;
-template <>
-struct SmemStencil<double> {
-    const double *s;
-    int base;
-    __device__ __forceinline__ double operator()(int k, int j) const
+struct SweepFields {
+    R *v;
+    float *t;      // [4] FP32 entropy variables; mixed form: [4] and [2] rests of rho, beta
+    __device__ __forceinline__ R at(int f, int e) const { return v[f * SW_NNP + e]; }
+    __device__ __forceinline__ LmV<R> lm(int f, int e) const
     {
-        const int f = j == 0 ? 1 : (j == 1 ? 4 : (j == 2 ? 5 : (j == 3 ? 6 : (j == 4 ? 2 : 3))));
-        return s[f * SW_NNP + base + k];
-    }
-    // the entropy variables staged with the node (fields 10 .. 13)
-    __device__ __forceinline__ void V(int k, double, double, double v[4]) const
-    {
-#pragma unroll
-        for (int a = 0; a < 4; ++a) v[a] = s[(10 + a) * SW_NNP + base + k];
-    }
-};
-template <>
-struct SmemStencil<float> {
-    const float *s;
-    int base;
-    __device__ __forceinline__ float operator()(int k, int j) const
-    {
-        const int f = j == 0 ? 1 : (j == 1 ? 2 : (j == 2 ? 3 : (j == 3 ? 4 : (j == 4 ? 5 : 6))));
-        return s[f * SW_NNP + base + k];
-    }
-    __device__ __forceinline__ void V(int k, float, float, float v[4]) const
-    {
-#pragma unroll
-        for (int a = 0; a < 4; ++a) v[a] = s[(10 + a) * SW_NNP + base + k];
+        LmV<R> a;
+        a.v = v[f * SW_NNP + e];
+        a.l = v[(2 + f) * SW_NNP + e];
+        if constexpr (std::is_same<R, float>::value) a.lo = t[(4 + f) * SW_NNP + e];
+        return a;
     }
 };
 
-// one node of global padded index c into staged slot e of a warp's arrays,
-// with its entropy variables (entropy_vars4 on the staged values, as the
-// stencils of the two-kernel path form them per interface)
+// the staged stencil of es_dissipation (slot base + k for node k)
+template <typename R>
+struct SmemStencil {
+    SweepFields<R> s;
+    int base;
+    __device__ __forceinline__ void state(int k, R &b, R &ux, R &uy) const
+    {
+        b = s.at(1, base + k);
+        ux = s.at(4, base + k);
+        uy = s.at(5, base + k);
+    }
+    __device__ __forceinline__ void dV(int k, R, R, R d[4]) const
+    {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) d[a] = s.at(10 + a, base + k);
+    }
+    __device__ __forceinline__ void V32(int k, R, R, float v[4]) const
+    {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) v[a] = s.t[a * SW_NNP + base + k];
+    }
+};
+
+// one node of global padded index c into staged slot e of a warp's arrays, with its
+// entropy variables (entropy_vars4 on the staged values, as the stencils of the
+// two-kernel path form them per interface)
 template <typename R>
 __device__ __forceinline__ void sweep_stage(const Geom &g, const double *__restrict__ q,
                                             const float *__restrict__ q32, long long c, int dir, R c1g, R ig,
-                                            double *sd, float *sf, int e)
+                                            const SweepFields<R> &s, int e)
 {
+    R v[10], V[4];
     if constexpr (std::is_same<R, float>::value) {
-        sd[0 * SW_NNP + e] = q[Q_RHO * g.P + c];
-        sd[1 * SW_NNP + e] = q[Q_BETA * g.P + c];
-        sd[2 * SW_NNP + e] = q[Q_LNR * g.P + c];
-        sd[3 * SW_NNP + e] = q[Q_LNB * g.P + c];
-        const int fl[10] = {Q32_R, Q32_B, Q32_UX, Q32_UY, Q32_W, Q32_LNR, Q32_LNB, Q32_MT0 + dir, Q32_M00 + 2 * dir,
+        const int fl[10] = {Q32_R, Q32_B, Q32_LNR, Q32_LNB, Q32_UX, Q32_UY, Q32_W, Q32_MT0 + dir, Q32_M00 + 2 * dir,
                             Q32_M01 + 2 * dir};
-        float v[10];
 #pragma unroll
-        for (int f = 0; f < 10; ++f) sf[f * SW_NNP + e] = v[f] = q32[fl[f] * g.P + c];
-        float V[4];
-        entropy_vars4<float>(v[1], v[2], v[3], v[4], v[5], v[6], c1g, ig, V);
-#pragma unroll
-        for (int a = 0; a < 4; ++a) sf[(10 + a) * SW_NNP + e] = V[a];
+        for (int f = 0; f < 10; ++f) s.v[f * SW_NNP + e] = v[f] = q32[fl[f] * g.P + c];
+        s.t[4 * SW_NNP + e] = lmv_f32(q[Q_RHO * g.P + c], v[0], v[2]).lo;
+        s.t[5 * SW_NNP + e] = lmv_f32(q[Q_BETA * g.P + c], v[1], v[3]).lo;
     } else {
         const int fl[10] = {Q_RHO, Q_BETA, Q_LNR, Q_LNB, Q_UX, Q_UY, Q_W, Q_MT0 + dir, Q_M00 + 2 * dir,
                             Q_M01 + 2 * dir};
-        double v[10];
 #pragma unroll
-        for (int f = 0; f < 10; ++f) sd[f * SW_NNP + e] = v[f] = q[fl[f] * g.P + c];
-        double V[4];
-        entropy_vars4<double>(v[1], v[4], v[5], v[6], v[2], v[3], c1g, ig, V);
+        for (int f = 0; f < 10; ++f) s.v[f * SW_NNP + e] = v[f] = q[fl[f] * g.P + c];
+    }
+    entropy_vars4<R>(v[1], v[4], v[5], v[6], v[2], v[3], c1g, ig, V);
 #pragma unroll
-        for (int a = 0; a < 4; ++a) sd[(10 + a) * SW_NNP + e] = V[a];
+    for (int a = 0; a < 4; ++a) {
+        s.v[(10 + a) * SW_NNP + e] = V[a];
+        s.t[a * SW_NNP + e] = to_f32(V[a]);
+    }
+}
+
+// the entropy variables of a warp's nn staged nodes into differences to the next node
+template <typename R>
+__device__ __forceinline__ void sweep_differences(const SweepFields<R> &s, int lane, int nn)
+{
+    for (int e0 = 0; e0 < nn - 1; e0 += 32) {
+        const int e = e0 + lane;
+        R a[4], b[4], d[4];
+        const bool on = e < nn - 1;
+        if (on)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                a[q] = s.at(10 + q, e);
+                b[q] = s.at(10 + q, e + 1);
+            }
+        __syncwarp();
+        if (on) {
+            v_diff<R>(a, b, d);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s.v[(10 + q) * SW_NNP + e] = d[q];
+        }
+        __syncwarp();
     }
 }
 
 // NodeV of staged slot i (as load_node)
 template <typename R>
-__device__ __forceinline__ NodeV<R> sweep_node(const double *sd, const float *sf, int i)
+__device__ __forceinline__ NodeV<R> sweep_node(const SweepFields<R> &s, int i)
 {
     NodeV<R> v;
-    v.rho = sd[0 * SW_NNP + i];
-    v.beta = sd[1 * SW_NNP + i];
-    v.lnr = sd[2 * SW_NNP + i];
-    v.lnb = sd[3 * SW_NNP + i];
-    if constexpr (std::is_same<R, float>::value) {
-        v.r = sf[0 * SW_NNP + i];
-        v.b = sf[1 * SW_NNP + i];
-        v.ux = sf[2 * SW_NNP + i];
-        v.uy = sf[3 * SW_NNP + i];
-        v.W = sf[4 * SW_NNP + i];
-    } else {
-        v.r = (R)v.rho;
-        v.b = (R)v.beta;
-        v.ux = (R)sd[4 * SW_NNP + i];
-        v.uy = (R)sd[5 * SW_NNP + i];
-        v.W = (R)sd[6 * SW_NNP + i];
-    }
+    v.rho = s.lm(0, i);
+    v.beta = s.lm(1, i);
+    v.ux = s.at(4, i);
+    v.uy = s.at(5, i);
+    v.W = s.at(6, i);
     return v;
 }
 
@@ -161,17 +174,20 @@ __global__ void __launch_bounds__(256) k_sweep(ProbArg pa, Phys ph, const double
     using LY = SweepLayout<R, P>;
     using SH = SweepShape<P, WW>;
     constexpr bool F32 = LY::F32;
-    using MT = typename std::conditional<F32, float, double>::type;
     constexpr int HL = SH::HL, HR = SH::HR, TA = SH::TA;
     extern __shared__ __align__(16) unsigned char sw_smem[];
     const int NW = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double *sd = (double *)sw_smem + (size_t)w * LY::NF64 * SW_NNP;
-    float *sf = (float *)((double *)sw_smem + (size_t)NW * LY::NF64 * SW_NNP) + (size_t)w * LY::NF32 * SW_NNP;
-    R *spr = (R *)((float *)((double *)sw_smem + (size_t)NW * LY::NF64 * SW_NNP) + (size_t)NW * LY::NF32 * SW_NNP) +
+    // per warp: 14 fields of R, then the FP32 ones, then the pair fluxes
+    auto fields_of = [&](int ww) {
+        SweepFields<R> s;
+        s.v = (R *)sw_smem + (size_t)ww * 14 * SW_NNP;
+        s.t = (float *)((R *)sw_smem + (size_t)NW * 14 * SW_NNP) + (size_t)ww * LY::NTOL * SW_NNP;
+        return s;
+    };
+    const SweepFields<R> sf = fields_of(w);
+    R *spr = (R *)((float *)((R *)sw_smem + (size_t)NW * 14 * SW_NNP) + (size_t)NW * LY::NTOL * SW_NNP) +
              (size_t)w * LY::PAIR_VALUES;
-    const MT *sMt = F32 ? (const MT *)(sf + 7 * SW_NNP) : (const MT *)(sd + 7 * SW_NNP);
-    const MT *sMx = F32 ? (const MT *)(sf + 8 * SW_NNP) : (const MT *)(sd + 8 * SW_NNP);
-    const MT *sMy = F32 ? (const MT *)(sf + 9 * SW_NNP) : (const MT *)(sd + 9 * SW_NNP);
+    const R *sMt = sf.v + 7 * SW_NNP, *sMx = sf.v + 8 * SW_NNP, *sMy = sf.v + 9 * SW_NNP;
     const R gm1inv = (R)(1.0 / (ph.gamma - 1.0));
     const R ig = (R)ph.gm1i, c1g = (R)ph.gamma * ig;   // as es_dissipation forms them
 
@@ -196,34 +212,31 @@ __global__ void __launch_bounds__(256) k_sweep(ProbArg pa, Phys ph, const double
         if (dir == 0) {
             if (line < no)
                 for (int e = lane; e < nn; e += 32)
-                    sweep_stage<R>(g, qq, qq32, pidx(g, nlo + e, line), 0, c1g, ig, sd, sf, e);
+                    sweep_stage<R>(g, qq, qq32, pidx(g, nlo + e, line), 0, c1g, ig, sf, e);
         } else {
             for (int e = threadIdx.x; e < nn * NW; e += blockDim.x) {
                 const int ww = e % NW, node = e / NW;
                 if (grp * NW + ww < no)
-                    sweep_stage<R>(g, qq, qq32, pidx(g, grp * NW + ww, nlo + node), 1, c1g, ig,
-                                   (double *)sw_smem + (size_t)ww * LY::NF64 * SW_NNP,
-                                   (float *)((double *)sw_smem + (size_t)NW * LY::NF64 * SW_NNP) +
-                                       (size_t)ww * LY::NF32 * SW_NNP,
-                                   node);
+                    sweep_stage<R>(g, qq, qq32, pidx(g, grp * NW + ww, nlo + node), 1, c1g, ig, fields_of(ww), node);
             }
         }
         __syncthreads();
 
         if (line < no) {
+            if constexpr (WW > 0) sweep_differences<R>(sf, lane, nn);
             // the anchors' pair fluxes (k_pairs): lane -> anchor L0 - (p - 1) + lane
             const int A = L0 - (P - 1) + lane;
             if (A <= Llast) {
                 const int ia = A - nlo;
-                NodeV<R> l = sweep_node<R>(sd, sf, ia);
-                const MT mtl = sMt[ia], mxl = sMx[ia], myl = sMy[ia];
+                NodeV<R> l = sweep_node<R>(sf, ia);
+                const R mtl = sMt[ia], mxl = sMx[ia], myl = sMy[ia];
 #pragma unroll
                 for (int n = 1; n <= P; ++n) {
                     const int ir = ia + n;
-                    NodeV<R> r = sweep_node<R>(sd, sf, ir);
-                    R mt = (R)((MT)0.5 * (mtl + sMt[ir]));
-                    R mx = (R)((MT)0.5 * (mxl + sMx[ir]));
-                    R my = (R)((MT)0.5 * (myl + sMy[ir]));
+                    NodeV<R> r = sweep_node<R>(sf, ir);
+                    R mt = (R)0.5 * (mtl + sMt[ir]);
+                    R mx = (R)0.5 * (mxl + sMx[ir]);
+                    R my = (R)0.5 * (myl + sMy[ir]);
                     R out[4];
                     ec_pair<R>(l, r, mt, mx, my, gm1inv, ph.ln_thr, out);
 #pragma unroll
@@ -237,41 +250,29 @@ __global__ void __launch_bounds__(256) k_sweep(ProbArg pa, Phys ph, const double
             if (lane < TA && L <= Llast) {
                 const int i0 = L - nlo;
                 R F[4] = {(R)0, (R)0, (R)0, (R)0};
-                MT Ft = (MT)0;
+                R Ft = (R)0;
 #pragma unroll
                 for (int n = 1; n <= P; ++n) {
                     R Fs[4] = {(R)0, (R)0, (R)0, (R)0};
-                    MT Fts = (MT)0;
+                    R Fts = (R)0;
 #pragma unroll
                     for (int s = 0; s < n; ++s) {
                         const R *pr = spr + (n - 1) * 4 * 32 + (lane + P - 1 - s);
 #pragma unroll
                         for (int a = 0; a < 4; ++a) Fs[a] += pr[a * 32];
-                        Fts += (MT)0.5 * (sMt[i0 - s] + sMt[i0 - s + n]);
+                        Fts += (R)0.5 * (sMt[i0 - s] + sMt[i0 - s + n]);
                     }
                     const R an = (R)ph.alpha[n - 1];
 #pragma unroll
-                    for (int a = 0; a < 4; ++a) F[a] += an * Fs[a];
-                    Ft += (MT)ph.alpha[n - 1] * Fts;
+                    for (int a = 0; a < 4; ++a) F[a] = fma_<R>(an, Fs[a], F[a]);
+                    Ft += an * Fts;
                 }
                 if constexpr (WW > 0) {
                     const int i1 = i0 + 1;
-                    const R nvx = (R)((MT)0.5 * (sMx[i0] + sMx[i1])), nvy = (R)((MT)0.5 * (sMy[i0] + sMy[i1]));
-                    const R jt = (R)((MT)0.5 * (sMt[i0] + sMt[i1]));
-                    const double rho0 = sd[0 * SW_NNP + i0], rho1 = sd[0 * SW_NNP + i1];
-                    const double lnr0 = sd[2 * SW_NNP + i0], lnr1 = sd[2 * SW_NNP + i1];
-                    R diss[4];
-                    if constexpr (F32) {
-                        SmemStencil<float> st{sf, i0 - (WW - 1) / 2};
-                        es_dissipation<R, double, WW>(nvx, nvy, jt, rho0, rho1, lnr0, lnr1, sf[0 * SW_NNP + i0],
-                                                      sf[0 * SW_NNP + i1], st, ph, diss);
-                    } else {
-                        SmemStencil<double> st{sd, i0 - (WW - 1) / 2};
-                        es_dissipation<R, double, WW>(nvx, nvy, jt, rho0, rho1, lnr0, lnr1, (R)rho0, (R)rho1, st, ph,
-                                                      diss);
-                    }
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) F[a] -= diss[a];
+                    const R nvx = (R)0.5 * (sMx[i0] + sMx[i1]), nvy = (R)0.5 * (sMy[i0] + sMy[i1]);
+                    const R jt = (R)0.5 * (sMt[i0] + sMt[i1]);
+                    const SmemStencil<R> st{sf, i0 - (WW - 1) / 2};
+                    es_dissipation<R, WW>(nvx, nvy, jt, sf.lm(0, i0), sf.lm(0, i1), st, ph, F);
                 }
                 const long long c0 = dir == 0 ? pidx(g, L, line) : pidx(g, line, L);
                 R *out = fl + (long long)(dir * 5) * g.P + c0;
