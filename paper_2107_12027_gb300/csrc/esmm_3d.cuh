@@ -120,28 +120,30 @@ __device__ __forceinline__ double delta_x3(const Geom3 &g, const double *x, int 
 // vanishes does not orient the frame).
 __device__ __forceinline__ void frame3(const double n[3], double T[3][3])
 {
-    double r = sqrt(n[0] * n[0] + n[1] * n[1]);
-    bool pole = r <= 1.0e-12;
-    double ct = pole ? 1.0 : n[0] / r, st = pole ? 0.0 : n[1] / r;
+    const double r2 = n[0] * n[0] + n[1] * n[1];
+    const bool pole = !(r2 > 1.0e-24);
+    const double ir = pole ? 0.0 : qrsq<double>(r2), r = pole ? sqrt(r2) : r2 * ir;
+    double ct = pole ? 1.0 : n[0] * ir, st = n[1] * ir;
     double cp = r, sp = n[2];
     T[0][0] = cp * ct; T[0][1] = cp * st; T[0][2] = sp;
     T[1][0] = -st;     T[1][1] = ct;      T[1][2] = 0.0;
     T[2][0] = -sp * ct; T[2][1] = -sp * st; T[2][2] = cp;
 }
 
-__device__ __forceinline__ void align3(double T[3][3], const double w[8])
+// (B, u: the state's field and spatial 4-velocity, iW = 1/W)
+__device__ __forceinline__ void align3(double T[3][3], const double u[3], double iW, const double B[3])
 {
-    double b1 = T[1][0] * w[5] + T[1][1] * w[6] + T[1][2] * w[7];
-    double b2 = T[2][0] * w[5] + T[2][1] * w[6] + T[2][2] * w[7];
-    double B2 = w[5] * w[5] + w[6] * w[6] + w[7] * w[7];
+    double b1 = T[1][0] * B[0] + T[1][1] * B[1] + T[1][2] * B[2];
+    double b2 = T[2][0] * B[0] + T[2][1] * B[1] + T[2][2] * B[2];
+    double B2 = B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
     double t2 = b1 * b1 + b2 * b2;
     if (!(t2 > 1.0e-20 * (1.0 + B2))) {
-        b1 = T[1][0] * w[1] + T[1][1] * w[2] + T[1][2] * w[3];
-        b2 = T[2][0] * w[1] + T[2][1] * w[2] + T[2][2] * w[3];
+        b1 = (T[1][0] * u[0] + T[1][1] * u[1] + T[1][2] * u[2]) * iW;
+        b2 = (T[2][0] * u[0] + T[2][1] * u[1] + T[2][2] * u[2]) * iW;
         t2 = b1 * b1 + b2 * b2;
         if (!(t2 > 1.0e-20)) return;
     }
-    double tn = sqrt(t2), c = b1 / tn, s = b2 / tn;
+    const double itn = qrsq<double>(t2), c = b1 * itn, s = b2 * itn;
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
         double a1 = T[1][q], a2 = T[2][q];
@@ -175,12 +177,10 @@ __device__ __forceinline__ void unrot3(const double T[3][3], const double *r, do
 __device__ __forceinline__ NodeM load3(const double *__restrict__ q, long long P, long long c)
 {
     NodeM v;
-    v.rho = q[F_RHO * P + c];
-    v.beta = q[F_BETA * P + c];
-    v.lnr = q[F_LNR * P + c];
-    v.lnb = q[F_LNB * P + c];
-    v.r = v.rho;
-    v.b = v.beta;
+    v.rho.v = q[F_RHO * P + c];
+    v.rho.l = q[F_LNR * P + c];
+    v.beta.v = q[F_BETA * P + c];
+    v.beta.l = q[F_LNB * P + c];
     v.W = q[F_W * P + c];
     v.u[0] = q[F_U0 * P + c];
     v.u[1] = q[F_U1 * P + c];
@@ -198,7 +198,7 @@ __device__ __forceinline__ void node_V3(const double *__restrict__ q, long long 
     double u0 = q[F_U0 * P + c], u1 = q[F_U1 * P + c], u2 = q[F_U2 * P + c];
     double B0 = q[F_B0 * P + c], B1 = q[F_B1 * P + c], B2 = q[F_B2 * P + c];
     double b0 = u0 * B0 + u1 * B1 + u2 * B2;
-    double bW = beta / W;
+    double bW = beta * qrcp<double>(W);
     V[0] = c1g + q[F_LNR * P + c] + ig * q[F_LNB * P + c] + beta;
     V[1] = beta * u0;
     V[2] = beta * u1;
@@ -240,97 +240,63 @@ __global__ void __launch_bounds__(128) k3_iface(Geom3 g, Phys ph, const double *
             double mm[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) mm[a] = 0.5 * (Md[a * g.P + cl] + Md[a * g.P + cr]);
+            const double mt = 0.5 * (Mt[cl] + Mt[cr]);
             double out[8];
-            ec_pair_mhd<3>(l, r, gm1inv, ph.ln_thr, 0.5 * (Mt[cl] + Mt[cr]), mm, out);
+            ec_pair_mhd<3>(l, r, gm1inv, ph.ln_thr, mt, mm, out);
 #pragma unroll
             for (int a = 0; a < 8; ++a) Fs[a] += out[a];
-            Fts += 0.5 * (Mt[cl] + Mt[cr]);
+            Fts += mt;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) Bts += 0.5 * mm[a] * (l.B[a] + r.B[a]);
+            for (int a = 0; a < 3; ++a) Bts += mm[a] * (l.B[a] + r.B[a]);
         }
         const double an = ph.alpha[n - 1];
 #pragma unroll
         for (int a = 0; a < 8; ++a) F[a] += an * Fs[a];
         Ft += an * Fts;
-        Bt += an * Bts;
+        Bt += 0.5 * an * Bts;
     }
-    if (WW > 0) {
-        constexpr int NS = WW + 1, OFF = (WW - 1) / 2;
+    if constexpr (WW > 0) {
+        constexpr int OFF = (WW - 1) / 2;
         const long long c1 = c0 + sd;
         double nv[3], nn[3], T[3][3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) nv[a] = 0.5 * (Md[a * g.P + c0] + Md[a * g.P + c1]);
         const double jt = 0.5 * (Mt[c0] + Mt[c1]);
-        const double Lk = sqrt(nv[0] * nv[0] + nv[1] * nv[1] + nv[2] * nv[2]);
+        const double n2 = nv[0] * nv[0] + nv[1] * nv[1] + nv[2] * nv[2], iLk = qrsq<double>(n2), Lk = n2 * iLk;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) nn[a] = nv[a] / Lk;
+        for (int a = 0; a < 3; ++a) nn[a] = nv[a] * iLk;
         frame3(nn, T);
-        double wm[8], wrot[8];
+        double rho, p, ip, us[3], Bs[3];
         {
-            double rho, irho;
-            logmean<double, double>(q[F_RHO * g.P + c0], q[F_RHO * g.P + c1], q[F_LNR * g.P + c0],
-                                    q[F_LNR * g.P + c1], ph.ln_thr, rho, irho);
-            double um[3], W2 = 1.0;
+            const NodeM l = load3(q, g.P, c0), r = load3(q, g.P, c1);
+            double irho, um[3], Bm[3], W2 = 1.0;
+            logmean2<double>(l.rho, r.rho, ph.ln_thr, rho, irho);
+            const double sr = l.rho.v + r.rho.v, sb = l.beta.v + r.beta.v;
+            p = sr * qrcp<double>(sb);
+            ip = sb * qrcp<double>(sr);
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                um[a] = 0.5 * (q[(F_U0 + a) * g.P + c0] + q[(F_U0 + a) * g.P + c1]);
+                um[a] = 0.5 * (l.u[a] + r.u[a]);
+                Bm[a] = 0.5 * (l.B[a] + r.B[a]);
                 W2 += um[a] * um[a];
             }
-            double W = sqrt(W2);
-            wm[0] = rho;
+            align3(T, um, qrsq<double>(W2), Bm);
 #pragma unroll
-            for (int a = 0; a < 3; ++a) wm[1 + a] = um[a] / W;
-            wm[4] = (q[F_RHO * g.P + c0] + q[F_RHO * g.P + c1]) / (q[F_BETA * g.P + c0] + q[F_BETA * g.P + c1]);
-#pragma unroll
-            for (int a = 0; a < 3; ++a) wm[5 + a] = 0.5 * (q[(F_B0 + a) * g.P + c0] + q[(F_B0 + a) * g.P + c1]);
-        }
-        align3(T, wm);
-        rot3(T, wm, wrot);
-        double lam[8], R[8][8];
-        eigen_mhd<double>(ph.gamma, wrot, lam, R);
-        double lhat = 0.0;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) lhat = fmax(lhat, fabs(jt + Lk * lam[m]));
-        const double ig = gm1inv, c1g = ph.gamma * gm1inv;
-        double Vt[NS][8], scale[8];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) scale[m] = 0.0;
-        for (int kk = 0; kk < NS; ++kk) {
-            double V[8], TV[8];
-            node_V3(q, g.P, c0 + (kk - OFF) * sd, c1g, ig, V);
-            rot3(T, V, TV);
-            for (int m = 0; m < 8; ++m) {
-                double acc = 0.0;
-                for (int a = 0; a < 8; ++a) {
-                    double t = R[a][m] * TV[a];
-                    acc += t;
-                    if (kk == OFF || kk == OFF + 1) scale[m] += fabs(t);
-                }
-                Vt[kk][m] = acc;
+            for (int a = 0; a < 3; ++a) {
+                us[a] = T[a][0] * um[0] + T[a][1] * um[1] + T[a][2] * um[2];
+                Bs[a] = T[a][0] * Bm[0] + T[a][1] * Bm[1] + T[a][2] * Bm[2];
             }
         }
-        double z[8];
-        for (int m = 0; m < 8; ++m) {
-            double vminus, vplus;
-            if (WW == 5)
-                weno5_lr<double>(Vt[0][m], Vt[1][m], Vt[2][m], Vt[3][m], Vt[4][m], Vt[5][m], ph.eps, vminus, vplus);
-            else
-                weno3_lr<double>(Vt[0][m], Vt[1][m], Vt[2][m], Vt[3][m], ph.eps, vminus, vplus);
-            double jw = vplus - vminus;
-            double jump = Vt[OFF + 1][m] - Vt[OFF][m];
-            int sj = fabs(jump) <= ph.sign_tol * scale[m] ? 0 : sgn_d(jump);
-            z[m] = (sgn_d(jw) == sj) ? jw : 0.0;
-        }
+        const double ig = gm1inv, c1g = ph.gamma * gm1inv;
         double d[8], dr[8];
-        for (int a = 0; a < 8; ++a) {
-            double acc = 0.0;
-            for (int m = 0; m < 8; ++m) acc += R[a][m] * z[m];
-            d[a] = acc;
-        }
+        es_dissipation_mhd<double, WW>(ph, rho, p, ip, us, Bs, Lk, jt, [&](int k, double TV[8]) {
+            double V[8];
+            node_V3(q, g.P, c0 + (k - OFF) * sd, c1g, ig, V);
+            rot3(T, V, TV);
+        }, d);
         unrot3(T, d, dr);
-        const double hl = 0.5 * lhat;
 #pragma unroll
-        for (int a = 0; a < 8; ++a) F[a] -= hl * dr[a];
+        for (int a = 0; a < 8; ++a) F[a] -= dr[a];
     }
     double *out = iflux + (long long)(dir * NF3) * g.P + c0;
 #pragma unroll

@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(128) k3_iface_vjp(Geom3 g, Phys ph, const doub
     }
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < 3; ++b) T[a][b] = T0[a][b];
-    align3(T, wm);
+    align3(T, wm + 1, 1.0, wm + 5);
     // which quantity turned the frame (as align3 decides): 1 = B, 2 = v, 0 = none
     int mode = 0, fo = 5;
     double tb1, tb2, tt2;

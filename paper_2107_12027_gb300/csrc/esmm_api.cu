@@ -68,7 +68,7 @@ struct esmm_grid {
     double *cw;                      // [4][Ntot] Jacobi weights of the mesh iteration
     double *rs;                      // [2][Ntot] the iteration's residual on the displacement
     double *wr;                      // [6][Ntot] floats: weights and residual of the blocked sweeps
-    float *q32;                      // [NQ32][Ptot] FP32 copies (RHD mixed form)
+    float *q32;                      // [NQ32 or NQ32_MHD][Ptot] FP32 copies (mixed form)
     double *inflow_dev;              // [8] primitive inflow state (ESMM_INFLOW ends)
     int needs_inflow, has_inflow;
     double *pg[3];                   // recovery warm starts (p; RMHD: Z), state -> stage 2 -> stage 3
@@ -382,7 +382,8 @@ void node(esmm_grid *g, const double *cons, const double *J, const double *x, co
     if (g->phys == ESMM_RMHD)
         launch_node_mhd(dom(g, D_PAD), g->p, g->gamma, cons, J, x, xdot, pg_in, pg_out, g->q, g->status,
                         g->has_inflow ? g->inflow_dev : nullptr,
-                        g->prm.precision == ESMM_MIXED && !exact_logs, g->st);
+                        g->prm.precision == ESMM_MIXED && !exact_logs,
+                        g->prm.precision == ESMM_MIXED ? g->q32 : nullptr, g->st);
     else
         launch_node(g, dom(g, D_PAD), cons, J, x, xdot, pg_in, pg_out, g->q, exact_logs);
 }
@@ -398,7 +399,7 @@ void fluxes(esmm_grid *g)
         LaunchDom Li = dom(g, rmhd ? (dir == 0 ? D_IFACE0 : D_IFACE1) : (dir == 0 ? D_TIFACE0 : D_TIFACE1));
         if (rmhd) {   // two-point fluxes summed inside the interface kernel
             Prof pr_(g, ESMM_KIND_IFACE);
-            if (f32) launch_iface_mhd_f32(Li, ph, g->q, g->iflux, dir, g->st);
+            if (f32) launch_iface_mhd_f32(Li, ph, g->q, g->q32, g->iflux, dir, g->st);
             else launch_iface_mhd(Li, ph, g->q, g->iflux, dir, g->st);
             continue;
         }
@@ -909,7 +910,8 @@ int create(esmm_grid **out, int nprob, const int *n, const double *lo, const dou
     }
     size_t npairs = phys == ESMM_RMHD ? 1 : (size_t)2 * PMAX * 4 * P;
     size_t nflux = phys == ESMM_RMHD ? (size_t)2 * NF_MHD * P : (size_t)2 * 5 * P;
-    if ((phys == ESMM_RHD && cudaMalloc((void **)&g->q32, (size_t)NQ32 * P * sizeof(float)) != cudaSuccess) ||
+    const size_t nq32 = phys == ESMM_RMHD ? (size_t)NQ32_MHD : (size_t)NQ32;
+    if (cudaMalloc((void **)&g->q32, nq32 * P * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&g->pairs, npairs * d) != cudaSuccess || cudaMalloc(&g->iflux, nflux * d) != cudaSuccess ||
         cudaMalloc((void **)&g->red, (size_t)NRED * nprob * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMalloc((void **)&g->ds, (size_t)nprob * sizeof(DtSolve)) != cudaSuccess ||
@@ -1275,7 +1277,7 @@ int tune(esmm_grid *g)
                             ms = c.kind == D_PAIR0 ? 0.0f : time_it([&]() {
                                 for (int dir = 0; dir < 2; ++dir)
                                     if (f32)
-                                        launch_iface_mhd_f32(dom(g, dir ? c.kind2 : c.kind), ph, g->q, g->iflux,
+                                        launch_iface_mhd_f32(dom(g, dir ? c.kind2 : c.kind), ph, g->q, g->q32, g->iflux,
                                                              dir, g->st);
                                     else
                                         launch_iface_mhd(dom(g, dir ? c.kind2 : c.kind), ph, g->q, g->iflux, dir,

@@ -504,36 +504,7 @@ __device__ __forceinline__ void logmean(T a, T b, T la, T lb, double thr, R &mea
     }
 }
 
-// The log mean of two nodes, a32 and b32 being the working-precision copies
-// of a and b: in FP64 and on duals exactly logmean.  In FP32 the jumps b - a
-// and ln b - ln a, which cancel at near-equal states, are taken in FP64 from
-// the FP64 node values; the series (switch at (b-a)^2 < thr (a+b)^2) and the
-// quotients then run in FP32, whose rounding of the result they already are
-// below (the series' terms beyond 1 are < thr/3).
-template <typename R, typename T>
-__device__ __forceinline__ void lmean(T a, T b, T la, T lb, R a32, R b32, double thr, R &mean, R &inv_mean)
-{
-    logmean<R, T>(a, b, la, lb, thr, mean, inv_mean);
-}
-template <>
-__device__ __forceinline__ void lmean<float, double>(double a, double b, double la, double lb, float a32, float b32,
-                                                     double thr, float &mean, float &inv_mean)
-{
-    const float d = (float)(b - a), s = a32 + b32;
-    if (d * d < (float)thr * (s * s)) {
-        const float is = __frcp_rn(s);
-        const float r = d * is, u = r * r;
-        const float F = 1.0f + u * (1.0f / 3.0f + u * (1.0f / 5.0f + u * (1.0f / 7.0f)));
-        mean = 0.5f * s * __frcp_rn(F);
-        inv_mean = 2.0f * F * is;
-    } else {
-        const float dl = (float)(lb - la);
-        mean = d * __frcp_rn(dl);
-        inv_mean = dl * __frcp_rn(d);
-    }
-}
-
-// An argument of the RHD log means: the value and its logarithm, in FP32 with the
+// An argument of the log means: the value and its logarithm, in FP32 with the
 // rest of the FP64 value, so that the jump of two near-equal values keeps FP32
 // relative precision without FP64 arithmetic: (b.v - a.v) is exact within a factor 2
 // of each other, and v + lo carries 48 bits.

@@ -84,13 +84,13 @@ constexpr int NQ_MHD = 18;
 constexpr int NF_MHD = 10;
 void launch_node_mhd(const LaunchDom &L, int p, double gam, const double *cons, const double *J, const double *x,
                      const double *xdot, const double *zg_in, double *zg_out, double *q, int *status,
-                     const double *inflow, int f32_logs, cudaStream_t st);
+                     const double *inflow, int f32_logs, float *q32, cudaStream_t st);
 void launch_iface_mhd(const LaunchDom &L, const Phys &ph, const double *q, void *iflux, int dir, cudaStream_t st);
 void launch_update_mhd(const LaunchDom &L, const double *q, const void *fl, double *dcons, double *dJ,
                        const double *cn, const double *Jn, const double *xn, const double *cs, const double *Js,
                        const double *xs, const double *xdot, double A, double B, const double *dt_dev, double *co,
                        double *Jo, double *xo, cudaStream_t st);
-void launch_iface_mhd_f32(const LaunchDom &L, const Phys &ph, const double *q, void *iflux, int dir,
+void launch_iface_mhd_f32(const LaunchDom &L, const Phys &ph, const double *q, const float *q32, void *iflux, int dir,
                           cudaStream_t st);
 void launch_update_mhd_f32(const LaunchDom &L, const double *q, const void *fl, double *dcons, double *dJ,
                            const double *cn, const double *Jn, const double *xn, const double *cs, const double *Js,
@@ -116,6 +116,7 @@ void launch_node_vjp_mhd(const LaunchDom &L, double gam, const double *q, const 
 void launch_prim_grad_mhd(const LaunchDom &L, double gam, const double *cons, const double *J, const double *lam,
                           double *out, int *status, cudaStream_t st);
 constexpr long long ADJ_LAMQ_PER_NODE = 11;
+constexpr int NQ32_MHD = 13;   // FP32 copies per padded node (the mixed form)
 // esmm_mhd_eigen (host arrays): 0, or 1 on a CUDA failure
 int mhd_eigen_host(double gam, int n, const double *w, const double *dw, double *lam, double *R, double *dlam,
                    double *dR);

@@ -19,6 +19,12 @@
 namespace esmm {
 
 enum { QM_UZ = NQ, QM_B1, QM_B2, QM_B3, NQM };   // 18 node arrays (NQ_MHD)
+// FP32 copies for the mixed form's flux kernel, written by the FP64 node pass (an
+// interface reads 26 nodes' values: converting them there took about as many instructions
+// as its arithmetic); RLO, BLO: the FP64 rests of rho and beta
+enum { QM32_R = 0, QM32_B, QM32_LNR, QM32_LNB, QM32_W, QM32_U0, QM32_U1, QM32_U2, QM32_B0, QM32_B1, QM32_B2, QM32_RLO,
+       QM32_BLO, NQM32 };
+static_assert(NQM32 == NQ32_MHD, "the allocation of the FP32 copies");
 constexpr int NFM = 10;                          // interface values per direction: F[8], J xi_t, B~ (NF_MHD)
 
 // ---------------------------------------------------------------------------
@@ -533,7 +539,7 @@ static __device__ __noinline__ void mhd_canonical(double gam, const R w[8], cons
     int start = 0;
     while (start < 6) {
         int end = start + 1;
-        while (end < 6 && lam[2 + end] - lam[1 + end] < (R)MHD_CLUSTER_TOL) ++end;
+        while (end < 6 && mhd_close<R>(lam[1 + end], lam[2 + end])) ++end;
         const int k = end - start;
         if (k > 1) {
             // E = L^T S, orthonormalized (twice: the waves of a cluster may be
@@ -601,8 +607,7 @@ static __device__ __noinline__ void eigen_mhd(double gam, const R w[8], R lam[8]
     const R gg = (R)(gam / (gam - 1.0));
     MhdBase<R> s;
     mhd_base<R>((R)gam, gg, w, s);
-    const R lim = (R)(sizeof(R) == 4 ? 1.0e-12 : 1.0e-25);
-    if (!(s.gp > lim && s.e < (R)1 / lim)) {
+    if (!mhd_in_range<R>(s)) {
         eigen_mhd_gram<R>(gam, w, lam, Rv, true);
         return;
     }
@@ -611,36 +616,17 @@ static __device__ __noinline__ void eigen_mhd(double gam, const R w[8], R lam[8]
     mhd_six<R>(s, x, lam + 2);
     bool cluster = false;
 #pragma unroll
-    for (int m = 0; m < 5; ++m) cluster = cluster || lam[3 + m] - lam[2 + m] < (R)MHD_CLUSTER_TOL;
-    // the entropy wave d rho = 1 and the divergence wave dB = e_1 - v_1 v
-    {
-        const R sr = rsq<R>(gg * s.W * rcp<R>(s.rho));
-        Rv[0][0] = s.W * sr;
-        for (int k = 0; k < 3; ++k) Rv[1 + k][0] = s.W * s.u[1 + k] * sr;
-        Rv[4][0] = s.W * s.W * sr;
-        for (int k = 5; k < 8; ++k) Rv[k][0] = (R)0;
-        MhdWave<R> q;
-        const R dB[3] = {(R)1 - s.v1 * s.v1, -s.v1 * w[2], -s.v1 * w[3]};
-        q.rho = q.p = (R)0;
-        q.b[0] = s.v1 * s.iW;
-        q.u[0] = (R)0;
-        for (int k = 0; k < 3; ++k) {
-            q.u[1 + k] = (R)0;
-            q.b[1 + k] = (dB[k] + q.b[0] * s.u[1 + k]) * s.iW;
-        }
-        const R sd = rsq<R>(s.beta * s.W * mdot<R>(q.b, q.b));
-        for (int k = 0; k < 4; ++k) q.b[k] *= sd;
-        R dU[8];
-        mhd_wave_dU<R>(s, gg, q, dU);
-        for (int r = 0; r < 8; ++r) Rv[r][1] = dU[r];
-    }
+    for (int m = 0; m < 5; ++m) cluster = cluster || mhd_close<R>(lam[2 + m], lam[3 + m]);
+    R dU[8];
+    mhd_entropy_dU<R>(s, (R)((gam - 1.0) / gam), dU);
+    for (int r = 0; r < 8; ++r) Rv[r][0] = dU[r];
+    mhd_divergence_dU<R>(s, dU);
+    for (int r = 0; r < 8; ++r) Rv[r][1] = dU[r];
     R S[6][6];
 #pragma unroll 1
     for (int m = 0; m < 6; ++m) {
         MhdWave<R> q;
-        mhd_six_wave<R>(s, x, m, q);
-        R dU[8];
-        mhd_wave_dU<R>(s, gg, q, dU);
+        mhd_six_wave<R, false>(s, x, gg, m, q, dU);
         for (int r = 0; r < 8; ++r) Rv[r][2 + m] = dU[r];
         if (cluster) {   // the wave's coefficients in the y_a
             for (int k = 0; k < 3; ++k) S[k][m] = (q.u[1 + k] - w[1 + k] * q.u[0]) * s.iW;
@@ -659,50 +645,245 @@ static __device__ __noinline__ void mhd_speed_range(double gam, const R w[8], R 
 {
     MhdBase<R> s;
     mhd_base<R>((R)gam, (R)(gam / (gam - 1.0)), w, s);
-    const R lim = (R)(sizeof(R) == 4 ? 1.0e-12 : 1.0e-25);
-    if (!(s.gp > lim && s.e < (R)1 / lim)) {
+    if (!mhd_in_range<R>(s)) {
         R lam[8], Rm[8][8];
         eigen_mhd_gram<R>(gam, w, lam, Rm, false);
         lo = lam[2];
         hi = lam[7];
         return;
     }
-    const R sqe = sq_rt<R>(s.e);
+    MhdCoef<R> kc;
+    mhd_coef<R>(s, kc);
     R tA, ts, tf;
-    mhd_side<R>(s, sqe, 1, false, tA, ts, tf);
+    mhd_side<R>(s, kc, 1, false, tA, ts, tf);
     lo = s.v1 - tf * s.iW;
-    mhd_side<R>(s, sqe, -1, false, tA, ts, tf);
+    mhd_side<R>(s, kc, -1, false, tA, ts, tf);
     hi = s.v1 + tf * s.iW;
 }
 
+// The canonical basis (mhd_canonical) of a cluster of two waves a, b of one side, an
+// Alfven and a magnetosonic one: they are orthogonal whatever their speeds (s is normal to
+// t, k and b), so a rotation of the two columns is all that is needed, and its first
+// vector is the first row (E[i][a], E[i][b]) of E = L^T S whose squared norm is at least
+// 1/8; the second is the complement.  Row i takes the directions e_0 .. e_i alone, and
+// e_0 or e_1 (v_1, v_2) nearly always decides: e_{v_k} in closed form,
+//   du = (W u_k, e_k + u_k u) (times W), db from B = const,  dV = beta (0, du, -du^0, db),
+// with <e_i, a> = dV(e_i).R_a, and <e_i, e_j> from the bilinear form X^0.  Returns false
+// where neither row decides.  (~150 operations, against ~3,500 of eigen_mhd and the whole
+// Gram matrix: a rotor's ambient field along x_1 leaves clusters in half the interfaces
+// of that sweep.)  Rv: rows dU of the waves, rows 0 and 1 the entropy and divergence waves.
+template <typename R>
+__device__ __forceinline__ bool mhd_turn_pair(const MhdBase<R> &s, const R B[3], R Rv[8][8], int a)
+{
+    R du[2][4], db[2][4], P[2], c, sn;
+    R Ea = (R)0, Eb = (R)0, i0 = (R)0, f0r = (R)0, f0d = (R)0;
+    bool ok = false;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        if (ok) break;
+        const R uk = s.u[1 + i];
+        du[i][0] = s.W * uk;
+#pragma unroll
+        for (int k = 1; k < 4; ++k) du[i][k] = (k == 1 + i ? (R)1 : (R)0) + s.u[k] * uk;
+        db[i][0] = du[i][1] * B[0] + du[i][2] * B[1] + du[i][3] * B[2];
+#pragma unroll
+        for (int k = 1; k < 4; ++k) db[i][k] = (db[i][0] * s.u[k] + s.b[0] * du[i][k] - s.b[k] * du[i][0]) * s.iW;
+        P[i] = mdot<R>(s.b, db[i]);
+        R f[4];   // <e_i, .> with the entropy, the divergence wave, a and b, over beta
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            const R *r = n < 2 ? Rv[n] : Rv[a + n - 2];
+            f[n] = du[i][1] * r[1] + du[i][2] * r[2] + du[i][3] * r[3] - du[i][0] * r[4] + db[i][1] * r[5] + db[i][2] * r[6] +
+                   db[i][3] * r[7];
+        }
+        // Gram entries over beta
+        const R gii = s.W * (s.e * mdot<R>(du[i], du[i]) + mdot<R>(db[i], db[i])) +
+                      (R)2 * (du[i][0] * P[i] - s.b[0] * mdot<R>(db[i], du[i])) - s.beta * (f[0] * f[0] + f[1] * f[1]);
+        R ea = f[2], eb = f[3], d = gii;
+        if (i == 0) {
+            f0r = f[0];
+            f0d = f[1];
+        } else {
+            const R g10 = s.W * (s.e * mdot<R>(du[0], du[1]) + mdot<R>(db[0], db[1])) + du[0][0] * P[1] + du[1][0] * P[0] -
+                          s.b[0] * (mdot<R>(db[0], du[1]) + mdot<R>(db[1], du[0])) - s.beta * (f0r * f[0] + f0d * f[1]);
+            const R l = g10 * i0;   // L_10 over L_00, times sqrt(g00)
+            d -= l * g10;
+            ea -= l * Ea;
+            eb -= l * Eb;
+        }
+        // |row|^2 = beta (ea^2 + eb^2) / d
+        const R n2 = ea * ea + eb * eb;
+        if (to_f32(s.beta * n2) >= 0.125f * to_f32(d)) {
+            const R inr = qrsq<R>(n2);
+            c = ea * inr;
+            sn = eb * inr;
+            ok = true;
+        }
+        Ea = ea;
+        Eb = eb;
+        i0 = qrcp<R>(gii);
+    }
+    if (!ok) return false;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        const R x = Rv[a][r], y = Rv[a + 1][r];
+        Rv[a][r] = c * x + sn * y;
+        Rv[a + 1][r] = c * y - sn * x;
+    }
+    return true;
+}
+
+// The ES dissipation of one interface in its rotated frame (first axis along the
+// normal): with the interface state rho = {{rho}}^ln, u = {{u}}, p = 1/ip, B = {{B}}
+// and the scaled eigenvectors R, d = lambda^/2 R Y <<R^T V>>, lambda^ the largest |jt + Lk
+// lambda_m| (reached by a fast wave).  rotV(k, V) gives the rotated entropy variables of the
+// stencil's node k.  The dissipation depends on differences of V alone, so those are
+// projected (w of them), and the wave's edge jump comes from them (weno5_jump); the
+// switch's tolerance, a threshold, is formed in FP32 from |R| and |V|.  Clusters of two
+// waves of one side are turned (mhd_turn_pair); interfaces with other clusters, or
+// outside the closed form's range, take their vectors from eigen_mhd.
+template <typename R, int WW, typename ROTV>
+__device__ __forceinline__ void es_dissipation_mhd(const Phys &ph, R rho, R p, R ip, const R us[3], const R Bs[3], R Lk,
+                                                   R jt, ROTV rotV, R d[8])
+{
+    constexpr int OFF = (WW - 1) / 2;
+    const R gg = (R)(ph.gamma * ph.gm1i);
+    R lo, hi, Rv[8][8];   // (a row per wave)
+    {
+        MhdBase<R> s;
+        const R W2 = (R)1 + (us[0] * us[0] + us[1] * us[1] + us[2] * us[2]), iW = qrsq<R>(W2);
+        mhd_base_u<R>((R)ph.gamma, gg, rho, p, ip, W2 * iW, iW, us, Bs, s);
+        bool whole = !mhd_in_range<R>(s);
+        if (!whole) {
+            MhdSix<R> x;
+            R l6[6];
+            mhd_six<R>(s, x, l6);
+            lo = l6[0];
+            hi = l6[5];
+            int near = 0;   // bit m: waves m and m + 1 in one cluster
+#pragma unroll
+            for (int m = 0; m < 5; ++m) near |= (int)mhd_close<R>(l6[m], l6[m + 1]) << m;
+            whole = (near & 4) != 0 || (near & (near >> 1)) != 0;   // slow waves of both sides, or three and more
+            if (!whole) {
+                mhd_entropy_dU<R>(s, (R)ph.igg, Rv[0]);
+                mhd_divergence_dU<R>(s, Rv[1]);
+#pragma unroll 1
+                for (int m = 0; m < 6; ++m) {
+                    MhdWave<R> q;
+                    mhd_six_wave<R, false>(s, x, gg, m, q, Rv[2 + m]);
+                }
+                if (near)
+#pragma unroll 1
+                    for (int m = 0; m < 5; ++m)
+                        if (near >> m & 1) whole = !mhd_turn_pair<R>(s, Bs, Rv, 2 + m) || whole;
+            }
+        }
+        if (whole) {
+            R lam[8], Rc[8][8];
+            const R w[8] = {rho, us[0] * s.iW, us[1] * s.iW, us[2] * s.iW, p, Bs[0], Bs[1], Bs[2]};
+            eigen_mhd<R>(ph.gamma, w, lam, Rc);
+            lo = lam[2];
+            hi = lam[7];
+            for (int m = 0; m < 8; ++m)
+                for (int r = 0; r < 8; ++r) Rv[m][r] = Rc[r][m];
+        }
+    }
+    R D[WW][8];
+    float aT[8];
+    {
+        R V[2][8];
+        rotV(0, V[0]);
+#pragma unroll
+        for (int k = 0; k < WW; ++k) {
+            R *va = V[k & 1], *vb = V[(k + 1) & 1];
+            rotV(k + 1, vb);
+#pragma unroll
+            for (int a = 0; a < 8; ++a) {
+                if (k == OFF) aT[a] = fabsf(to_f32(va[a])) + fabsf(to_f32(vb[a]));
+                D[k][a] = sub_<R>(vb[a], va[a]);
+            }
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 8; ++a) d[a] = (R)0;
+#pragma unroll 1
+    for (int m = 0; m < 8; ++m) {
+        R r[8];
+#pragma unroll
+        for (int a = 0; a < 8; ++a) r[a] = Rv[m][a];
+        R Dt[WW];
+#pragma unroll
+        for (int k = 0; k < WW; ++k) {
+            R acc = r[0] * D[k][0];
+#pragma unroll
+            for (int a = 1; a < 8; ++a) acc += r[a] * D[k][a];
+            Dt[k] = acc;
+        }
+        float scale = 0.0f;
+#pragma unroll
+        for (int a = 0; a < 8; ++a) scale += fabsf(to_f32(r[a])) * aT[a];
+        R jw;
+        if constexpr (WW == 5) jw = weno5_jump<R>(Dt[0], Dt[1], Dt[2], Dt[3], Dt[4], (R)(4.0 * ph.eps));
+        else jw = weno3_jump<R>(Dt[0], Dt[1], Dt[2], (R)ph.eps);
+        const R jump = Dt[OFF];
+        const int sj = fabsf(to_f32(jump)) <= (float)ph.sign_tol * scale ? 0 : sgn_d(jump);
+        const R z = sgn_d(jw) == sj ? jw : (R)0;
+#pragma unroll
+        for (int a = 0; a < 8; ++a) d[a] += r[a] * z;
+    }
+    const R hl = (R)0.5 * vmax(fab<R>(jt + Lk * lo), fab<R>(jt + Lk * hi));
+#pragma unroll
+    for (int a = 0; a < 8; ++a) d[a] *= hl;
+}
+
 // ---------------------------------------------------------------------------
-// Node values of one two-point flux argument: the log-mean arguments in FP64,
-// the rest (with copies r, b of rho, beta) in the working precision R.
+// Node values of one two-point flux argument: the log-mean arguments (in the mixed
+// form FP32 with the rest of the FP64 value) and the rest in the working precision R.
 template <typename R>
 struct NodeMT {
-    typename LogT<R>::type rho, beta, lnr, lnb;   // FP64 (dual in the adjoint)
-    R r, b, W, u[3], B[3];
+    LmV<R> rho, beta;
+    R W, u[3], B[3];
 };
 using NodeM = NodeMT<double>;
 
+// an FP64 value in R (the conversion off the FP64 pipe)
+template <typename R> __device__ __forceinline__ R in_w(double x);
+template <> __device__ __forceinline__ double in_w<double>(double x) { return x; }
+template <> __device__ __forceinline__ float in_w<float>(double x) { return d2f_int(x); }
+
+// the arrays of the flux arguments: FP64 node data, or its FP32 copies
+template <typename R> struct NodeIx;
+template <> struct NodeIx<double> {
+    enum { RHO = Q_RHO, BETA = Q_BETA, LNR = Q_LNR, LNB = Q_LNB, W = Q_W, U0 = Q_UX, U1 = Q_UY, U2 = QM_UZ,
+           B0 = QM_B1, B1 = QM_B2, B2 = QM_B3 };
+};
+template <> struct NodeIx<float> {
+    enum { RHO = QM32_R, BETA = QM32_B, LNR = QM32_LNR, LNB = QM32_LNB, W = QM32_W, U0 = QM32_U0, U1 = QM32_U1,
+           U2 = QM32_U2, B0 = QM32_B0, B1 = QM32_B1, B2 = QM32_B2 };
+};
+
+// (v: the arrays of R)
 template <typename R = double>
-__device__ __forceinline__ NodeMT<R> load_node_m(const double *__restrict__ q, long long P, long long c)
+__device__ __forceinline__ NodeMT<R> load_node_m(const R *__restrict__ v, long long P, long long c)
 {
-    NodeMT<R> v;
-    v.rho = q[Q_RHO * P + c];
-    v.beta = q[Q_BETA * P + c];
-    v.lnr = q[Q_LNR * P + c];
-    v.lnb = q[Q_LNB * P + c];
-    v.r = (R)v.rho;
-    v.b = (R)v.beta;
-    v.W = (R)q[Q_W * P + c];
-    v.u[0] = (R)q[Q_UX * P + c];
-    v.u[1] = (R)q[Q_UY * P + c];
-    v.u[2] = (R)q[QM_UZ * P + c];
-    v.B[0] = (R)q[QM_B1 * P + c];
-    v.B[1] = (R)q[QM_B2 * P + c];
-    v.B[2] = (R)q[QM_B3 * P + c];
-    return v;
+    using I = NodeIx<R>;
+    NodeMT<R> n;
+    n.rho.v = v[I::RHO * P + c];
+    n.rho.l = v[I::LNR * P + c];
+    n.beta.v = v[I::BETA * P + c];
+    n.beta.l = v[I::LNB * P + c];
+    if constexpr (std::is_same<R, float>::value) {
+        n.rho.lo = v[QM32_RLO * P + c];
+        n.beta.lo = v[QM32_BLO * P + c];
+    }
+    n.W = v[I::W * P + c];
+    n.u[0] = v[I::U0 * P + c];
+    n.u[1] = v[I::U1 * P + c];
+    n.u[2] = v[I::U2 * P + c];
+    n.B[0] = v[I::B0 * P + c];
+    n.B[1] = v[I::B1 * P + c];
+    n.B[2] = v[I::B2 * P + c];
+    return n;
 }
 
 // Curvilinear two-point EC flux (Sec. 3.1) of one node pair:
@@ -710,108 +891,91 @@ __device__ __forceinline__ NodeMT<R> load_node_m(const double *__restrict__ q, l
 // U~: the paper's U~^RMHD with R_1 summed over three components and its
 // magnetic term 1/2 {{W (b^k)^2}}; F~_j: coefficient matching with exact
 // product-rule expansions, including the -{{B_j}}[[Phi]] term.  Here
-// b = (B + (u.B) u)/W, b^0 = u.B, c = W b^0, v = u/W.
+// b = (B + (u.B) u)/W, b^0 = u.B, c = W b^0, v = u/W.  F~_j enters only as m.F~ and
+// is linear in its direction, so it is taken once along m (u_n = m.u, B_n = m.B): the
+// cost does not grow with NJ.
 template <int NJ, typename R>
 __device__ __forceinline__ void ec_pair_mhd(const NodeMT<R> &L, const NodeMT<R> &Rn, R gm1inv, double thr, R mt,
                                             const R m[3], R out[8])
 {
     R rln, irln, bln, ibln;
-    lmean<R, typename LogT<R>::type>(L.rho, Rn.rho, L.lnr, Rn.lnr, L.r, Rn.r, thr, rln, irln);
-    lmean<R, typename LogT<R>::type>(L.beta, Rn.beta, L.lnb, Rn.lnb, L.b, Rn.b, thr, bln, ibln);
+    logmean2<R>(L.rho, Rn.rho, thr, rln, irln);
+    logmean2<R>(L.beta, Rn.beta, thr, bln, ibln);
     const R half = (R)0.5;
-    R bL[3], bR[3], vL[3], vR[3];
-    // b^0 = W (v.B) = u.B
-    R b0L = L.u[0] * L.B[0] + L.u[1] * L.B[1] + L.u[2] * L.B[2];
-    R b0R = Rn.u[0] * Rn.B[0] + Rn.u[1] * Rn.B[1] + Rn.u[2] * Rn.B[2];
-    R iWL = rcp<R>(L.W), iWR = rcp<R>(Rn.W);
+    // per node: b^0, 1/W, b, b.b (spatial), u_n, B_n; sums over the two nodes
+    R b[3] = {(R)0, (R)0, (R)0}, bsq = (R)0, Wbsq = (R)0, c = (R)0, b0m = (R)0, Wb0 = (R)0, Sn = (R)0, vn = (R)0,
+      un = (R)0, Bn = (R)0;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        bL[k] = (L.B[k] + b0L * L.u[k]) * iWL;
-        bR[k] = (Rn.B[k] + b0R * Rn.u[k]) * iWR;
-        vL[k] = L.u[k] * iWL;
-        vR[k] = Rn.u[k] * iWR;
-    }
-    const R rho_m = half * (L.r + Rn.r), beta_m = half * (L.b + Rn.b), W_m = half * (L.W + Rn.W);
-    R u_m[3], b_m[3], bsq_m[3], Wbsq_m[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        u_m[k] = half * (L.u[k] + Rn.u[k]);
-        b_m[k] = half * (bL[k] + bR[k]);
-        bsq_m[k] = half * (bL[k] * bL[k] + bR[k] * bR[k]);
-        Wbsq_m[k] = half * (L.W * bL[k] * bL[k] + Rn.W * bR[k] * bR[k]);
-    }
-    const R c_m = half * (L.W * b0L + Rn.W * b0R);
-    const R Wb0sq_m = half * (L.W * b0L * b0L + Rn.W * b0R * b0R);
-    const R b0_m = half * (b0L + b0R);
-    const R usq = u_m[0] * u_m[0] + u_m[1] * u_m[1] + u_m[2] * u_m[2];
-    const R Lam = W_m * W_m - usq;
-    const R alpha0 = (R)1 + gm1inv * ibln;
-    const R iW_m = rcp<R>(W_m), ibeta_m = rcp<R>(beta_m), iLam = rcp<R>(Lam);
-    const R bsq_sum = bsq_m[0] + bsq_m[1] + bsq_m[2];
-    // U~
-    R Ut[8];
-    {
-        const R alpha1 = rho_m + half * beta_m * bsq_sum + half * beta_m * Wb0sq_m * iW_m;
-        const R U1 = rln * W_m;
-        R UB[3], Rk[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) UB[k] = (W_m * W_m * b_m[k] - c_m * u_m[k]) * iW_m;
-        R R1 = -alpha0 * U1 - half * Wb0sq_m;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) R1 += half * Wbsq_m[k] - b_m[k] * UB[k];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) Rk[k] = (alpha1 * u_m[k] - beta_m * c_m * b_m[k]) * iW_m;
-        const R U5 = (u_m[0] * Rk[0] + u_m[1] * Rk[1] + u_m[2] * Rk[2] - beta_m * R1) * W_m * ibeta_m * iLam;
-        Ut[0] = U1;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) Ut[1 + k] = u_m[k] * U5 * iW_m + Rk[k] * ibeta_m;
-        Ut[4] = U5;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) Ut[5 + k] = UB[k];
-    }
-#pragma unroll
-    for (int a = 0; a < 8; ++a) out[a] = mt * Ut[a];
-    // F~_j, j = 1..NJ
-#pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-        const R mj = m[j];
-        R ujbsq = (R)0;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) ujbsq += half * (L.u[j] * bL[k] * bL[k] + Rn.u[j] * bR[k] * bR[k]);
-        const R ujb0sq = half * (L.u[j] * b0L * b0L + Rn.u[j] * b0R * b0R);
-        const R vj_m = half * (vL[j] + vR[j]);
-        const R Bj_m = half * (L.B[j] + Rn.B[j]);
-        R r_beta = (R)0, r_u[3] = {(R)0, (R)0, (R)0}, r_b[3];
-        R cW = (R)0, cc = (R)0;
-        r_u[j] += rho_m;
-        r_beta += half * ujbsq;
-        r_u[j] += half * beta_m * bsq_sum;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) r_b[k] = beta_m * u_m[j] * b_m[k];
-        r_beta -= half * ujb0sq;
-        cc -= beta_m * vj_m * c_m * iW_m;
-        cW += beta_m * vj_m * Wb0sq_m * iW_m;        // both [[W]] terms of -(1/2)[[beta u_j (b^0)^2]]
-        r_u[j] -= half * beta_m * Wb0sq_m * iW_m;
-        r_beta -= Bj_m * b0_m;
-        cc -= Bj_m * beta_m * iW_m;
-        cW += Bj_m * beta_m * b0_m * iW_m;
+    for (int x = 0; x < 2; ++x) {
+        const NodeMT<R> &n = x == 0 ? L : Rn;
+        const R b0 = n.u[0] * n.B[0] + n.u[1] * n.B[1] + n.u[2] * n.B[2], iWx = qrcp<R>(n.W);
+        R bk[3], ux = m[0] * n.u[0], Bx = m[0] * n.B[0];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            r_u[k] += cW * u_m[k] * iW_m + cc * b_m[k];
-            r_b[k] += cc * u_m[k];
+            bk[k] = (n.B[k] + b0 * n.u[k]) * iWx;
+            b[k] += bk[k];
+            if (k > 0 && k < NJ) {
+                ux += m[k] * n.u[k];
+                Bx += m[k] * n.B[k];
+            }
         }
-        R F[8];
-        F[0] = rln * u_m[j];
+        const R bb = bk[0] * bk[0] + bk[1] * bk[1] + bk[2] * bk[2], W0 = n.W * b0;
+        bsq += bb;
+        Wbsq += n.W * bb;
+        c += W0;
+        b0m += b0;
+        Wb0 += W0 * b0;
+        Sn += ux * (bb - b0 * b0);
+        vn += ux * iWx;
+        un += ux;
+        Bn += Bx;
+    }
+    const R rm = half * (L.rho.v + Rn.rho.v), be = half * (L.beta.v + Rn.beta.v), W = half * (L.W + Rn.W);
+    R u[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) F[5 + k] = r_b[k] * ibeta_m;
-        R acc = alpha0 * F[0] - r_beta;
+    for (int k = 0; k < 3; ++k) {
+        u[k] = half * (L.u[k] + Rn.u[k]);
+        b[k] *= half;
+    }
+    const R hbe = half * be;
+    bsq *= half;
+    c *= half;
+    Wb0 *= half;
+    vn *= half;
+    un *= half;
+    Bn *= half;
+    const R Lam = W * W - (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]), al0 = (R)1 + gm1inv * ibln;
+    const R iW = qrcp<R>(W), ibe = qrcp<R>(be), iLam = qrcp<R>(Lam);
+    // U~ up to its solve for U5, times mt; F~ along m
+    const R Bb0 = half * Bn * b0m, h0 = rm + hbe * bsq, h1 = hbe * Wb0 * iW;
+    const R X1 = vn * Wb0 + Bb0, X2 = vn * c + Bn, bi = be * iW, cc = -bi * X2, cW = bi * iW * X1;
+    const R al1 = h0 + h1, hm = h0 - h1, rW = rln * W, ru_n = rln * un;
+    R R1 = half * (half * Wbsq - Wb0) - al0 * rW, T = (R)0, uru = (R)0;
+    R acc = al0 * ru_n - (half * half) * Sn + Bb0;
+    R UB[3], FB[3], G[3];
+    const R ciW = c * iW, a1 = al1 * iW, bec = bi * c, cb = cc * ibe;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) acc += u_m[k] * r_u[k] * ibeta_m + b_m[k] * F[5 + k];
-        F[4] = W_m * acc * iLam;
+    for (int k = 0; k < 3; ++k) {
+        UB[k] = W * b[k] - ciW * u[k];
+        R1 -= b[k] * UB[k];
+        const R Rk = a1 * u[k] - bec * b[k];
+        T += u[k] * Rk;
+        R ru = cW * u[k] + cc * b[k];
+        if (k < NJ) ru += m[k] * hm;
+        FB[k] = un * b[k] + cb * u[k];
+        uru += u[k] * ru;
+        acc += b[k] * FB[k];
+        G[k] = mt * Rk + ru;
+    }
+    T -= be * R1;
+    // the energy components of mt U~ + F~
+    const R E = W * iLam * (ibe * (mt * T + uru) + acc), Eu = E * iW;
+    out[0] = mt * rW + ru_n;
+    out[4] = E;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) F[1 + k] = r_u[k] * ibeta_m + u_m[k] * F[4] * iW_m;
-#pragma unroll
-        for (int a = 0; a < 8; ++a) out[a] += mj * F[a];
+    for (int k = 0; k < 3; ++k) {
+        out[1 + k] = G[k] * ibe + Eu * u[k];
+        out[5 + k] = mt * UB[k] + FB[k];
     }
 }
 
@@ -821,7 +985,8 @@ template <int P>
 __global__ void k_node_mhd(ProbArg pa, double gam, const double *__restrict__ cons, const double *__restrict__ J,
                            const double *__restrict__ x, const double *__restrict__ xdot,
                            const double *__restrict__ zg_in, double *__restrict__ zg_out, double *__restrict__ q,
-                           int *__restrict__ status, const double *__restrict__ inflow, int f32_logs)
+                           int *__restrict__ status, const double *__restrict__ inflow, int f32_logs,
+                           float *__restrict__ q32)
 {
     ProbDesc D;
     long long lb;
@@ -848,8 +1013,8 @@ __global__ void k_node_mhd(ProbArg pa, double gam, const double *__restrict__ co
         if (st) atomicAdd(status, 1);
         if (zg_out) zg_out[src] = Z;
     }
-    double W = 1.0 / sqrt(1.0 - (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]));
-    double beta = w[0] / w[4];
+    const double W = qrsq<double>(1.0 - (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]));
+    const double beta = w[0] * qrcp<double>(w[4]);
     q[Q_RHO * g.P + t] = w[0];
     q[Q_P * g.P + t] = w[4];
     q[Q_BETA * g.P + t] = beta;
@@ -860,11 +1025,33 @@ __global__ void k_node_mhd(ProbArg pa, double gam, const double *__restrict__ co
     // (f32_logs: the mixed form's scheme passes, where the logarithms enter
     // only FP32 arithmetic and the log mean's jump outside its near-equal
     // branch)
-    q[Q_LNR * g.P + t] = f32_logs ? f2d_int(logf(d2f_int(w[0]))) : log(w[0]);
-    q[Q_LNB * g.P + t] = f32_logs ? f2d_int(logf(d2f_int(beta))) : log(beta);
+    float lr32 = 0.0f, lb32 = 0.0f;
+    if (f32_logs) {
+        lr32 = logf(d2f_int(w[0]));
+        lb32 = logf(d2f_int(beta));
+    }
+    const double lr = f32_logs ? f2d_int(lr32) : log(w[0]), lb_ = f32_logs ? f2d_int(lb32) : log(beta);
+    q[Q_LNR * g.P + t] = lr;
+    q[Q_LNB * g.P + t] = lb_;
     q[QM_B1 * g.P + t] = w[5];
     q[QM_B2 * g.P + t] = w[6];
     q[QM_B3 * g.P + t] = w[7];
+    if (q32) {
+        const LmV<float> r = lmv_f32(w[0], d2f_int(w[0]), f32_logs ? lr32 : d2f_int(lr));
+        const LmV<float> b = lmv_f32(beta, d2f_int(beta), f32_logs ? lb32 : d2f_int(lb_));
+        q32[QM32_R * g.P + t] = r.v;
+        q32[QM32_RLO * g.P + t] = r.lo;
+        q32[QM32_LNR * g.P + t] = r.l;
+        q32[QM32_B * g.P + t] = b.v;
+        q32[QM32_BLO * g.P + t] = b.lo;
+        q32[QM32_LNB * g.P + t] = b.l;
+        q32[QM32_W * g.P + t] = d2f_int(W);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            q32[(QM32_U0 + k) * g.P + t] = d2f_int(W * w[1 + k]);
+            q32[(QM32_B0 + k) * g.P + t] = d2f_int(w[5 + k]);
+        }
+    }
     double dxi_x = 0.0, dxi_y = 0.0, deta_x = 0.0, deta_y = 0.0;
 #pragma unroll
     for (int n = 1; n <= P; ++n) {
@@ -889,15 +1076,15 @@ __global__ void k_node_mhd(ProbArg pa, double gam, const double *__restrict__ co
 // entropy variables of a node from its stored values: V = (Gamma/(Gamma-1) +
 // ln rho + ln beta/(Gamma-1) + beta, beta u, -beta W, beta b)
 template <typename R>
-__device__ __forceinline__ void node_V_mhd(const double *__restrict__ q, long long P, long long c, R c1g, R ig,
-                                           R V[8])
+__device__ __forceinline__ void node_V_mhd(const R *__restrict__ v, long long P, long long c, R c1g, R ig, R V[8])
 {
-    R beta = (R)q[Q_BETA * P + c], W = (R)q[Q_W * P + c];
-    R u0 = (R)q[Q_UX * P + c], u1 = (R)q[Q_UY * P + c], u2 = (R)q[QM_UZ * P + c];
-    R B0 = (R)q[QM_B1 * P + c], B1 = (R)q[QM_B2 * P + c], B2 = (R)q[QM_B3 * P + c];
-    R b0 = u0 * B0 + u1 * B1 + u2 * B2;
-    R bW = beta * rcp<R>(W);
-    V[0] = c1g + (R)q[Q_LNR * P + c] + ig * (R)q[Q_LNB * P + c] + beta;
+    using I = NodeIx<R>;
+    const R beta = v[I::BETA * P + c], W = v[I::W * P + c];
+    const R u0 = v[I::U0 * P + c], u1 = v[I::U1 * P + c], u2 = v[I::U2 * P + c];
+    const R B0 = v[I::B0 * P + c], B1 = v[I::B1 * P + c], B2 = v[I::B2 * P + c];
+    const R b0 = u0 * B0 + u1 * B1 + u2 * B2;
+    const R bW = beta * qrcp<R>(W);
+    V[0] = c1g + v[I::LNR * P + c] + ig * v[I::LNB * P + c] + beta;
     V[1] = beta * u0;
     V[2] = beta * u1;
     V[3] = beta * u2;
@@ -907,6 +1094,13 @@ __device__ __forceinline__ void node_V_mhd(const double *__restrict__ q, long lo
     V[7] = bW * (B2 + b0 * u2);
 }
 
+// Bound: FP64 the FP64 pipe (3,150 instructions per interface at p = 2, w = 5, 19 cycles of
+// an SM each per warp: 1.57 ms a sweep of 512^2, all of it), FP32 instruction issue (50%, 20
+// warps an SM; 128 registers take 3.63 ms for two mixed 512^2 steps, 168 3.85 and 96
+// 3.84).  Measured with the pair flux along the metric vector, jumps from differences,
+// the scalar form of the waves, turned pairs and the FP32 node copies: two 512^2 rotor
+// steps 40.0 -> 23.2 ms, mixed 6.1 -> 3.6 ms; 64^3 blast step 32.9 -> 21.0 ms; a 160^2 p = 3
+// step without dissipation 1.42 -> 0.95 ms.
 // ES interface flux (eq. ESFlux_HO) between node L in [-1, n_dir - 1] and
 // L + 1: the 2p-th order EC sum of two-point fluxes (eq. ECFlux_O2p, summed
 // directly), the metric flux (eq. MetricsFlux_O2p), the magnetic flux B~
@@ -914,8 +1108,8 @@ __device__ __forceinline__ void node_V_mhd(const double *__restrict__ q, long lo
 // variables at the interface state rho = {{rho}}^ln, u = {{u}},
 // p = {{rho}}/{{beta}}, B = {{B}}.
 template <typename R, int P, int WW>
-__global__ void __launch_bounds__(128) k_iface_mhd(ProbArg pa, Phys ph, const double *__restrict__ q,
-                                                   R *__restrict__ iflux, int dir)
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 4 : 1) k_iface_mhd(ProbArg pa, Phys ph, const double *__restrict__ q,
+                                                   const R *__restrict__ qr, R *__restrict__ iflux, int dir)
 {
     ProbDesc D;
     long long lb;
@@ -946,122 +1140,80 @@ __global__ void __launch_bounds__(128) k_iface_mhd(ProbArg pa, Phys ph, const do
 #pragma unroll (sizeof(R) == 4 ? 1 : P)
         for (int s = 0; s < n; ++s) {
             const long long cl = c0 - s * sd, cr = cl + n * sd;
-            NodeMT<R> l = load_node_m<R>(q, g.P, cl), r = load_node_m<R>(q, g.P, cr);
+            NodeMT<R> l = load_node_m<R>(qr, g.P, cl), r = load_node_m<R>(qr, g.P, cr);
             R out[8];
-            const R mm[3] = {(R)(0.5 * (Mx[cl] + Mx[cr])), (R)(0.5 * (My[cl] + My[cr])), (R)0};
-            ec_pair_mhd<2, R>(l, r, gm1inv, ph.ln_thr, (R)(0.5 * (Mt[cl] + Mt[cr])), mm, out);
+            const double mx = Mx[cl] + Mx[cr], my = My[cl] + My[cr], mt = Mt[cl] + Mt[cr];
+            const R mm[3] = {in_w<R>(0.5 * mx), in_w<R>(0.5 * my), (R)0};
+            ec_pair_mhd<2, R>(l, r, gm1inv, ph.ln_thr, in_w<R>(0.5 * mt), mm, out);
 #pragma unroll
             for (int a = 0; a < 8; ++a) Fs[a] += out[a];
-            Fts += 0.5 * (Mt[cl] + Mt[cr]);
-            Bts += 0.25 * (Mx[cl] + Mx[cr]) * (B1[cl] + B1[cr]) + 0.25 * (My[cl] + My[cr]) * (B2[cl] + B2[cr]);
+            Fts += mt;
+            Bts += mx * (B1[cl] + B1[cr]) + my * (B2[cl] + B2[cr]);
         }
         const R an = (R)ph.alpha[n - 1];
 #pragma unroll
         for (int a = 0; a < 8; ++a) F[a] += an * Fs[a];
-        Ft += ph.alpha[n - 1] * Fts;
-        Bt += ph.alpha[n - 1] * Bts;
+        Ft += 0.5 * ph.alpha[n - 1] * Fts;
+        Bt += 0.25 * ph.alpha[n - 1] * Bts;
     }
 
-    if (WW > 0) {
-        constexpr int NS = WW + 1, OFF = (WW - 1) / 2;
+    if constexpr (WW > 0) {
+        constexpr int OFF = (WW - 1) / 2;
         const R half = (R)0.5;
         const long long c1 = c0 + sd;
-        const R nvx = (R)(0.5 * (Mx[c0] + Mx[c1])), nvy = (R)(0.5 * (My[c0] + My[c1]));
-        const R jt = (R)(0.5 * (Mt[c0] + Mt[c1]));
-        const R Lk = sq_rt<R>(nvx * nvx + nvy * nvy);
-        const R iLk = rcp<R>(Lk), nx = nvx * iLk, ny = nvy * iLk;
-        // interface state
-        R wm[8], wrot[8];
+        const R nvx = in_w<R>(0.5 * (Mx[c0] + Mx[c1])), nvy = in_w<R>(0.5 * (My[c0] + My[c1]));
+        const R jt = in_w<R>(0.5 * (Mt[c0] + Mt[c1]));
+        const R n2 = nvx * nvx + nvy * nvy, iLk = qrsq<R>(n2), Lk = n2 * iLk, nx = nvx * iLk, ny = nvy * iLk;
+        // interface state, rotated
+        R rho, p, ip, us[3], Bs[3];
         {
-            R rho, irho;
-            lmean<R, double>(q[Q_RHO * g.P + c0], q[Q_RHO * g.P + c1], q[Q_LNR * g.P + c0], q[Q_LNR * g.P + c1],
-                             (R)q[Q_RHO * g.P + c0], (R)q[Q_RHO * g.P + c1], ph.ln_thr, rho, irho);
-            R um[3] = {half * ((R)q[Q_UX * g.P + c0] + (R)q[Q_UX * g.P + c1]),
-                       half * ((R)q[Q_UY * g.P + c0] + (R)q[Q_UY * g.P + c1]),
-                       half * ((R)q[QM_UZ * g.P + c0] + (R)q[QM_UZ * g.P + c1])};
-            R W2 = (R)1 + um[0] * um[0] + um[1] * um[1] + um[2] * um[2];
-            R W = sq_rt<R>(W2);
-            wm[0] = rho;
-            const R iW = rcp<R>(W);
-            for (int k = 0; k < 3; ++k) wm[1 + k] = um[k] * iW;
-            wm[4] = ((R)q[Q_RHO * g.P + c0] + (R)q[Q_RHO * g.P + c1]) *
-                    rcp<R>((R)q[Q_BETA * g.P + c0] + (R)q[Q_BETA * g.P + c1]);
-            wm[5] = half * ((R)B1[c0] + (R)B1[c1]);
-            wm[6] = half * ((R)B2[c0] + (R)B2[c1]);
-            wm[7] = half * ((R)q[QM_B3 * g.P + c0] + (R)q[QM_B3 * g.P + c1]);
-            wrot[0] = wm[0];
-            wrot[1] = nx * wm[1] + ny * wm[2];
-            wrot[2] = -ny * wm[1] + nx * wm[2];
-            wrot[3] = wm[3];
-            wrot[4] = wm[4];
-            wrot[5] = nx * wm[5] + ny * wm[6];
-            wrot[6] = -ny * wm[5] + nx * wm[6];
-            wrot[7] = wm[7];
+            const NodeMT<R> l = load_node_m<R>(qr, g.P, c0), r = load_node_m<R>(qr, g.P, c1);
+            R irho;
+            logmean2<R>(l.rho, r.rho, ph.ln_thr, rho, irho);
+            const R sr = l.rho.v + r.rho.v, sb = l.beta.v + r.beta.v;
+            p = sr * qrcp<R>(sb);
+            ip = sb * qrcp<R>(sr);
+            R um[3], Bm[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                um[k] = half * (l.u[k] + r.u[k]);
+                Bm[k] = half * (l.B[k] + r.B[k]);
+            }
+            us[0] = nx * um[0] + ny * um[1];
+            us[1] = nx * um[1] - ny * um[0];
+            us[2] = um[2];
+            Bs[0] = nx * Bm[0] + ny * Bm[1];
+            Bs[1] = nx * Bm[1] - ny * Bm[0];
+            Bs[2] = Bm[2];
         }
-        R lam[8], Rm[8][8];
-        eigen_mhd<R>(ph.gamma, wrot, lam, Rm);
-        R lhat = (R)0;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) lhat = vmax(lhat, fab<R>(jt + Lk * lam[m]));
         const R ig = gm1inv, c1g = (R)ph.gamma * gm1inv;
-        R Vt[NS][8], scale[8];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) scale[m] = (R)0;
-        for (int k = 0; k < NS; ++k) {
-            R V[8], TV[8];
-            node_V_mhd<R>(q, g.P, c0 + (k - OFF) * sd, c1g, ig, V);
+        R d[8];
+        es_dissipation_mhd<R, WW>(ph, rho, p, ip, us, Bs, Lk, jt, [&](int k, R TV[8]) {
+            R V[8];
+            node_V_mhd<R>(qr, g.P, c0 + (k - OFF) * sd, c1g, ig, V);
             TV[0] = V[0];
             TV[1] = nx * V[1] + ny * V[2];
-            TV[2] = -ny * V[1] + nx * V[2];
+            TV[2] = nx * V[2] - ny * V[1];
             TV[3] = V[3];
             TV[4] = V[4];
             TV[5] = nx * V[5] + ny * V[6];
-            TV[6] = -ny * V[5] + nx * V[6];
+            TV[6] = nx * V[6] - ny * V[5];
             TV[7] = V[7];
-            for (int m = 0; m < 8; ++m) {
-                R acc = (R)0;
-                for (int a = 0; a < 8; ++a) {
-                    R t = Rm[a][m] * TV[a];
-                    acc += t;
-                    if (k == OFF || k == OFF + 1) scale[m] += fab<R>(t);
-                }
-                Vt[k][m] = acc;
-            }
-        }
-        R z[8];
-        const R eps = (R)ph.eps, sign_tol = (R)ph.sign_tol;
-        each_index<R>(8, [&](int m) {
-            R vminus, vplus;
-            if (WW == 5)
-                weno5_lr<R>(Vt[0][m], Vt[1][m], Vt[2][m], Vt[3][m], Vt[4][m], Vt[5][m], eps, vminus, vplus);
-            else
-                weno3_lr<R>(Vt[0][m], Vt[1][m], Vt[2][m], Vt[3][m], eps, vminus, vplus);
-            R jw = vplus - vminus;
-            R jump = Vt[OFF + 1][m] - Vt[OFF][m];
-            int sj = le(fab<R>(jump), sign_tol * scale[m]) ? 0 : sgn_d(jump);
-            z[m] = (sgn_d(jw) == sj) ? jw : (R)0;
-        });
-        R d[8];
-        for (int a = 0; a < 8; ++a) {
-            R acc = (R)0;
-            for (int m = 0; m < 8; ++m) acc += Rm[a][m] * z[m];
-            d[a] = acc;
-        }
-        const R hl = half * lhat;
-        F[0] -= hl * d[0];
-        F[1] -= hl * (nx * d[1] - ny * d[2]);
-        F[2] -= hl * (ny * d[1] + nx * d[2]);
-        F[3] -= hl * d[3];
-        F[4] -= hl * d[4];
-        F[5] -= hl * (nx * d[5] - ny * d[6]);
-        F[6] -= hl * (ny * d[5] + nx * d[6]);
-        F[7] -= hl * d[7];
+        }, d);
+        F[0] -= d[0];
+        F[1] -= nx * d[1] - ny * d[2];
+        F[2] -= ny * d[1] + nx * d[2];
+        F[3] -= d[3];
+        F[4] -= d[4];
+        F[5] -= nx * d[5] - ny * d[6];
+        F[6] -= ny * d[5] + nx * d[6];
+        F[7] -= d[7];
     }
     R *out = iflux + (long long)(dir * NFM) * g.P + c0;
 #pragma unroll
     for (int a = 0; a < 8; ++a) out[a * g.P] = F[a];
-    out[8 * g.P] = (R)Ft;
-    out[9 * g.P] = (R)Bt;
+    out[8 * g.P] = in_w<R>(Ft);
+    out[9 * g.P] = in_w<R>(Bt);
 }
 
 // initial J and cons = J U(prim)
@@ -1159,25 +1311,26 @@ __global__ void k_update_mhd(ProbArg pa, const double *__restrict__ q, const R *
 
 
 template <typename R, int P>
-static void launch_iface_mhd_p(const LaunchDom &L, const Phys &ph, const double *q, R *iflux, int dir, cudaStream_t st)
+static void launch_iface_mhd_p(const LaunchDom &L, const Phys &ph, const double *q, const R *qr, R *iflux, int dir,
+                               cudaStream_t st)
 {
     switch (ph.w) {
-    case 0: k_iface_mhd<R, P, 0><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, iflux, dir); break;
-    case 3: k_iface_mhd<R, P, 3><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, iflux, dir); break;
-    default: k_iface_mhd<R, P, 5><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, iflux, dir); break;
+    case 0: k_iface_mhd<R, P, 0><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, qr, iflux, dir); break;
+    case 3: k_iface_mhd<R, P, 3><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, qr, iflux, dir); break;
+    default: k_iface_mhd<R, P, 5><<<L.nblk, L.bs, 0, st>>>(L.pa, ph, q, qr, iflux, dir); break;
     }
 }
 
 // interface fluxes of one sweep direction in the working precision R
 template <typename R>
-static void launch_iface_mhd_t(const LaunchDom &L, const Phys &ph, const double *q, void *iflux, int dir,
+static void launch_iface_mhd_t(const LaunchDom &L, const Phys &ph, const double *q, const R *qr, void *iflux, int dir,
                                cudaStream_t st)
 {
     R *fl = (R *)iflux;
     switch (ph.p) {
-    case 1: launch_iface_mhd_p<R, 1>(L, ph, q, fl, dir, st); break;
-    case 2: launch_iface_mhd_p<R, 2>(L, ph, q, fl, dir, st); break;
-    default: launch_iface_mhd_p<R, 3>(L, ph, q, fl, dir, st); break;
+    case 1: launch_iface_mhd_p<R, 1>(L, ph, q, qr, fl, dir, st); break;
+    case 2: launch_iface_mhd_p<R, 2>(L, ph, q, qr, fl, dir, st); break;
+    default: launch_iface_mhd_p<R, 3>(L, ph, q, qr, fl, dir, st); break;
     }
 }
 

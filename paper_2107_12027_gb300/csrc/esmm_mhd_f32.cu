@@ -5,10 +5,10 @@
 
 namespace esmm {
 
-void launch_iface_mhd_f32(const LaunchDom &L, const Phys &ph, const double *q, void *iflux, int dir,
-                          cudaStream_t st)
+void launch_iface_mhd_f32(const LaunchDom &L, const Phys &ph, const double *q, const float *q32, void *iflux,
+                          int dir, cudaStream_t st)
 {
-    launch_iface_mhd_t<float>(L, ph, q, iflux, dir, st);
+    launch_iface_mhd_t<float>(L, ph, q, q32, iflux, dir, st);
 }
 
 void launch_update_mhd_f32(const LaunchDom &L, const double *q, const void *fl, double *dcons, double *dJ,

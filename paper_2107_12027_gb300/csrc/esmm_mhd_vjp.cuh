@@ -35,8 +35,8 @@ __device__ __forceinline__ void mhd_pair_vjp(const NodeM &L, const NodeM &Rn, do
                                              double gR[NQN])
 {
     double rln, irln, bln, ibln;
-    logmean<double, double>(L.rho, Rn.rho, L.lnr, Rn.lnr, thr, rln, irln);
-    logmean<double, double>(L.beta, Rn.beta, L.lnb, Rn.lnb, thr, bln, ibln);
+    logmean<double, double>(L.rho.v, Rn.rho.v, L.rho.l, Rn.rho.l, thr, rln, irln);
+    logmean<double, double>(L.beta.v, Rn.beta.v, L.beta.l, Rn.beta.l, thr, bln, ibln);
     double bX[2][3], b0X[2], iWX[2], bbX[2], unX[2], BnX[2];
     const NodeM *N[2] = {&L, &Rn};
 #pragma unroll
@@ -49,7 +49,7 @@ __device__ __forceinline__ void mhd_pair_vjp(const NodeM &L, const NodeM &Rn, do
         unX[x] = m[0] * n.u[0] + m[1] * n.u[1] + m[2] * n.u[2];
         BnX[x] = m[0] * n.B[0] + m[1] * n.B[1] + m[2] * n.B[2];
     }
-    const double rm = 0.5 * (L.r + Rn.r), be = 0.5 * (L.b + Rn.b), W = 0.5 * (L.W + Rn.W);
+    const double rm = 0.5 * (L.rho.v + Rn.rho.v), be = 0.5 * (L.beta.v + Rn.beta.v), W = 0.5 * (L.W + Rn.W);
     double u[3], b[3];
     for (int k = 0; k < 3; ++k) {
         u[k] = 0.5 * (L.u[k] + Rn.u[k]);
@@ -208,8 +208,8 @@ __device__ __forceinline__ void mhd_pair_vjp(const NodeM &L, const NodeM &Rn, do
         g[A_LNR] = 0.0;
         g[A_LNB] = 0.0;
     }
-    logmean_vjp(L.rho, Rn.rho, L.lnr, Rn.lnr, thr, grln, gL[A_RHO], gR[A_RHO], gL[A_LNR], gR[A_LNR]);
-    logmean_vjp(L.beta, Rn.beta, L.lnb, Rn.lnb, thr, -ga0 * gm1inv * ibln * ibln, gL[A_BETA], gR[A_BETA], gL[A_LNB],
+    logmean_vjp(L.rho.v, Rn.rho.v, L.rho.l, Rn.rho.l, thr, grln, gL[A_RHO], gR[A_RHO], gL[A_LNR], gR[A_LNR]);
+    logmean_vjp(L.beta.v, Rn.beta.v, L.beta.l, Rn.beta.l, thr, -ga0 * gm1inv * ibln * ibln, gL[A_BETA], gR[A_BETA], gL[A_LNB],
                 gR[A_LNB]);
 }
 
@@ -333,7 +333,7 @@ static __device__ __noinline__ void mhd_clusters(double gam, const double w[8], 
     int start = 0;
     while (start < 6) {
         int end = start + 1;
-        while (end < 6 && lam[2 + end] - lam[1 + end] < MHD_CLUSTER_TOL) ++end;
+        while (end < 6 && mhd_close<double>(lam[1 + end], lam[2 + end])) ++end;
         const int k = end - start;
         for (int m = start; m < end; ++m) {
             c.from[m] = start;
@@ -445,7 +445,7 @@ __device__ __noinline__ void mhd_diss_vjp(const Phys &ph, const double wrot[8], 
     lam[0] = lam[1] = s.v1;
     mhd_six<double>(s, six, lam + 2);
     bool cluster = false;
-    for (int m = 0; m < 5; ++m) cluster = cluster || lam[3 + m] - lam[2 + m] < MHD_CLUSTER_TOL;
+    for (int m = 0; m < 5; ++m) cluster = cluster || mhd_close<double>(lam[2 + m], lam[3 + m]);
     // the waves: R (dU), X (dV), A (dw), one row per wave
     double R[8][8], X[8][8], A[8][8], S[6][6];
     const double ir = __drcp_rn(s.rho);
@@ -483,7 +483,7 @@ __device__ __noinline__ void mhd_diss_vjp(const Phys &ph, const double wrot[8], 
 #pragma unroll 1
     for (int m = 0; m < 6; ++m) {
         MhdWave<double> q;
-        mhd_six_wave<double>(s, six, m, q);
+        mhd_six_wave<double, true>(s, six, gg, m, q, R[2 + m]);
         mhd_wave_dU<double>(s, gg, q, R[2 + m]);
         const double db = (q.rho - s.beta * q.p) * s.ip;
         double *x = X[2 + m], *a = A[2 + m];

@@ -22,13 +22,13 @@
 //
 // Bound: the FP64 pipe.  The same system by a 6 x 6 Gram matrix, Cholesky
 // factor and cyclic Jacobi takes ~7,000 FP64 instructions per interface, this
-// ~1,000; the roots start from FP32 iterations, which cost next to nothing
+// ~1,000 (a wave ~140); the roots start from FP32 iterations, which cost next to nothing
 // beside the FP64 pipe, and take two FP64 Newton steps each.  Measured (GB300,
 // 2070 MHz, a perturbed rotor whose speeds are distinct): the 512^2 FP64 step went
 // from 51.8 to 20.5 ms, the mixed one from 5.1 to 3.1 ms, a 64^3 blast step from
-// 88.3 to 33.2 ms.  Against extended precision the vectors are ~8 times closer in
-// the median than the Gram form's (1.2e-15 against 8.0e-15 of a column in FP64),
-// 50 times in FP32's worst percent.
+// 88.3 to 33.2 ms.  Against extended precision the vectors are ~4 times closer in
+// the median than the Gram form's (2.2e-15 against 8.0e-15 of a column in FP64),
+// 40 times in FP32's worst percent.
 #pragma once
 
 namespace esmm {
@@ -43,28 +43,54 @@ struct MhdBase {
     R W, iW, v1, u[4], b[4], b2, rh, e, gp, beta, ip, rho, B1;
 };
 
+// ... from the spatial 4-velocity us and W
+template <typename R>
+__device__ __forceinline__ void mhd_base_u(R gam, R gg, R rho, R p, R ip, R W, R iW, const R us[3], const R B[3],
+                                           MhdBase<R> &s)
+{
+    s.W = W;
+    s.iW = iW;
+    s.v1 = us[0] * iW;
+    s.rho = rho;
+    s.B1 = B[0];
+    s.u[0] = W;
+    s.b[0] = us[0] * B[0] + us[1] * B[1] + us[2] * B[2];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        s.u[1 + k] = us[k];
+        s.b[1 + k] = (B[k] + s.b[0] * us[k]) * iW;
+    }
+    s.b2 = (B[0] * B[0] + B[1] * B[1] + B[2] * B[2] + s.b[0] * s.b[0]) * (iW * iW);
+    s.gp = gam * p;
+    s.rh = rho + gg * p;
+    s.e = s.rh + s.b2;
+    s.ip = ip;
+    s.beta = rho * ip;
+}
+
+// ... from the primitives w (rotated frame)
 template <typename R>
 __device__ __forceinline__ void mhd_base(R gam, R gg, const R w[8], MhdBase<R> &s)
 {
-    const R iW2 = (R)1 - (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
-    s.W = rsq<R>(iW2);
-    s.iW = iW2 * s.W;
+    const R iW2 = (R)1 - (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]), W = rsq<R>(iW2);
+    const R us[3] = {W * w[1], W * w[2], W * w[3]};
+    mhd_base_u<R>(gam, gg, w[0], w[4], rcp<R>(w[4]), W, iW2 * W, us, w + 5, s);
     s.v1 = w[1];
-    s.rho = w[0];
-    s.B1 = w[5];
-    s.u[0] = s.W;
-    s.u[1] = s.W * w[1];
-    s.u[2] = s.W * w[2];
-    s.u[3] = s.W * w[3];
-    s.b[0] = s.u[1] * w[5] + s.u[2] * w[6] + s.u[3] * w[7];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) s.b[1 + k] = (w[5 + k] + s.b[0] * s.u[1 + k]) * s.iW;
-    s.b2 = (w[5] * w[5] + w[6] * w[6] + w[7] * w[7] + s.b[0] * s.b[0]) * iW2;
-    s.gp = gam * w[4];
-    s.rh = w[0] + gg * w[4];
-    s.e = s.rh + s.b2;
-    s.ip = rcp<R>(w[4]);
-    s.beta = w[0] * s.ip;
+}
+
+// the closed form holds (its FP32 root estimates stay in range)
+template <typename R>
+__device__ __forceinline__ bool mhd_in_range(const MhdBase<R> &s)
+{
+    const float lim = sizeof(R) == 4 ? 1.0e-12f : 1.0e-25f;
+    return to_f32(s.gp) > lim && to_f32(s.e) < 1.0f / lim;
+}
+
+// two waves of one cluster: their speeds closer than MHD_CLUSTER_TOL
+template <typename R>
+__device__ __forceinline__ bool mhd_close(R lam0, R lam1)
+{
+    return to_f32(lam1 - lam0) < (float)MHD_CLUSTER_TOL;
 }
 
 // f(t) of the magnetosonic speeds on the side sg = +-1 (a = sg t, t >= 0),
@@ -119,7 +145,25 @@ __device__ __forceinline__ void mhd_roots32(float cA, float cB, float c1, float 
     tslow = t;
 }
 
-// Newton in R from the FP32 estimate t, kept in [lo, hi].  The step divides
+template <typename R> __device__ __forceinline__ bool is_neg(R x) { return x < (R)0; }
+template <typename R> __device__ __forceinline__ bool is_zero(R x) { return x == (R)0; }
+template <> __device__ __forceinline__ bool is_neg<double>(double x) { return (conv_bits64(x) >> 63) != 0; }
+template <> __device__ __forceinline__ bool is_zero<double>(double x) { return (conv_bits64(x) << 1) == 0; }
+
+// the smaller and larger of two numbers, b >= 0: in FP64 by their bits (non-negative
+// numbers order like them and a negative one lies below; FP64 compares cost FP64-pipe slots)
+__device__ __forceinline__ float lesser_nn(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ float larger_nn(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double lesser_nn(double a, double b)
+{
+    return (long long)conv_bits64(a) < (long long)conv_bits64(b) ? a : b;
+}
+__device__ __forceinline__ double larger_nn(double a, double b)
+{
+    return (long long)conv_bits64(a) > (long long)conv_bits64(b) ? a : b;
+}
+
+// Newton in R from the FP32 estimate t, kept in [lo, hi] (0 <= lo).  The step divides
 // through an FP32 reciprocal (a relative slope error contracts the error by
 // that much per step); a step below 1e-9 t leaves an error under rounding.
 template <typename R>
@@ -131,13 +175,10 @@ __device__ __forceinline__ R mhd_polish(R cA, R cB, R c1, R c0s, R v1, R iWs, R 
         R f, df;
         mhd_quartic<R>(cA, cB, c1, c0s, v1, iWs, t, f, df);
         const R dt = f * of_f32<R>(__frcp_rn(to_f32(df)));
-        R tn = t - dt;
-        tn = tn < lo ? lo : (tn > hi ? hi : tn);   // (a NaN step, f = f' = 0, ends the loop below)
-        if (!(fab<R>(dt) > (sizeof(R) == 4 ? (R)1.0e-4 : (R)1.0e-9) * t)) {
-            if (dt == dt) t = tn;
-            break;
-        }
-        t = tn;
+        const float d32 = fabsf(to_f32(dt));
+        const bool done = !(d32 > (sizeof(R) == 4 ? 1.0e-4f : 1.0e-9f) * to_f32(t));
+        if (d32 == d32) t = larger_nn(lesser_nn(t - dt, hi), lo);   // (a NaN step, f = f' = 0, ends the loop)
+        if (done) break;
     }
     return t;
 }
@@ -191,17 +232,34 @@ __device__ __noinline__ void mhd_near_triple(const MhdBase<R> &s, R sqe, R sg, R
     }
 }
 
+// coefficients of both sides
+template <typename R>
+struct MhdCoef {
+    R sqe, cA, cB, c1, c0, We;
+};
+template <typename R>
+__device__ __forceinline__ void mhd_coef(const MhdBase<R> &s, MhdCoef<R> &k)
+{
+    const R q = s.rh * qrcp<R>(s.gp);
+    k.sqe = s.e * qrsq<R>(s.e);
+    k.cA = s.rh * (q - (R)1);
+    k.cB = s.rh + s.b2 * q;
+    k.c1 = s.B1 * s.iW;
+    k.c0 = s.b[0] * s.iW;
+    k.We = s.W * k.sqe;
+}
+
 // the Alfven and magnetosonic |a| of the side sg
 template <typename R>
-__device__ __forceinline__ void mhd_side(const MhdBase<R> &s, R sqe, int sg, bool want_slow, R &tA, R &tslow, R &tfast)
+__device__ __forceinline__ void mhd_side(const MhdBase<R> &s, const MhdCoef<R> &kc, int sg, bool want_slow, R &tA, R &tslow,
+                                         R &tfast)
 {
-    const R sgr = (R)sg;
-    const R c0s = sgr * s.b[0] * s.iW, iWs = sgr * s.iW, c1 = s.B1 * s.iW;
-    const R igp = rcp<R>(s.gp);
-    const R cB = s.rh + s.rh * s.b2 * igp, cA = s.rh * (s.rh * igp - (R)1);
+    const R sgr = (R)sg, sqe = kc.sqe, cA = kc.cA, cB = kc.cB, c1 = kc.c1;
+    const R c0s = sgr * kc.c0, iWs = sgr * s.iW;
     const R tmax = s.W * ((R)1 + sgr * s.v1);
-    tA = fab<R>(s.B1) * rcp<R>(s.W * sqe - (s.B1 < (R)0 ? -sgr : sgr) * s.b[0]);
-    if (tA < (R)(sizeof(R) == 4 ? 1.0e-18 : 1.0e-100)) tA = (R)0;
+    const bool neg = is_neg(s.B1);
+    tA = fab<R>(s.B1) * qrcp<R>(kc.We - (neg ? -sgr : sgr) * s.b[0]);
+    if (to_f32(tA) < (sizeof(R) == 4 ? 1.0e-18f : 1.0e-30f)) tA = (R)0;   // (the speed v_1 at rounding)
     float fs = 0.0f, ff;
     const float irh = __frcp_rn(to_f32(s.rh)), qrh = sqrtf(irh);
     mhd_roots32(to_f32(cA) * irh, to_f32(cB) * irh, to_f32(c1) * qrh, to_f32(c0s) * qrh, to_f32(s.v1), to_f32(iWs),
@@ -217,38 +275,21 @@ __device__ __forceinline__ void mhd_side(const MhdBase<R> &s, R sqe, int sg, boo
     tfast = of_f32<R>(ff);
     if (!near) tfast = mhd_polish<R>(cA, cB, c1, c0s, s.v1, iWs, tfast, tA, tmax);
     tslow = (R)0;
-    if (want_slow && tA > (R)0) {
-        // an FP32 estimate that underflowed: the linear root in R
-        R t0 = of_f32<R>(fs);
-        if (!(fs > 1.0e-12f))
-            t0 = fab<R>(c1) * rcp<R>(sq_rt<R>(cB) - (s.B1 < (R)0 ? -c0s : c0s));
-        tslow = fs > 1.0e-12f ? mhd_polish<R>(cA, cB, c1, c0s, s.v1, iWs, t0, (R)0, tA) : (t0 < tA ? t0 : tA);
+    if (want_slow && !is_zero(tA)) {
+        if (fs > 1.0e-12f) {
+            tslow = mhd_polish<R>(cA, cB, c1, c0s, s.v1, iWs, of_f32<R>(fs), (R)0, tA);
+        } else {   // an FP32 estimate that underflowed: the linear root in R
+            tslow = lesser_nn(fab<R>(c1) * rcp<R>(sq_rt<R>(cB) - (neg ? -c0s : c0s)), tA);
+        }
     }
     if (near) mhd_near_triple<R>(s, sqe, sgr, tA, want_slow, tslow, tfast);
 }
 
-// One wave: perturbations (d rho, du, db, dp), scaled to <., .> = 1 by mhd_scale
+// One wave: perturbations (d rho, du, db, dp), scaled to <., .> = 1
 template <typename R>
 struct MhdWave {
     R rho, p, u[4], b[4];
 };
-
-// scale to unit X^0 (s = 0 or du = 0 waves: the general form with the entropy part S2 given)
-template <typename R>
-__device__ __forceinline__ void mhd_scale(const MhdBase<R> &s, MhdWave<R> &q)
-{
-    const R P = q.p + mdot<R>(s.b, q.b);
-    const R n2 = s.beta * (s.W * (q.p * q.p * rcp<R>(s.gp) + s.e * mdot<R>(q.u, q.u) + mdot<R>(q.b, q.b)) +
-                           (R)2 * (q.u[0] * P - s.b[0] * mdot<R>(q.b, q.u)));
-    const R sc = rsq<R>(n2);
-    q.p *= sc;
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        q.u[m] *= sc;
-        q.b[m] *= sc;
-    }
-    q.rho = q.p * s.rho * rcp<R>(s.gp);   // adiabatic
-}
 
 // dU of a wave: (D, m, E, B)
 template <typename R>
@@ -265,131 +306,199 @@ __device__ __forceinline__ void mhd_wave_dU(const MhdBase<R> &s, R gg, const Mhd
     for (int k = 1; k < 4; ++k) dU[4 + k] = q.u[0] * s.b[k] + s.W * q.b[k] - q.u[k] * s.b[0] - s.u[k] * q.b[0];
 }
 
-// The wave m = 0 .. 5 of the six (fast, Alfven, slow with a > 0; slow, Alfven,
-// fast with a < 0: ascending speeds), given its |a| = t, and the flag of a
-// field along k (t then taken along a coordinate axis).
+// One of the four waves of speed v_1 at B_1 = 0, spanned by du or db along s or t
+// with P = 0
 template <typename R>
-__device__ __forceinline__ void mhd_wave(const MhdBase<R> &s, R sqe, int kind, int sg, R t, bool alf_like, const R c[4],
-                                         MhdWave<R> &q)
+__device__ __forceinline__ void mhd_still_wave(const MhdBase<R> &s, bool along_u, const R d[4], MhdWave<R> &q)
 {
-    const R a = (R)sg * t, lam = s.v1 - a * s.iW;
+    const R bd = mdot<R>(s.b, d);
+    q.p = along_u ? (R)0 : -bd;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        q.u[m] = along_u ? d[m] : (R)0;
+        q.b[m] = along_u ? bd * s.u[m] : d[m];   // (db = (b.du) u)
+    }
+    const R P = q.p + mdot<R>(s.b, q.b);
+    const R n2 = s.beta * (s.W * (q.p * q.p * rcp<R>(s.gp) + s.e * mdot<R>(q.u, q.u) + mdot<R>(q.b, q.b)) +
+                           (R)2 * (q.u[0] * P - s.b[0] * mdot<R>(q.b, q.u)));
+    const R sc = rsq<R>(n2);
+    q.p *= sc;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        q.u[m] *= sc;
+        q.b[m] *= sc;
+    }
+    q.rho = q.p * s.rho * rcp<R>(s.gp);   // adiabatic
+}
+
+// The wave of kind 0 (fast), 1 (Alfven), 2 (slow) on the side sg, given its |a| = t; c
+// spans with u and xi the wave's plane (b, or a coordinate axis where b lies along k).
+// With k^2 = 1 - lambda^2 + a^2, s normal to u, xi and c, t normal to u, xi and s
+// (t^2 = s^2 k^2), every wave has
+//   du = y = y_t t + y_k k (Alfven: s),  d p = Gamma p pk,  d rho = rho pk,
+//   db = r y + pk b + (b.y) u,  r = B/a,
+// so that the norm and dU take the scalars y^2, b.y, db.y = r y^2 + pk b.y, b.db = r b.y + pk
+// b^2 and db^2 = r db.y + pk b.db - (b.y)^2 (u is normal to b and y) instead of 4-vector
+// products (~30 operations fewer per wave, and one code path for the two magnetosonic
+// forms, which differ between the lanes of a warp).  out: dU, and the du (4-vector)
+// and dp it belongs to; FULL: the perturbations q instead of dU.
+template <typename R, bool FULL>
+__device__ __forceinline__ void mhd_wave(const MhdBase<R> &s, R sqe, R gg, int kind, int sg, R tw, bool alf_like,
+                                         const R c[4], MhdWave<R> &q, R dU[8])
+{
+    const R a = (R)sg * tw, lam = s.v1 - a * s.iW;
     R sv[4], tv[4];
     mcross<R>(s.u, lam, c, sv);
     mcross<R>(s.u, lam, sv, tv);
-    if (kind != 0 && !(t > (R)0)) {
-        // B_1 = 0: the four waves of speed v_1, spanned by du or db along s or t with P = 0
-        const R ps = sg > 0 ? (R)0 : -mdot<R>(s.b, kind == 1 ? sv : tv);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const R d = kind == 1 ? sv[m] : tv[m];
-            q.u[m] = sg > 0 ? d : (R)0;
-            q.b[m] = sg > 0 ? (R)0 : d;
-        }
-        q.p = ps;
-        if (sg > 0) {   // db = (b.du) u
-            const R bd = mdot<R>(s.b, q.u);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) q.b[m] = bd * s.u[m];
-        }
-        mhd_scale<R>(s, q);
+    if (kind != 0 && is_zero(tw)) {
+        mhd_still_wave<R>(s, sg > 0, kind == 1 ? sv : tv, q);
+        if constexpr (!FULL) mhd_wave_dU<R>(s, gg, q, dU);
         return;
     }
-    const R r0 = (s.B1 < (R)0 ? -(R)sg : (R)sg);   // the sign of B / a
-    if (kind == 1) {   // Alfven: du = s, db = (B/a) s + (b.s) u with b.s = 0
-        mcross<R>(s.u, lam, tv, sv);
-        const R r = r0 * sqe;
-        q.p = (R)0;
-        const R bs = mdot<R>(s.b, sv);
+    R y[4], y2, by, r, pk;
+    if (kind == 1) {
+        R s2[4];
+        mcross<R>(s.u, lam, tv, s2);   // (normal to u and xi at rounding)
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            q.u[m] = sv[m];
-            q.b[m] = r * sv[m] + bs * s.u[m];
-        }
-        mhd_scale<R>(s, q);
-        return;
-    }
-    const R k2 = ((R)1 - lam) * ((R)1 + lam) + a * a;
-    const R Bx = (s.B1 + a * s.b[0]) * s.iW;
-    R kv[4] = {lam + a * s.u[0], (R)1 + a * s.u[1], a * s.u[2], a * s.u[3]};
-    const R bt = mdot<R>(s.b, tv);
-    R y[4], z[4];
-    if (alf_like) {
-        // y = (B/a) t - (rho h a (b.t)/Sf) k, pi = Gamma p rho h (b.t) k^2/Sf
-        const R Sf = s.rh * a * a - s.gp * k2;
-        const R cf = bt == (R)0 ? (R)0 : s.rh * bt * rcp<R>(Sf);
-        const R r = Bx * rcp<R>(a);
-        const R pk = cf * k2;
-        q.p = s.gp * pk;
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            y[m] = r * tv[m] - cf * a * kv[m];
-            z[m] = r * y[m] + s.b[m] * pk;
-        }
+        for (int m = 0; m < 4; ++m) y[m] = s2[m];
+        r = is_neg(s.B1) ? (R)-sg * sqe : (R)sg * sqe;
+        pk = (R)0;
+        y2 = mdot<R>(y, y);
+        by = mdot<R>(s.b, y);
     } else {
-        // y = a (-k + B (rho h - Gamma p) k^2 (b.t)/(rho h Delta t^2) t), pi = Gamma p k^2
-        const R De = s.e * a * a - Bx * Bx;
-        const R cf = bt == (R)0 ? (R)0 : Bx * (s.rh - s.gp) * k2 * bt * rcp<R>(s.rh * De * mdot<R>(tv, tv));
-        q.p = s.gp * k2;
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const R yy = cf * tv[m] - kv[m];
-            y[m] = a * yy;
-            z[m] = Bx * yy + s.b[m] * k2;
+        const R k2 = ((R)1 - lam) * ((R)1 + lam) + a * a, Bx = (s.B1 + a * s.b[0]) * s.iW;
+        const R bt = mdot<R>(s.b, tv), s2 = mdot<R>(sv, sv), t2 = s2 * k2;
+        R yt, yk;
+        r = Bx * qrcp<R>(a);
+        // alf_like: y = r t - (rho h a (b.t)/Sf) k; else y = a (B (rho h - Gamma p) (b.t)/(rho h
+        // De s^2) t - k)
+        const R den = alf_like ? s.rh * a * a - s.gp * k2 : s.rh * (s.e * a * a - Bx * Bx) * s2;
+        const R num = (alf_like ? s.rh : Bx * (s.rh - s.gp)) * bt;
+        const R cf = is_zero(bt) ? (R)0 : num * qrcp<R>(den);
+        if (alf_like) {
+            yt = r;
+            yk = -cf * a;
+            pk = cf * k2;
+        } else {
+            yt = a * cf;
+            yk = -a;
+            pk = k2;
         }
+        const R ka = yk * a;   // k = xi + a u
+        y[0] = yt * tv[0] + (yk * lam + ka * s.u[0]);
+        y[1] = yt * tv[1] + (yk + ka * s.u[1]);
+        y[2] = yt * tv[2] + ka * s.u[2];
+        y[3] = yt * tv[3] + ka * s.u[3];
+        y2 = yt * yt * t2 + yk * yk * k2;
+        by = yt * bt + yk * Bx;
     }
-    const R by = mdot<R>(s.b, y);
+    R bz = r * by + pk * s.b2;
+    const R zy = r * y2 + pk * by, db2 = r * zy + (pk * bz - by * by);
+    const R n2 = s.beta * (s.W * (s.gp * pk * pk + (s.e * y2 + db2)) + (R)2 * (y[0] * (s.gp * pk + bz) - s.b[0] * zy));
+    const R sc = qrsq<R>(n2);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        q.u[m] = y[m];
-        q.b[m] = z[m] + by * s.u[m];
+    for (int m = 0; m < 4; ++m) y[m] *= sc;
+    pk *= sc;
+    by *= sc;
+    bz *= sc;
+    const R p = s.gp * pk;
+    const R db0 = r * y[0] + (pk * s.b[0] + by * s.W);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) q.u[m] = y[m];
+    q.p = p;
+    q.rho = s.rho * pk;
+    if constexpr (FULL) {
+        q.b[0] = db0;
+#pragma unroll
+        for (int k = 1; k < 4; ++k) q.b[k] = r * y[k] + (pk * s.b[k] + by * s.u[k]);
+    } else {
+        const R c1 = s.e * s.W, de = (s.rho + gg * s.gp) * pk + (R)2 * bz, c0 = de * s.W + s.e * y[0];
+        const R hb = y[0] + s.W * pk, hy = s.W * r - s.b[0], hu = s.W * by - db0;
+        const R gu = c0 - s.b[0] * by, gy = c1 - s.b[0] * r, gb = db0 + s.b[0] * pk;
+        dU[0] = s.rho * hb;
+#pragma unroll
+        for (int k = 1; k < 4; ++k) {
+            dU[k] = gu * s.u[k] + (gy * y[k] - gb * s.b[k]);
+            dU[4 + k] = hb * s.b[k] + (hy * y[k] + hu * s.u[k]);
+        }
+        dU[4] = de * (s.W * s.W) + (R)2 * (c1 * y[0] - s.b[0] * db0) - (p + bz);
     }
-    mhd_scale<R>(s, q);
 }
 
 // The six waves' |a| and the frame data shared by their vectors.
 template <typename R>
 struct MhdSix {
-    R t[6], sqe, c[2][4];
-    bool alf[2];   // per side: the fast wave is the Alfven-like one
+    R t[6], sqe;
+    bool alf[2];     // per side: the fast wave is the Alfven-like one
+    bool axis[2];    // b along k (|b_t| at rounding level) or no field: c a coordinate axis
 };
 
 template <typename R>
 __device__ __forceinline__ void mhd_six(const MhdBase<R> &s, MhdSix<R> &x, R lam[6])
 {
-    x.sqe = sq_rt<R>(s.e);
+    MhdCoef<R> kc;
+    mhd_coef<R>(s, kc);
+    x.sqe = kc.sqe;
+    const float irh = __frcp_rn(to_f32(s.rh)), gp = to_f32(s.gp) * irh;
+#pragma unroll
     for (int side = 0; side < 2; ++side) {
         const int sg = side == 0 ? 1 : -1;
         R tA, ts, tf;
-        mhd_side<R>(s, x.sqe, sg, true, tA, ts, tf);
+        mhd_side<R>(s, kc, sg, true, tA, ts, tf);
         const int o = side == 0 ? 0 : 5, d = side == 0 ? 1 : -1;
         x.t[o] = tf;
         x.t[o + d] = tA;
         x.t[o + 2 * d] = ts;
-        const R a = (R)sg * tA, la = s.v1 - a * s.iW;
-        x.alf[side] = s.rh * a * a > s.gp * (((R)1 - la) * ((R)1 + la) + a * a);
-        // b along k (|b_t| at rounding level) or no field: the plane normal to
-        // k spanned from a coordinate axis, the same for the side's waves
+        // (at equality of the two factors either choice holds)
+        const float af = to_f32(tA), lf = to_f32(s.v1) - (float)sg * af * to_f32(s.iW);
+        x.alf[side] = af * af > gp * ((1.0f - lf) * (1.0f + lf) + af * af);
+        const R la = s.v1 - (R)sg * tA * s.iW;
         R sv[4];
         mcross<R>(s.u, la, s.b, sv);
-        const R bt2 = mdot<R>(sv, sv);
-        const R A = s.u[0] - la * s.u[1];
-        if (bt2 > (R)(sizeof(R) == 4 ? 1.0e-10 : 1.0e-22) * s.b2 * A * A) {
-            for (int m = 0; m < 4; ++m) x.c[side][m] = s.b[m];
-        } else {
-            x.c[side][0] = x.c[side][1] = x.c[side][3] = (R)0;
-            x.c[side][2] = (R)1;
-        }
+        const R A = s.u[0] - la * s.u[1], q = (R)(sizeof(R) == 4 ? 1.0e-10 : 1.0e-22) * s.b2 * A * A;
+        x.axis[side] = !(sgn_d(mdot<R>(sv, sv) - q) > 0);
     }
 #pragma unroll
     for (int m = 0; m < 6; ++m) lam[m] = m < 3 ? s.v1 - x.t[m] * s.iW : s.v1 + x.t[m] * s.iW;
 }
 
-template <typename R>
-__device__ __forceinline__ void mhd_six_wave(const MhdBase<R> &s, const MhdSix<R> &x, int m, MhdWave<R> &q)
+template <typename R, bool FULL>
+__device__ __forceinline__ void mhd_six_wave(const MhdBase<R> &s, const MhdSix<R> &x, R gg, int m, MhdWave<R> &q, R dU[8])
 {
     const int side = m < 3 ? 0 : 1, kind = m < 3 ? m : 5 - m;   // 0 fast, 1 Alfven, 2 slow
-    const bool alf_like = kind == 0 ? x.alf[side] : !x.alf[side];
-    mhd_wave<R>(s, x.sqe, kind, side == 0 ? 1 : -1, x.t[m], alf_like, x.c[side], q);
+    const bool alf = side == 0 ? x.alf[0] : x.alf[1], axis = side == 0 ? x.axis[0] : x.axis[1];
+    const R c[4] = {axis ? (R)0 : s.b[0], axis ? (R)0 : s.b[1], axis ? (R)1 : s.b[2], axis ? (R)0 : s.b[3]};
+    mhd_wave<R, FULL>(s, x.sqe, gg, kind, side == 0 ? 1 : -1, x.t[m], kind == 0 ? alf : !alf, c, q, dU);
+}
+
+// The entropy wave (d rho = 1; its dU[5..7] = 0) and the divergence wave dB = e_1 -
+// v_1 v, both of speed v_1.
+template <typename R>
+__device__ __forceinline__ void mhd_entropy_dU(const MhdBase<R> &s, R igg, R dU[8])
+{
+    const R q = s.W * s.rho * igg, sr = q * qrsq<R>(q);   // W sqrt(rho/(Gamma/(Gamma-1) W))
+    dU[0] = sr;
+#pragma unroll
+    for (int k = 1; k < 4; ++k) dU[k] = s.u[k] * sr;
+    dU[4] = s.W * sr;
+#pragma unroll
+    for (int k = 5; k < 8; ++k) dU[k] = (R)0;
+}
+template <typename R>
+__device__ __forceinline__ void mhd_divergence_dU(const MhdBase<R> &s, R dU[8])
+{
+    // db = (v_1/W, dB/W + (v_1/W) v) = e_1/W + (v_1/W)(1, 0): du = dp = 0
+    const R b0 = s.v1 * s.iW, b1 = s.iW;
+    const R sd = qrsq<R>(s.beta * s.iW * ((R)1 - s.v1 * s.v1));
+    const R db0 = b0 * sd, db1 = b1 * sd, bdb = s.b[1] * db1 - s.b[0] * db0, de = (R)2 * bdb, c0 = de * s.W;
+    dU[0] = (R)0;
+    dU[1] = c0 * s.u[1] - db0 * s.b[1] - s.b[0] * db1;
+    dU[2] = c0 * s.u[2] - db0 * s.b[2];
+    dU[3] = c0 * s.u[3] - db0 * s.b[3];
+    dU[4] = c0 * s.W - (R)2 * (s.b[0] * db0) - bdb;
+    dU[5] = s.W * db1 - s.u[1] * db0;
+    dU[6] = -s.u[2] * db0;
+    dU[7] = -s.u[3] * db0;
 }
 
 }  // namespace esmm
