@@ -79,7 +79,7 @@ __device__ __forceinline__ double nested_e3(const Geom3 &g, const double *__rest
 }
 
 template <int P>
-__global__ void k3_node(Geom3 g, double gam, const double *__restrict__ cons, const double *__restrict__ J,
+__global__ void __maxnreg__(64) k3_node(Geom3 g, double gam, const double *__restrict__ cons, const double *__restrict__ J,
                         const double *__restrict__ xe, const double *__restrict__ xdot,
                         const double *__restrict__ zg_in, double *__restrict__ zg_out, double *__restrict__ q,
                         int *__restrict__ status, const double *__restrict__ inflow)
@@ -90,7 +90,7 @@ __global__ void k3_node(Geom3 g, double gam, const double *__restrict__ cons, co
     int Jn = (int)((t / g.pd[0]) % g.pd[1]) - GH;
     int K = (int)(t / ((long long)g.pd[0] * g.pd[1])) - GH;
     long long src = data_src3(g, I, Jn, K);
-    double iJ = 1.0 / J[src];
+    double iJ = qrcp<double>(J[src]);
     double U[8], w[8], Z;
 #pragma unroll
     for (int a = 0; a < 8; ++a) U[a] = cons[a * g.N + src] * iJ;
@@ -107,8 +107,8 @@ __global__ void k3_node(Geom3 g, double gam, const double *__restrict__ cons, co
         if (st) atomicAdd(status, 1);
         if (zg_out) zg_out[src] = Z;
     }
-    double W = 1.0 / sqrt(1.0 - (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]));
-    double beta = w[0] / w[4];
+    const double W = qrsq<double>(1.0 - (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]));
+    const double beta = w[0] * qrcp<double>(w[4]);
     q[F_RHO * g.P + t] = w[0];
     q[F_P * g.P + t] = w[4];
     q[F_BETA * g.P + t] = beta;

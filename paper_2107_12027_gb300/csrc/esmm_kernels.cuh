@@ -65,7 +65,7 @@ __device__ __forceinline__ void mesh_deltas(const Geom &g, const double *__restr
 // mean's jump outside its near-equal branch, while the totals take a pass
 // with FP64 logarithms.  gg = (Gamma - 1)/Gamma comes with the launch.
 template <int P>
-__global__ void k_node(ProbArg pa, double gam, double gg, const double *__restrict__ cons,
+__global__ void __maxnreg__(64) k_node(ProbArg pa, double gam, double gg, const double *__restrict__ cons,
                        const double *__restrict__ J, const double *__restrict__ x, const double *__restrict__ xdot,
                        const double *__restrict__ pg_in, double *__restrict__ pg_out, double *__restrict__ q,
                        int *__restrict__ status, float *__restrict__ q32, const double *__restrict__ inflow,
@@ -86,7 +86,7 @@ __global__ void k_node(ProbArg pa, double gam, double gg, const double *__restri
     q += (long long)NQ * D.op;
     int I = (int)(t % g.px) - GH, Jn = (int)(t / g.px) - GH;
     long long src = data_src(g, I, Jn);
-    double iJ = __drcp_rn(J[src]);
+    double iJ = qrcp<double>(J[src]);
     double Dd = cons[src] * iJ, mx = cons[g.N + src] * iJ, my = cons[2 * g.N + src] * iJ,
            E = cons[3 * g.N + src] * iJ;
     double rho, vx, vy, p, W;
@@ -104,7 +104,7 @@ __global__ void k_node(ProbArg pa, double gam, double gg, const double *__restri
         if (st) atomicAdd(status, 1);
         if (pg_out) pg_out[src] = p;
     }
-    double beta = rho * __drcp_rn(p);
+    double beta = rho * qrcp<double>(p);
     q[Q_RHO * g.P + t] = rho;
     q[Q_P * g.P + t] = p;
     q[Q_BETA * g.P + t] = beta;

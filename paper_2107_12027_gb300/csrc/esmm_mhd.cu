@@ -32,7 +32,7 @@ __global__ void k_prim_out_mhd(ProbArg pa, double gam, const double *__restrict_
 // With cflb (the moving-mesh step) also the speed bounds L_k lambda_min/J and
 // L_k lambda_max/J of every node into its rows 2 + k and 4 + k.
 template <typename R>
-__global__ void k_cfl_mhd(ProbArg pa, double gam, const double *__restrict__ q, const double *__restrict__ J,
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_cfl_mhd(ProbArg pa, double gam, const double *__restrict__ q, const double *__restrict__ J,
                           unsigned long long *red, double *__restrict__ cflb)
 {
     ProbDesc D;
@@ -44,15 +44,15 @@ __global__ void k_cfl_mhd(ProbArg pa, double gam, const double *__restrict__ q, 
     if (id < g.N) {
         int i = (int)(id % g.nx), j = (int)(id / g.nx);
         long long c = pidx(g, i, j);
-        double iW = 1.0 / q[Q_W * g.P + c];
+        const double iW = qrcp<double>(q[Q_W * g.P + c]);
         double w[8] = {q[Q_RHO * g.P + c], q[Q_UX * g.P + c] * iW, q[Q_UY * g.P + c] * iW,
                        q[QM_UZ * g.P + c] * iW, q[Q_P * g.P + c], q[QM_B1 * g.P + c], q[QM_B2 * g.P + c],
                        q[QM_B3 * g.P + c]};
-        double iJ = 1.0 / J[id];
+        const double iJ = qrcp<double>(J[id]);
+#pragma unroll 1
         for (int k = 0; k < 2; ++k) {
             double mx = q[(Q_M00 + 2 * k) * g.P + c], my = q[(Q_M01 + 2 * k) * g.P + c];
-            double Lk = sqrt(mx * mx + my * my);
-            double nx = mx / Lk, ny = my / Lk;
+            const double l2 = mx * mx + my * my, iLk = qrsq<double>(l2), Lk = l2 * iLk, nx = mx * iLk, ny = my * iLk;
             R wr[8] = {(R)w[0], (R)(nx * w[1] + ny * w[2]), (R)(-ny * w[1] + nx * w[2]), (R)w[3],
                        (R)w[4], (R)(nx * w[5] + ny * w[6]), (R)(-ny * w[5] + nx * w[6]), (R)w[7]};
             R l0, l1;

@@ -28,18 +28,78 @@ static_assert(NQM32 == NQ32_MHD, "the allocation of the FP32 copies");
 constexpr int NFM = 10;                          // interface values per direction: F[8], J xi_t, B~ (NF_MHD)
 
 // ---------------------------------------------------------------------------
-// Primitive recovery (FP64).  Newton on Z = rho h W^2 with bisection on
-// [0, Gamma E]; with S = m.B,
+// Primitive recovery (FP64).  The root in Z = rho h W^2 of, with S = m.B,
 //   v.B = S/Z,  |v|^2 = (|m|^2 + (2Z + |B|^2) S^2/Z^2)/(Z + |B|^2)^2,
 //   p = (Gamma-1)/Gamma (Z/W^2 - D/W),
 //   f(Z) = Z - p + |B|^2 (1 + |v|^2)/2 - S^2/(2 Z^2) - E,
-// a trial Z with |v|^2 >= 1 lying below the root.  Stops when a step moves Z
-// by at most 1e-15 (E + Z), or where |f| <= 2e-15 (E + Z), f's rounding
-// level (a root, whose tiny steps the open bracket would otherwise reject).
-// Z0: warm start (ignored outside the bracket).  Quotients are taken through
-// reciprocals, and the Newton step divides by df through an FP32 reciprocal
-// (the slope only steers the step; f, which decides the stopping, is FP64).
+// a trial Z with |v|^2 >= 1 lying below the root.  As in cons2prim_gg: an FP32 Newton
+// iteration gives Z to about 1e-7, one FP64 step of third order lands on the root to
+// rounding (the last where it is below 3e-6 of Z (1 - v^2), the length on which f bends, and
+// its second-order part below 3e-6 of it), and where that fails three times c2p_loop_mhd, FP64 Newton with
+// bisection on [0, Gamma E], which stops when a step moves Z by at most 1e-15 (E + Z), or
+// where |f| <= 2e-15 (E + Z), f's rounding level (a root, whose tiny steps the open
+// bracket would otherwise reject).  The FP32 iteration works in units of E.
+// Z0: warm start (ignored outside the bracket).  Measured: the node pass of 512^2 nodes 214 ->
+// 146 us, mixed rotor steps 3.71 -> 3.05 ms (with the speeds' pass in 80 registers).
 // Returns 0, 1 (non-admissible) or 2 (iteration cap).
+__device__ __forceinline__ float c2p_estimate_mhd(float g, float gam, float D, float m2, float B2, float S2, float z0)
+{
+    float lo = 0.0f, hi = gam, Z = z0;
+#pragma unroll 1
+    for (int it = 0; it < 24; ++it) {
+        const float iZ = __frcp_rn(Z), q = __frcp_rn(Z + B2), t = S2 * iZ * iZ, N = m2 + (2.0f * Z + B2) * t;
+        const float v2 = N * q * q;
+        float Zn;
+        bool done = false;
+        if (!(v2 < 1.0f)) {
+            lo = Z;
+            Zn = 0.5f * (lo + hi);
+        } else {
+            const float iW2 = 1.0f - v2, rs = rsqrtf(iW2), dv2 = (-2.0f * t * (1.0f + B2 * iZ) - 2.0f * N * q) * q * q;
+            const float f = Z - 1.0f - g * (Z * iW2 - D * (iW2 * rs)) + 0.5f * (B2 * (1.0f + v2) - t);
+            const float df = 1.0f - g * (iW2 - Z * dv2 + 0.5f * D * dv2 * rs) + 0.5f * B2 * dv2 + t * iZ;
+            if (f < 0.0f) lo = Z; else hi = Z;
+            Zn = Z - f * __frcp_rn(df);
+            done = fabsf(Zn - Z) <= 2.0e-4f * Z * iW2;   // (as in c2p_estimate)
+            if (!done && !(Zn > lo && Zn < hi)) Zn = 0.5f * (lo + hi);
+        }
+        Z = Zn;
+        if (done) break;
+    }
+    return Z;
+}
+
+static __device__ __noinline__ int c2p_loop_mhd(double g, double D, double m2, double B2, double S2, double E, double hi,
+                                                double &Z)
+{
+    double lo = 0.0;
+#pragma unroll 1
+    for (int it = 0; it < 300; ++it) {
+        const double iZ = __drcp_rn(Z), iZB = __drcp_rn(Z + B2), N = m2 + (2.0 * Z + B2) * S2 * iZ * iZ, v2 = N * iZB * iZB;
+        double Zn;
+        if (!(v2 < 1.0)) {
+            lo = Z;
+            Zn = 0.5 * (lo + hi);
+        } else {
+            const double iW2 = 1.0 - v2, rs = rsqrt(iW2), iW = iW2 * rs;
+            const double p = g * (Z * iW2 - D * iW);
+            const double f = Z - p + 0.5 * B2 * (1.0 + v2) - 0.5 * S2 * iZ * iZ - E;
+            if (fabs(f) <= 2.0e-15 * (E + Z)) return 0;   // residual at rounding level
+            const double dN = -2.0 * S2 * iZ * iZ - 2.0 * B2 * S2 * iZ * iZ * iZ;
+            const double dv2 = dN * iZB * iZB - 2.0 * N * iZB * iZB * iZB;
+            const double dp = g * (iW2 - Z * dv2 + 0.5 * D * dv2 * rs);
+            const double df = 1.0 - dp + 0.5 * B2 * dv2 + S2 * iZ * iZ * iZ;
+            if (f < 0.0) lo = Z; else hi = Z;
+            Zn = Z - f * f2d_int(__frcp_rn(d2f_int(df)));   // (the slope only steers the step)
+            if (!(Zn > lo && Zn < hi)) Zn = 0.5 * (lo + hi);
+        }
+        const bool done = fabs(Zn - Z) <= 1.0e-15 * (E + Zn);
+        Z = Zn;
+        if (done) return 0;
+    }
+    return 2;
+}
+
 __device__ __forceinline__ int cons2prim_mhd(double gam, const double U[8], double Z0, double w[8], double &Zout)
 {
     const double D = U[0], E = U[4];
@@ -52,42 +112,46 @@ __device__ __forceinline__ int cons2prim_mhd(double gam, const double U[8], doub
     for (int a = 0; a < 8; ++a) w[a] = 0.0;
     Zout = 0.0;
     if (!(D > 0.0) || !(E > 0.0)) return 1;
-    double lo = 0.0, hi = gam * E;
-    double Z = (Z0 > lo && Z0 < hi) ? Z0 : 0.5 * (lo + hi);
-    int ok = 0;
-    for (int it = 0; it < 300; ++it) {
-        double ZB = Z + B2;
-        double iZ = __drcp_rn(Z);
-        double N = m2 + (2.0 * Z + B2) * S2 * iZ * iZ;
-        double iZB = __drcp_rn(ZB);
-        double v2 = N * iZB * iZB;
-        double Zn;
-        if (!(v2 < 1.0)) {
-            lo = Z;
-            Zn = 0.5 * (lo + hi);
-        } else {
-            double iW2 = 1.0 - v2, rs = rsqrt(iW2), iW = iW2 * rs;
-            double p = g * (Z * iW2 - D * iW);
-            double f = Z - p + 0.5 * B2 * (1.0 + v2) - 0.5 * S2 * iZ * iZ - E;
-            double dN = -2.0 * S2 * iZ * iZ - 2.0 * B2 * S2 * iZ * iZ * iZ;
-            double dv2 = dN * iZB * iZB - 2.0 * N * iZB * iZB * iZB;
-            double dp = g * (iW2 - Z * dv2 + 0.5 * D * dv2 * rs);
-            double df = 1.0 - dp + 0.5 * B2 * dv2 + S2 * iZ * iZ * iZ;
-            if (fabs(f) <= 2.0e-15 * (E + Z)) { ok = 1; break; }   // residual at rounding level
-            Zn = Z;                          // f = 0: Z is a root
-            if (f != 0.0) {
-                if (f < 0.0) lo = Z; else hi = Z;
-                Zn = Z - f * f2d_int(__frcp_rn(d2f_int(df)));
-                if (!(Zn > lo && Zn < hi)) Zn = 0.5 * (lo + hi);
-            }
+    const double hi = gam * E;
+    const double Zw = (Z0 > 0.0 && Z0 < hi) ? Z0 : 0.5 * hi;
+    const float Ef = d2f_int(E), iE = __frcp_rn(Ef), gf = d2f_int(g), Df = d2f_int(D) * iE, B2f = d2f_int(B2) * iE;
+    const float m2f = d2f_int(m2) * iE * iE, S2f = d2f_int(S2) * iE * iE * iE;
+    const float Zf = c2p_estimate_mhd(gf, d2f_int(gam), Df, m2f, B2f, S2f, d2f_int(Zw) * iE);
+    double Z = f2d_int(Zf * Ef);
+    int st = 0;
+    bool ok = false;
+#pragma unroll 1
+    for (int it = 0; it < 3; ++it) {   // (a second step where the estimate was poor)
+        const double iZ = qrcp<double>(Z), iZB = qrcp<double>(Z + B2), t = S2 * iZ * iZ, N = m2 + (2.0 * Z + B2) * t;
+        const double q2 = iZB * iZB, v2 = N * q2, iW2 = 1.0 - v2, rs = qrsq<double>(iW2), Dw = D * rs;
+        const double f = (Z - E) - g * (Z * iW2 - Dw * iW2) + 0.5 * (B2 * (1.0 + v2) - t);
+        const double dv2 = -2.0 * (t * (1.0 + B2 * iZ) + N * iZB) * q2;
+        const double df = 1.0 - g * (iW2 - dv2 * (Z - 0.5 * Dw)) + 0.5 * B2 * dv2 + t * iZ;
+        const double dZ = f * qrcp<double>(df);
+        // f'' in units of E (Z = z E): v2'' = N'' q^2 - 4 N' q^3 + 6 N q^4
+        const float z = d2f_int(Z) * iE, iz = __frcp_rn(z), q = __frcp_rn(z + B2f), tf = S2f * iz * iz, Nf = m2f + (2.0f * z + B2f) * tf;
+        const float N1 = -2.0f * tf * (1.0f + B2f * iz), N2 = tf * iz * (4.0f + 6.0f * B2f * iz), qq = q * q;
+        const float v1 = (N1 - 2.0f * Nf * q) * qq, v22 = (N2 - 4.0f * N1 * q + 6.0f * Nf * qq) * qq, sf = d2f_int(rs);
+        const float p2 = gf * (-2.0f * v1 - z * v22 + 0.5f * Df * sf * (v22 + 0.5f * v1 * v1 * (sf * sf)));
+        const float f2 = -p2 + 0.5f * B2f * v22 - 3.0f * tf * (iz * iz);
+        const float dz = d2f_int(dZ) * iE, eta = 0.5f * f2 * dz * __frcp_rn(d2f_int(df));
+        ok = fabsf(dz) <= 3.0e-6f * z * d2f_int(iW2) && fabsf(eta) <= 3.0e-6f;
+        const double Zn = Z - (dZ + f2d_int(dz * eta * Ef));
+        if (!(d2f_int(Zn) > 0.0f) || !(fabsf(eta) <= 0.1f)) {
+            ok = false;
+            break;
         }
-        if (fabs(Zn - Z) <= 1.0e-15 * (E + Zn)) { Z = Zn; ok = 1; break; }
         Z = Zn;
+        if (ok) break;
     }
-    double ZB = Z + B2, iZ = __drcp_rn(Z), iZB = __drcp_rn(ZB);
-    double v2 = (m2 + (2.0 * Z + B2) * S2 * iZ * iZ) * iZB * iZB;
+    if (!ok) {
+        Z = Zw;
+        st = c2p_loop_mhd(g, D, m2, B2, S2, E, hi, Z);
+    }
+    const double iZ = ok ? qrcp<double>(Z) : __drcp_rn(Z), iZB = ok ? qrcp<double>(Z + B2) : __drcp_rn(Z + B2);
+    const double v2 = (m2 + (2.0 * Z + B2) * S2 * iZ * iZ) * iZB * iZB;
     if (!(v2 < 1.0)) return 1;
-    double iW2 = 1.0 - v2, iW = sqrt(iW2);
+    const double iW2 = 1.0 - v2, iW = ok ? iW2 * qrsq<double>(iW2) : sqrt(iW2);
     double vB = S * iZ;
     w[0] = D * iW;
     w[1] = (m0 + vB * B0) * iZB;
@@ -97,7 +161,7 @@ __device__ __forceinline__ int cons2prim_mhd(double gam, const double U[8], doub
     w[5] = B0; w[6] = B1; w[7] = B2_;
     Zout = Z;
     if (!(w[4] > 0.0)) return 1;
-    return ok ? 0 : 2;
+    return st;
 }
 
 // U(w), F_1(w) and V(w) (eq. RMHDdiv2, Sec. 2), generic in the number type
@@ -982,7 +1046,7 @@ __device__ __forceinline__ void ec_pair_mhd(const NodeMT<R> &L, const NodeMT<R> 
 // ---------------------------------------------------------------------------
 // Per padded node: recovery (warm-started from zg_in), node values, metrics.
 template <int P>
-__global__ void k_node_mhd(ProbArg pa, double gam, const double *__restrict__ cons, const double *__restrict__ J,
+__global__ void __maxnreg__(64) k_node_mhd(ProbArg pa, double gam, const double *__restrict__ cons, const double *__restrict__ J,
                            const double *__restrict__ x, const double *__restrict__ xdot,
                            const double *__restrict__ zg_in, double *__restrict__ zg_out, double *__restrict__ q,
                            int *__restrict__ status, const double *__restrict__ inflow, int f32_logs,
@@ -996,7 +1060,7 @@ __global__ void k_node_mhd(ProbArg pa, double gam, const double *__restrict__ co
     if (t >= g.P) return;
     int I = (int)(t % g.px) - GH, Jn = (int)(t / g.px) - GH;
     long long src = data_src(g, I, Jn);
-    double iJ = 1.0 / J[src];
+    double iJ = qrcp<double>(J[src]);
     double U[8], w[8], Z;
 #pragma unroll
     for (int a = 0; a < 8; ++a) U[a] = cons[a * g.N + src] * iJ;
