@@ -526,6 +526,7 @@ struct esmm3 {
     int p, w;
     esmm_params prm;
     cudaStream_t st;
+    SideStream side;   // the second of the three sweep directions
     int has_state, xdot_zero;
     int needs_inflow, has_inflow;
     double *inflow_dev;        // [8] primitive inflow state (ESMM_INFLOW ends)
@@ -636,16 +637,23 @@ void node3(esmm3 *g, const double *cons, const double *J, const double *x, const
     }
 }
 
+// the stream of the second sweep direction, whose buffers are its own (timed launches
+// stay in line on the grid's stream)
+cudaStream_t side_begin3(esmm3 *g)
+{
+    const bool timed = g->prof_mask & ((1 << ESMM_KIND_IFACE) | (1 << ESMM_KIND_PAIRS));
+    return g->side.begin(g->st, !timed);
+}
+
 void fluxes3(esmm3 *g)
 {
     Phys ph = phys3(g);
+    const cudaStream_t side = side_begin3(g);
     for (int dir = 0; dir < 3; ++dir) {
-        int oa = dir == 0 ? 1 : 0, ob = dir == 2 ? 1 : 2;
-        long long count = (long long)(g->g.n[dir] + 1) * g->g.n[oa] * g->g.n[ob];
-        unsigned nb = nb3(count, 128);
         Prof3 pr_(g, ESMM_KIND_IFACE);
-        launch3_iface(g->g, ph, g->p, g->w, g->q, g->iflux, dir, nb, g->st);
+        launch3_iface(g->g, ph, g->p, g->w, g->q, g->iflux, dir, dir == 1 ? side : g->st);
     }
+    g->side.end(g->st, side);
 }
 
 void update3(esmm3 *g, double *dc, double *dJ, const double *cn, const double *Jn, const double *xn, const double *cs,
@@ -753,6 +761,7 @@ void free3(esmm3 *g)
                     &g->inflow_dev, &g->cflb, &g->npart};
     for (double **p : b)
         if (*p) { cudaFree(*p); *p = nullptr; }
+    g->side.destroy();
     if (g->ck) {
         for (double *c : *g->ck) cudaFree(c);
         delete g->ck;
@@ -790,20 +799,23 @@ int rhs_vjp_core3(esmm3 *g, const double *cons, const double *J, const double *x
     CK3(cudaMemsetAsync(g->lamq, 0, 11 * P * d, g->st));
     CK3(cudaMemsetAsync(lam, 0, 8 * N * d, g->st));
     Phys ph = phys3(g);
+    const cudaStream_t side = side_begin3(g);
     for (int dir = 0; dir < 3; ++dir) {
+        const cudaStream_t st = dir == 1 ? side : g->st;
         {
             Prof3 pr_(g, ESMM_KIND_IFACE);   // the Powell term's div B~
-            launch3_bflux(g->g, ph, g->q, g->iflux, dir, g->st);
+            launch3_bflux(g->g, ph, g->q, g->iflux, dir, st);
         }
         {
             Prof3 pr_(g, ESMM_KIND_PAIRS);
-            launch3_pairs_vjp(g->g, ph, g->q, mu, g->lamq, dir, g->st);
+            launch3_pairs_vjp(g->g, ph, g->q, mu, g->lamq, dir, st);
         }
         if (g->w > 0) {
             Prof3 pr_(g, ESMM_KIND_IFACE);
-            launch3_iface_vjp(g->g, ph, g->q, mu, g->lamq, dir, g->st);
+            launch3_iface_vjp(g->g, ph, g->q, mu, g->lamq, dir, st);
         }
     }
+    g->side.end(g->st, side);
     {
         Prof3 pr_(g, ESMM_KIND_NODE);
         launch3_node_vjp(g->g, g->gamma, g->q, g->lamq, g->iflux, mu, J, lam, g->st);
@@ -879,7 +891,7 @@ int esmm3_create(esmm3 **out, const int n[3], const double lo[3], const double h
         {&g->grad, N}, {&g->om, N}, {&g->om2, N}, {&g->X, 3 * N}, {&g->Xn, 3 * N}, {&g->dt_dev, 1},
         {&g->t_dev, 1}, {&g->partials, 3 * nb}, {&g->tot, 3}, {&g->xe, (size_t)NXE * ext_count3(g->g)},
         {&g->inflow_dev, 8}, {&g->cflb, 9 * N}, {&g->npart, 6 * nb}};
-    bool ok = true;
+    bool ok = g->side.create();
     for (auto &a : al) ok = ok && cudaMalloc((void **)a.p, a.n * d) == cudaSuccess;
     ok = ok && cudaMalloc((void **)&g->red, NR3 * sizeof(unsigned long long)) == cudaSuccess &&
          cudaMalloc((void **)&g->ds, sizeof(DtSolve)) == cudaSuccess &&

@@ -307,7 +307,13 @@ __global__ void __launch_bounds__(128) k3_iface(Geom3 g, Phys ph, const double *
 
 // launch of the interface kernel of one direction (esmm_3d_iface.cu)
 void launch3_iface(const Geom3 &g, const Phys &ph, int p, int w, const double *q, double *iflux, int dir,
-                   unsigned nb, cudaStream_t st);
+                   cudaStream_t st);
+
+// sites of a sweep direction extended by ext
+inline long long sites3(const Geom3 &g, int dir, int ext)
+{
+    return (long long)(g.n[dir] + ext) * g.n[dir == 0 ? 1 : 0] * g.n[dir == 2 ? 1 : 2];
+}
 
 // adjoint kernels (esmm_3d_adjoint.cu): node-quantity adjoints lamq[11][P]
 // from the pair and interface passes, then the node pass into lam [8][N]

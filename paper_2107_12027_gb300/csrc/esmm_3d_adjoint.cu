@@ -448,29 +448,32 @@ inline unsigned nbk(long long n, int bs = 128) { return (unsigned)((n + bs - 1) 
 void launch3_pairs_vjp(const Geom3 &g, const Phys &ph, const double *q, const double *mu, double *lamq, int dir,
                        cudaStream_t st)
 {
-    const int oa = dir == 0 ? 1 : 0, ob = dir == 2 ? 1 : 2;
-    const unsigned nb = nbk((long long)(g.n[dir] + ph.p) * g.n[oa] * g.n[ob]);
-    if (ph.p == 1) k3_pairs_vjp<1><<<nb, 128, 0, st>>>(g, ph, q, mu, lamq, dir);
-    else if (ph.p == 2) k3_pairs_vjp<2><<<nb, 128, 0, st>>>(g, ph, q, mu, lamq, dir);
-    else k3_pairs_vjp<3><<<nb, 128, 0, st>>>(g, ph, q, mu, lamq, dir);
+    const long long n = sites3(g, dir, ph.p);
+    const int bs = block_for(n, 128, 64);
+    const unsigned nb = nbk(n, bs);
+    if (ph.p == 1) k3_pairs_vjp<1><<<nb, bs, 0, st>>>(g, ph, q, mu, lamq, dir);
+    else if (ph.p == 2) k3_pairs_vjp<2><<<nb, bs, 0, st>>>(g, ph, q, mu, lamq, dir);
+    else k3_pairs_vjp<3><<<nb, bs, 0, st>>>(g, ph, q, mu, lamq, dir);
 }
 
 void launch3_iface_vjp(const Geom3 &g, const Phys &ph, const double *q, const double *mu, double *lamq, int dir,
                        cudaStream_t st)
 {
-    const int oa = dir == 0 ? 1 : 0, ob = dir == 2 ? 1 : 2;
-    const unsigned nb = nbk((long long)(g.n[dir] + 1) * g.n[oa] * g.n[ob]);
-    if (ph.w == 5) k3_iface_vjp<5><<<nb, 128, 0, st>>>(g, ph, q, mu, lamq, dir);
-    else if (ph.w == 3) k3_iface_vjp<3><<<nb, 128, 0, st>>>(g, ph, q, mu, lamq, dir);
+    const long long n = sites3(g, dir, 1);
+    const int bs = block_for(n, 128, 64);
+    const unsigned nb = nbk(n, bs);
+    if (ph.w == 5) k3_iface_vjp<5><<<nb, bs, 0, st>>>(g, ph, q, mu, lamq, dir);
+    else if (ph.w == 3) k3_iface_vjp<3><<<nb, bs, 0, st>>>(g, ph, q, mu, lamq, dir);
 }
 
 void launch3_bflux(const Geom3 &g, const Phys &ph, const double *q, double *iflux, int dir, cudaStream_t st)
 {
-    const int oa = dir == 0 ? 1 : 0, ob = dir == 2 ? 1 : 2;
-    const unsigned nb = nbk((long long)(g.n[dir] + 1) * g.n[oa] * g.n[ob]);
-    if (ph.p == 1) k3_bflux<1><<<nb, 128, 0, st>>>(g, ph, q, iflux, dir);
-    else if (ph.p == 2) k3_bflux<2><<<nb, 128, 0, st>>>(g, ph, q, iflux, dir);
-    else k3_bflux<3><<<nb, 128, 0, st>>>(g, ph, q, iflux, dir);
+    const long long n = sites3(g, dir, 1);
+    const int bs = block_for(n, 128, 64);
+    const unsigned nb = nbk(n, bs);
+    if (ph.p == 1) k3_bflux<1><<<nb, bs, 0, st>>>(g, ph, q, iflux, dir);
+    else if (ph.p == 2) k3_bflux<2><<<nb, bs, 0, st>>>(g, ph, q, iflux, dir);
+    else k3_bflux<3><<<nb, bs, 0, st>>>(g, ph, q, iflux, dir);
 }
 
 void launch3_node_vjp(const Geom3 &g, double gam, const double *q, const double *lamq, const double *iflux,

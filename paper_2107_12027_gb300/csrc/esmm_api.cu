@@ -58,6 +58,7 @@ struct esmm_grid {
     esmm_params prm;
     cudaStream_t st;
     cudaStream_t own_st;             // stream created by the library (batches without one)
+    SideStream side;                 // the second sweep direction
     int has_state;
     int xdot_zero;
     // state y^n = (cons, J, x), mesh velocity, stage buffers
@@ -258,13 +259,13 @@ long long dom_blocks(const esmm_grid *g, const Geom &G, int kind)
 }
 
 // The 2D RHD flux variant of both sweep directions (esmm_params.sweep):
-// the fused kernel (tx = -1 in the interface domains, 128 threads = 4 lines
+// the fused kernel (tx = -1 in the interface domains, a line per warp, up to 4
 // per block) or the pair and interface kernels (flat runs of 128 sites);
 // ESMM_SWEEP_AUTO starts from the fused kernel until the tuner decides.
 void set_sweep(esmm_grid *g, int sweep)
 {
     for (int k : {D_TPAIR0, D_TPAIR1, D_TIFACE0, D_TIFACE1}) {
-        g->bs[k] = 128;
+        g->bs[k] = block_for(g->Ntot, 128, 64);
         g->tx[k] = 0;
         g->persist[k] = 0;
     }
@@ -388,38 +389,49 @@ void node(esmm_grid *g, const double *cons, const double *J, const double *x, co
         launch_node(g, dom(g, D_PAD), cons, J, x, xdot, pg_in, pg_out, g->q, exact_logs);
 }
 
+// the stream of the second sweep direction, whose buffers are its own (timed launches
+// stay in line on the grid's stream)
+cudaStream_t side_begin(esmm_grid *g)
+{
+    const bool timed = g->prof_mask & ((1 << ESMM_KIND_IFACE) | (1 << ESMM_KIND_PAIRS));
+    return g->side.begin(g->st, !timed);
+}
+
 // both sweeps of the flux kernels for the node data in g->q
 void fluxes(esmm_grid *g)
 {
     Phys ph = phys(g);
     bool f32 = g->prm.precision == ESMM_MIXED;
+    const cudaStream_t side = side_begin(g);
     for (int dir = 0; dir < 2; ++dir) {
         const bool rmhd = g->phys == ESMM_RMHD;
+        const cudaStream_t st = dir ? side : g->st;
         LaunchDom Lp = dom(g, dir == 0 ? D_TPAIR0 : D_TPAIR1);
         LaunchDom Li = dom(g, rmhd ? (dir == 0 ? D_IFACE0 : D_IFACE1) : (dir == 0 ? D_TIFACE0 : D_TIFACE1));
         if (rmhd) {   // two-point fluxes summed inside the interface kernel
             Prof pr_(g, ESMM_KIND_IFACE);
-            if (f32) launch_iface_mhd_f32(Li, ph, g->q, g->q32, g->iflux, dir, g->st);
-            else launch_iface_mhd(Li, ph, g->q, g->iflux, dir, g->st);
+            if (f32) launch_iface_mhd_f32(Li, ph, g->q, g->q32, g->iflux, dir, st);
+            else launch_iface_mhd(Li, ph, g->q, g->iflux, dir, st);
             continue;
         }
         if (Li.tx < 0) {   // the fused sweep: pair fluxes kept in shared memory
             Prof pr_(g, ESMM_KIND_IFACE);
-            if (f32) launch_sweep_f32(Li, ph, g->q, g->q32, g->iflux, dir, g->st);
-            else launch_sweep_f64(Li, ph, g->q, nullptr, g->iflux, dir, g->st);
+            if (f32) launch_sweep_f32(Li, ph, g->q, g->q32, g->iflux, dir, st);
+            else launch_sweep_f64(Li, ph, g->q, nullptr, g->iflux, dir, st);
             continue;
         }
         {
             Prof pr_(g, ESMM_KIND_PAIRS);
-            if (f32) launch_pairs_f32(Lp, ph, g->q, g->q32, g->pairs, dir, g->st);
-            else launch_pairs_f64(Lp, ph, g->q, nullptr, g->pairs, dir, g->st);
+            if (f32) launch_pairs_f32(Lp, ph, g->q, g->q32, g->pairs, dir, st);
+            else launch_pairs_f64(Lp, ph, g->q, nullptr, g->pairs, dir, st);
         }
         {
             Prof pr_(g, ESMM_KIND_IFACE);
-            if (f32) launch_iface_f32(Li, ph, g->q, g->q32, g->pairs, g->iflux, dir, g->st);
-            else launch_iface_f64(Li, ph, g->q, nullptr, g->pairs, g->iflux, dir, g->st);
+            if (f32) launch_iface_f32(Li, ph, g->q, g->q32, g->pairs, g->iflux, dir, st);
+            else launch_iface_f64(Li, ph, g->q, nullptr, g->pairs, g->iflux, dir, st);
         }
     }
+    g->side.end(g->st, side);
 }
 
 void update(esmm_grid *g, double *dcons, double *dJ, const double *cn, const double *Jn, const double *xn,
@@ -748,6 +760,7 @@ void free_all(esmm_grid *g)
     for (double **b : abufs)
         if (*b) { cudaFree(*b); *b = nullptr; }
     if (g->own_st) { cudaStreamDestroy(g->own_st); g->own_st = nullptr; }
+    g->side.destroy();
     g->pairs = g->iflux = nullptr;
     g->red = nullptr;
     g->status = nullptr;
@@ -828,6 +841,10 @@ int create(esmm_grid **out, int nprob, const int *n, const double *lo, const dou
     }
     g->nprob = nprob;
     g->st = (cudaStream_t)stream;
+    if (!g->side.create()) {
+        release(g);
+        return ESMM_ERR_CUDA;
+    }
     if (!stream && own_stream) {
         if (cudaStreamCreateWithFlags(&g->own_st, cudaStreamNonBlocking) != cudaSuccess) {
             release(g);
@@ -877,7 +894,9 @@ int create(esmm_grid **out, int nprob, const int *n, const double *lo, const dou
     g->prm.move_mesh = 1;
     g->prm.precision = ESMM_FP64;
     for (int k = 0; k < ND; ++k) {
-        g->bs[k] = ((k >= D_PAIR0 && k <= D_IFACE1) || k >= D_TPAIR0) ? 128 : BS;
+        const bool flux = (k >= D_PAIR0 && k <= D_IFACE1) || (k >= D_TPAIR0 && k <= D_TIFACE1);
+        // (the node domains' partial results are sized for 64 threads or more)
+        g->bs[k] = k == D_MTILE ? BS : block_for(g->Ntot, flux ? 128 : BS, 64);
         g->tx[k] = 0;
         g->persist[k] = 0;
     }
@@ -1337,21 +1356,24 @@ int rhs_vjp_core(esmm_grid *g, const double *cons, const double *J, const double
         CK(cudaMemsetAsync(g->adjG, 0, ADJ_LAMQ_PER_NODE * P * d, g->st));
         CK(cudaMemsetAsync(lam, 0, 8 * N * d, g->st));
         Phys ph = phys(g);
+        const cudaStream_t side = side_begin(g);
         for (int dir = 0; dir < 2; ++dir) {
             const LaunchDom Li = dom(g, dir ? D_IFACE1 : D_IFACE0);
+            const cudaStream_t st = dir ? side : g->st;
             {
                 Prof pr_(g, ESMM_KIND_IFACE);   // the Powell term needs div B~
-                launch_bflux_mhd(Li, ph, g->q, (double *)g->iflux, dir, g->st);
+                launch_bflux_mhd(Li, ph, g->q, (double *)g->iflux, dir, st);
             }
             {
                 Prof pr_(g, ESMM_KIND_PAIRS);
-                launch_pairs_vjp_mhd(dom(g, dir ? D_PAIR1 : D_PAIR0), ph, g->q, mu, g->adjG, dir, g->st);
+                launch_pairs_vjp_mhd(dom(g, dir ? D_PAIR1 : D_PAIR0), ph, g->q, mu, g->adjG, dir, st);
             }
             if (g->w > 0) {
                 Prof pr_(g, ESMM_KIND_IFACE);
-                launch_iface_vjp_mhd(Li, ph, g->q, mu, g->adjG, dir, g->st);
+                launch_iface_vjp_mhd(Li, ph, g->q, mu, g->adjG, dir, st);
             }
         }
+        g->side.end(g->st, side);
         {
             Prof pr_(g, ESMM_KIND_NODE);
             launch_node_vjp_mhd(dom(g, D_PAD), g->gamma, g->q, g->adjG, (const double *)g->iflux, mu, J, lam,
@@ -1363,16 +1385,19 @@ int rhs_vjp_core(esmm_grid *g, const double *cons, const double *J, const double
     // (the pair and interface passes write every contribution the node pass reads)
     CK(cudaMemsetAsync(lam, 0, 4 * N * d, g->st));
     Phys ph = phys(g);
+    const cudaStream_t side = side_begin(g);
     for (int dir = 0; dir < 2; ++dir) {
+        const cudaStream_t st = dir ? side : g->st;
         {
             Prof pr_(g, ESMM_KIND_PAIRS);
-            launch_pairs_vjp(dom(g, dir ? D_PAIR1 : D_PAIR0), ph, g->q, mu, g->adjGp, dir, g->st);
+            launch_pairs_vjp(dom(g, dir ? D_PAIR1 : D_PAIR0), ph, g->q, mu, g->adjGp, dir, st);
         }
         if (g->w > 0) {
             Prof pr_(g, ESMM_KIND_IFACE);
-            launch_iface_vjp(dom(g, dir ? D_IFACE1 : D_IFACE0), ph, g->q, mu, g->adjG, dir, g->st);
+            launch_iface_vjp(dom(g, dir ? D_IFACE1 : D_IFACE0), ph, g->q, mu, g->adjG, dir, st);
         }
     }
+    g->side.end(g->st, side);
     {
         Prof pr_(g, ESMM_KIND_NODE);
         launch_node_vjp(dom(g, D_PAD), g->gamma, g->p, g->w, g->q, g->adjG, g->adjGp, J, lam, g->st);

@@ -11,6 +11,57 @@
 
 namespace esmm {
 
+// Threads per block of a launch over n sites: the largest size that leaves every SM about
+// four blocks, so that a small grid reaches the whole chip and the last round of blocks is
+// short (each quarter of an SM has its own FP64 pipe, at 76 cycles a warp instruction: a
+// warp too many on one is time lost).  The line: 4 blocks an SM of the larger size; below
+// it 64 threads win (64^2 steps 1.67 -> 1.52 ms, a 160^2 RMHD step 0.91 -> 0.77 ms, both with
+// the flux launches in line), above it they are equal (400^2 mixed 1.166, 1.162 ms).
+constexpr int CHIP_SMS = 152;
+inline int block_for(long long n, int most, int least)
+{
+    int bs = most;
+    while (bs > least && n < 4LL * CHIP_SMS * bs) bs /= 2;
+    return bs;
+}
+
+// A second stream for launches without an order between them: begin() orders it after
+// everything on st and gives the stream to use, end() orders st after it (both also while
+// st is being captured).  The second sweep direction of a grid takes it, as one alone
+// would leave FP64 pipes idle at its start or end: 64^2 steps 1.66 -> 1.15 ms, two recorded
+// 96^2 RMHD steps and their gradient 12.7 -> 7.4 ms, a 64^3 blast step 20.6 -> 19.7 ms, 400^2
+// steps 4.22 -> 4.18 ms (with block_for); no size was slower, so there is no line.
+struct SideStream {
+    cudaStream_t s;
+    cudaEvent_t from, to;
+    bool create()
+    {
+        return cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess &&
+               cudaEventCreateWithFlags(&from, cudaEventDisableTiming) == cudaSuccess &&
+               cudaEventCreateWithFlags(&to, cudaEventDisableTiming) == cudaSuccess;
+    }
+    void destroy()
+    {
+        if (s) cudaStreamDestroy(s);
+        if (from) cudaEventDestroy(from);
+        if (to) cudaEventDestroy(to);
+        s = nullptr;
+        from = to = nullptr;
+    }
+    cudaStream_t begin(cudaStream_t st, bool use)
+    {
+        if (!use || !s || cudaEventRecord(from, st) != cudaSuccess || cudaStreamWaitEvent(s, from, 0) != cudaSuccess)
+            return st;
+        return s;
+    }
+    void end(cudaStream_t st, cudaStream_t used)
+    {
+        if (used == st) return;
+        if (cudaEventRecord(to, used) != cudaSuccess || cudaStreamWaitEvent(st, to, 0) != cudaSuccess)
+            cudaStreamSynchronize(used);
+    }
+};
+
 // Launch domain of one kernel: the problem addressing and the grid shape.
 // The RHD flux kernels also take a tile shape (tx threads along x_1 by
 // bs / tx along x_2; 0: one flat run of sites along the sweep) and the
