@@ -29,6 +29,7 @@ namespace d3 {
 // M[k][j] = delta_{k2}[delta_{k1}[x_{j1}] x_{j2}] - delta_{k1}[delta_{k2}[x_{j1}] x_{j2}]
 // from those values at +-n along k2 and k1 (eq. SCLCoeff's nested central
 // differences, evaluated once per difference instead of once per use).
+constexpr int BS3 = 128;   // threads per block of the node kernels
 constexpr int HE = GH + PMAX;
 constexpr int NXE = 12;
 
@@ -216,7 +217,7 @@ __global__ void k3_update(Geom3 g, const double *__restrict__ q, const double *_
 // static spectral radius per direction (eq. cfl); with cflb (the moving-mesh
 // step) also the speed bounds L_k lambda_min/J and L_k lambda_max/J of every
 // node into its rows 3 + d and 6 + d
-__global__ void k3_cfl(Geom3 g, double gam, const double *__restrict__ q, const double *__restrict__ J,
+__global__ void __launch_bounds__(BS3, 4) k3_cfl(Geom3 g, double gam, const double *__restrict__ q, const double *__restrict__ J,
                        unsigned long long *red, double *__restrict__ cflb)
 {
     long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -224,15 +225,16 @@ __global__ void k3_cfl(Geom3 g, double gam, const double *__restrict__ q, const 
     if (id < g.N) {
         int i = (int)(id % g.n[0]), j = (int)((id / g.n[0]) % g.n[1]), k = (int)(id / ((long long)g.n[0] * g.n[1]));
         long long c = pidx3(g, i, j, k);
-        double iW = 1.0 / q[F_W * g.P + c];
+        const double iW = qrcp<double>(q[F_W * g.P + c]);
         double w[8] = {q[F_RHO * g.P + c], q[F_U0 * g.P + c] * iW, q[F_U1 * g.P + c] * iW, q[F_U2 * g.P + c] * iW,
                        q[F_P * g.P + c], q[F_B0 * g.P + c], q[F_B1 * g.P + c], q[F_B2 * g.P + c]};
-        double iJ = 1.0 / J[id];
+        const double iJ = 1.0 / J[id];
+#pragma unroll 1
         for (int d = 0; d < 3; ++d) {
             double m[3];
             for (int a = 0; a < 3; ++a) m[a] = q[(F_M + 3 * d + a) * g.P + c];
-            double Lk = sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
-            double nn[3] = {m[0] / Lk, m[1] / Lk, m[2] / Lk}, T[3][3], wr[8], lo, hi;
+            const double l2 = m[0] * m[0] + m[1] * m[1] + m[2] * m[2], iLk = qrsq<double>(l2), Lk = l2 * iLk;
+            double nn[3] = {m[0] * iLk, m[1] * iLk, m[2] * iLk}, T[3][3], wr[8], lo, hi;
             frame3(nn, T);
             rot3(T, w, wr);
             mhd_speed_range<double>(gam, wr, lo, hi);
@@ -555,7 +557,6 @@ struct esmm3 {
 
 namespace {
 
-constexpr int BS3 = 128;
 inline unsigned nb3(long long n, int bs = BS3) { return (unsigned)((n + bs - 1) / bs); }
 
 int fail3(esmm3 *g, int code, const char *what, cudaError_t e = cudaSuccess)

@@ -298,18 +298,19 @@ __global__ void k_cfl(ProbArg pa, double gam, double gg, const double *__restric
         int i = (int)(id % g.nx), j = (int)(id / g.nx);
         long long c = pidx(g, i, j);
         double rho = q[Q_RHO * g.P + c], p = q[Q_P * g.P + c], W = q[Q_W * g.P + c];
-        double iW = __drcp_rn(W);
+        const double iW = qrcp<double>(W);
         double vx = q[Q_UX * g.P + c] * iW, vy = q[Q_UY * g.P + c] * iW;
         double v2 = vx * vx + vy * vy;
         double rh = rho + p * gg;
-        double c2 = gam * p * __drcp_rn(rh), cs = sqrt(c2);
+        const double c2 = gam * p * qrcp<double>(rh), cs = c2 * qrsq<double>(c2);
         double iJ = __drcp_rn(J[id]);
-        const double iden = __drcp_rn(1.0 - v2 * c2);   // the same for both directions
+        const double iden = qrcp<double>(1.0 - v2 * c2);   // the same for both directions
+#pragma unroll
         for (int k = 0; k < 2; ++k) {
             double mx = q[(Q_M00 + 2 * k) * g.P + c], my = q[(Q_M01 + 2 * k) * g.P + c];
-            const double n2 = mx * mx + my * my, iL = rsqrt(n2), Lk = n2 * iL;
+            const double n2 = mx * mx + my * my, iL = qrsq<double>(n2), Lk = n2 * iL;
             double vn = (mx * vx + my * vy) * iL;
-            double disc = sqrt((1.0 - v2) * (1.0 - v2 * c2 - vn * vn * (1.0 - c2)));
+            const double d2 = (1.0 - v2) * (1.0 - v2 * c2 - vn * vn * (1.0 - c2)), disc = d2 * qrsq<double>(d2);
             double lm = (vn * (1.0 - c2) - cs * disc) * iden, lp = (vn * (1.0 - c2) + cs * disc) * iden;
             r[k] = owned_row(g, j) ? Lk * fmax(fabs(lm), fabs(lp)) * iJ : 0.0;
             if (cflb) {

@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 2) k_cfl_mhd(ProbArg
         double w[8] = {q[Q_RHO * g.P + c], q[Q_UX * g.P + c] * iW, q[Q_UY * g.P + c] * iW,
                        q[QM_UZ * g.P + c] * iW, q[Q_P * g.P + c], q[QM_B1 * g.P + c], q[QM_B2 * g.P + c],
                        q[QM_B3 * g.P + c]};
-        const double iJ = qrcp<double>(J[id]);
+        const double iJ = 1.0 / J[id];
 #pragma unroll 1
         for (int k = 0; k < 2; ++k) {
             double mx = q[(Q_M00 + 2 * k) * g.P + c], my = q[(Q_M01 + 2 * k) * g.P + c];

@@ -1347,7 +1347,7 @@ __global__ void k_update_mhd(ProbArg pa, const double *__restrict__ q, const R *
         L[a] = -(d0 + d1);
     }
     // Powell source: L[9] = -div B~ here
-    double iW = 1.0 / q[Q_W * g.P + c];
+    const double iW = qrcp<double>(q[Q_W * g.P + c]);
     double w[8];
     w[1] = q[Q_UX * g.P + c] * iW;
     w[2] = q[Q_UY * g.P + c] * iW;
@@ -1358,7 +1358,7 @@ __global__ void k_update_mhd(ProbArg pa, const double *__restrict__ q, const R *
     double Pp[8];
     mhd_phiprime(w, Pp);
 #pragma unroll
-    for (int a = 0; a < 8; ++a) L[a] += Pp[a] * L[9];
+    for (int a = 1; a < 8; ++a) L[a] += Pp[a] * L[9];   // (Phi'_1 = 0)
     if (dcons) {
 #pragma unroll
         for (int a = 0; a < 8; ++a) dcons[a * g.N + id] = L[a];
