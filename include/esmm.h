@@ -66,9 +66,9 @@ extern "C" {
 #define ESMM_MEM_DEVICE 1
 
 #define ESMM_FP64 0         /* every step in FP64                              */
-#define ESMM_MIXED 1        /* fluxes, WENO and metrics in FP32; FP64 for the
-                               primitive recovery, near-equal log means, the
-                               state, and all totals                            */
+#define ESMM_MIXED 1        /* fluxes, WENO and metrics in FP32 (log means' jumps
+                               from FP64 values); FP64 for the primitive
+                               recovery, the state, and all totals              */
 
 #define ESMM_MONITOR_RHO 0  /* monitor variable sigma = rho                    */
 #define ESMM_MONITOR_LNRHO 1/* monitor variable sigma = ln rho                 */

@@ -465,9 +465,8 @@ void step_radius(esmm_grid *g, double dt, bool moving)
     Prof pr_(g, ESMM_KIND_OTHER);
     LaunchDom L = dom(g, D_NODE);
     double *cflb = moving ? g->cflb : nullptr;
-    if (g->phys == ESMM_RMHD)   // at most 256 threads per block, whatever the node kind's tuned size: the
-                                // eigen-system holds up to 255 registers per thread (RMHD grids are single
-                                // problems)
+    if (g->phys == ESMM_RMHD)   // at most 256 threads per block (its launch bounds), whatever the node
+                                // kind's tuned size (RMHD grids are single problems)
         launch_cfl_mhd(dom_one(g, 0, D_NODE, std::min(L.bs, 256)), g->gamma, g->q, g->J, g->red,
                        g->prm.precision == ESMM_MIXED, cflb, g->st);
     else
@@ -1339,7 +1338,7 @@ int adj_alloc(esmm_grid *g)
 {
     size_t P = (size_t)g->Ptot, N = (size_t)g->Ntot, d = sizeof(double);
     if (!g->adjG) CK(cudaMalloc((void **)&g->adjG, ADJ_G_PER_NODE * P * d));
-    if (!g->adjGp) CK(cudaMalloc((void **)&g->adjGp, ADJ_GP_PER_NODE * P * d));
+    if (!g->adjGp && g->phys == ESMM_RHD) CK(cudaMalloc((void **)&g->adjGp, ADJ_GP_PER_NODE * P * d));
     double **bufs[] = {&g->lam_a, &g->lam_b, &g->lam_c, &g->lam_v};
     for (double **b : bufs)
         if (!*b) CK(cudaMalloc((void **)b, (size_t)g->nv * N * d));

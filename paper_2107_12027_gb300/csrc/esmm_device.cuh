@@ -1,7 +1,8 @@
 // esmm_device.cuh -- device arithmetic of the ES adaptive moving-mesh scheme
 // (Duan & Tang, arXiv 2107.12027), 2D RHD, templated on the working precision
 // R (double for the FP64 form, float for the mixed form).  The primitive
-// recovery is always FP64, and so are the jumps of the logarithmic mean.
+// recovery is always FP64; the jumps of the logarithmic mean are formed in FP64, or in
+// FP32 from values carried with their FP64 rest (LmV).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -187,7 +188,7 @@ __device__ __forceinline__ double mesh_at(const Geom &g, const double *a, int i,
 // Dual number a + b eps (eps^2 = 0): the flux arithmetic below is templated on
 // its working type, and evaluating it on duals seeded at one input gives the
 // derivative of every output with respect to that input.  The adjoint kernels
-// use this for the local (per pair / per interface) Jacobian-vector products.
+// use this for the interface state and for the second derivatives of (U, V, F).
 struct dual {
     double v, d;
     __host__ __device__ dual() {}

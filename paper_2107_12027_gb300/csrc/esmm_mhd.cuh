@@ -281,7 +281,8 @@ __device__ __forceinline__ void mhd_phiprime(const R w[8], R P[8])
 // their span (Gram-Schmidt, in index order, of the projected C-space unit
 // vectors whose remaining squared norm is at least 1/8: continuous in the
 // span, unlike a largest-norm choice, which switches on the exact ties of
-// symmetric states).
+// symmetric states).  eigen_mhd_gram builds them so; the flux kernels take the same waves
+// in closed form (eigen_mhd, es_dissipation_mhd).
 constexpr double MHD_CLUSTER_TOL = 1.0e-5;
 
 // Cyclic Jacobi on the symmetric 6 x 6 C (in place: its diagonal becomes the
@@ -1086,9 +1087,8 @@ __global__ void __maxnreg__(64) k_node_mhd(ProbArg pa, double gam, const double 
     q[Q_UY * g.P + t] = W * w[2];
     q[QM_UZ * g.P + t] = W * w[3];
     q[Q_W * g.P + t] = W;
-    // (f32_logs: the mixed form's scheme passes, where the logarithms enter
-    // only FP32 arithmetic and the log mean's jump outside its near-equal
-    // branch)
+    // (f32_logs: the mixed form's scheme passes, where the logarithms enter only FP32
+    // arithmetic)
     float lr32 = 0.0f, lb32 = 0.0f;
     if (f32_logs) {
         lr32 = logf(d2f_int(w[0]));

@@ -1,5 +1,5 @@
 // esmm_mhd_f32.cu -- the RMHD interface and update kernels instantiated for
-// the FP32 bulk form (FP64 recovery, near-equal log means and state).
+// the FP32 bulk form (FP64 recovery, magnetic and metric fluxes, and state).
 #include "esmm_launch.h"
 #include "esmm_mhd.cuh"
 
