@@ -282,7 +282,7 @@ __device__ __forceinline__ void mhd_phiprime(const R w[8], R P[8])
 // vectors whose remaining squared norm is at least 1/8: continuous in the
 // span, unlike a largest-norm choice, which switches on the exact ties of
 // symmetric states).  eigen_mhd_gram builds them so; the flux kernels take the same waves
-// in closed form (eigen_mhd, es_dissipation_mhd).
+// in closed form (es_dissipation_mhd).
 constexpr double MHD_CLUSTER_TOL = 1.0e-5;
 
 // Cyclic Jacobi on the symmetric 6 x 6 C (in place: its diagonal becomes the
@@ -548,161 +548,6 @@ static __device__ __noinline__ void eigen_mhd_gram(double gam, const R w[8], R l
 
 namespace esmm {
 
-// The canonical basis of the clusters (consecutive speeds closer than
-// MHD_CLUSTER_TOL) among the six waves, whose columns of Rv it replaces: with
-// G = L L^T the Gram matrix of the y_a of eigen_mhd_gram and S[a][m] the wave
-// m's coefficients in them, E = L^T S are the waves in C-space; the basis is the
-// Gram-Schmidt of the unit vectors projected on the cluster's span, as there.
-template <typename R>
-static __device__ __noinline__ void mhd_canonical(double gam, const R w[8], const R lam[8], R S[6][6], R Rv[8][8])
-{
-    R Pp[8];
-    mhd_phiprime(w, Pp);
-    const R v1 = w[1];
-    R a_rho[8] = {(R)1, (R)0, (R)0, (R)0, (R)0, (R)0, (R)0, (R)0};
-    R a_div[8] = {(R)0, (R)0, (R)0, (R)0, (R)0, (R)1 - v1 * v1, -v1 * w[2], -v1 * w[3]};
-    R Ur[8], Vr[8], Ud[8], Vd[8], Fx[8];
-    mhd_images(gam, w, a_rho, Pp, Ur, Vr, Fx);
-    mhd_images(gam, w, a_div, Pp, Ud, Vd, Fx);
-    const R in_rho = rcp<R>(dot8(Ur, Vr)), in_div = rcp<R>(dot8(Ud, Vd));
-    const int comp[6] = {1, 2, 3, 4, 6, 7};
-    R Uy[6][8], Vy[6][8], Gm[6][6], idg[6];
-#pragma unroll 1
-    for (int a = 0; a < 6; ++a) {
-        R e[8] = {(R)0, (R)0, (R)0, (R)0, (R)0, (R)0, (R)0, (R)0};
-        e[comp[a]] = (R)1;
-        R Ue[8], Ve[8];
-        mhd_images(gam, w, e, Pp, Ue, Ve, Fx);
-        const R cr = dot8(Ue, Vr) * in_rho, cd = dot8(Ue, Vd) * in_div;
-        for (int r = 0; r < 8; ++r) {
-            Uy[a][r] = Ue[r] - cr * Ur[r] - cd * Ud[r];
-            Vy[a][r] = Ve[r] - cr * Vr[r] - cd * Vd[r];
-        }
-        // y_a of unit <y_a, y_a> (E is unchanged by the scaling)
-        const R sa = rsq<R>(dot8(Uy[a], Vy[a])), isa = rcp<R>(sa);
-        for (int r = 0; r < 8; ++r) {
-            Uy[a][r] *= sa;
-            Vy[a][r] *= sa;
-        }
-        for (int m = 0; m < 6; ++m) S[a][m] *= isa;
-    }
-    for (int a = 0; a < 6; ++a)
-        for (int b = 0; b <= a; ++b) Gm[a][b] = (R)0.5 * (dot8(Uy[a], Vy[b]) + dot8(Uy[b], Vy[a]));
-    for (int j = 0; j < 6; ++j) {
-        R d = Gm[j][j];
-        for (int k = 0; k < j; ++k) d -= Gm[j][k] * Gm[j][k];
-        if constexpr (sizeof(R) == 4)
-            if (!(d > (R)1.0e-12)) d = (R)1.0e-12;   // FP32: keep the factor finite
-        idg[j] = rsq<R>(d);
-        Gm[j][j] = d * idg[j];
-        for (int i = j + 1; i < 6; ++i) {
-            R s = Gm[i][j];
-            for (int k = 0; k < j; ++k) s -= Gm[i][k] * Gm[j][k];
-            Gm[i][j] = s * idg[j];
-        }
-    }
-    int start = 0;
-    while (start < 6) {
-        int end = start + 1;
-        while (end < 6 && mhd_close<R>(lam[1 + end], lam[2 + end])) ++end;
-        const int k = end - start;
-        if (k > 1) {
-            // E = L^T S, orthonormalized (twice: the waves of a cluster may be
-            // oblique at rounding level over their gap)
-            R E[6][6], z[6][6];
-            for (int c = 0; c < k; ++c) {
-                for (int i = 0; i < 6; ++i) {
-                    R acc = (R)0;
-                    for (int j = i; j < 6; ++j) acc += Gm[j][i] * S[j][start + c];
-                    E[i][c] = acc;
-                }
-                for (int pass = 0; pass < 2; ++pass)
-                    for (int b = 0; b < c; ++b) {
-                        R pr = (R)0;
-                        for (int i = 0; i < 6; ++i) pr += E[i][b] * E[i][c];
-                        for (int i = 0; i < 6; ++i) E[i][c] -= pr * E[i][b];
-                    }
-                R n2 = (R)0;
-                for (int i = 0; i < 6; ++i) n2 += E[i][c] * E[i][c];
-                const R inr = rsq<R>(n2);
-                for (int i = 0; i < 6; ++i) E[i][c] *= inr;
-            }
-            R basis[6][6];
-            for (int i = 0; i < 6; ++i)
-                for (int c = 0; c < k; ++c) z[i][c] = E[i][c];
-            int nt = 0;
-            for (int i = 0; i < 6 && nt < k; ++i) {
-                R n2 = (R)0;
-                for (int c = 0; c < k; ++c) n2 += z[i][c] * z[i][c];
-                if (!(n2 >= (R)0.125)) continue;
-                const R inr = rsq<R>(n2);
-                for (int c = 0; c < k; ++c) basis[nt][c] = z[i][c] * inr;
-                for (int ii = i + 1; ii < 6; ++ii) {
-                    R pr = (R)0;
-                    for (int c = 0; c < k; ++c) pr += z[ii][c] * basis[nt][c];
-                    for (int c = 0; c < k; ++c) z[ii][c] -= pr * basis[nt][c];
-                }
-                ++nt;
-            }
-            for (int t = 0; t < nt && nt == k; ++t) {   // (nt < k: non-finite input)
-                R s[6];
-                for (int i = 5; i >= 0; --i) {
-                    R acc = (R)0;
-                    for (int c = 0; c < k; ++c) acc += E[i][c] * basis[t][c];
-                    for (int j = i + 1; j < 6; ++j) acc -= Gm[j][i] * s[j];
-                    s[i] = acc * idg[i];
-                }
-                for (int r = 0; r < 8; ++r) {
-                    R acc = (R)0;
-                    for (int a = 0; a < 6; ++a) acc += s[a] * Uy[a][r];
-                    Rv[r][2 + start + t] = acc;
-                }
-            }
-        }
-        start = end;
-    }
-}
-
-// The eigen-system of eigen_mhd_gram from the waves in closed form
-// (esmm_mhd_waves.cuh); clusters get their canonical basis, and states whose
-// coefficients leave the FP32 range of the root estimates take the Gram path.
-template <typename R>
-static __device__ __noinline__ void eigen_mhd(double gam, const R w[8], R lam[8], R Rv[8][8])
-{
-    const R gg = (R)(gam / (gam - 1.0));
-    MhdBase<R> s;
-    mhd_base<R>((R)gam, gg, w, s);
-    if (!mhd_in_range<R>(s)) {
-        eigen_mhd_gram<R>(gam, w, lam, Rv, true);
-        return;
-    }
-    MhdSix<R> x;
-    lam[0] = lam[1] = s.v1;
-    mhd_six<R>(s, x, lam + 2);
-    bool cluster = false;
-#pragma unroll
-    for (int m = 0; m < 5; ++m) cluster = cluster || mhd_close<R>(lam[2 + m], lam[3 + m]);
-    R dU[8];
-    mhd_entropy_dU<R>(s, (R)((gam - 1.0) / gam), dU);
-    for (int r = 0; r < 8; ++r) Rv[r][0] = dU[r];
-    mhd_divergence_dU<R>(s, dU);
-    for (int r = 0; r < 8; ++r) Rv[r][1] = dU[r];
-    R S[6][6];
-#pragma unroll 1
-    for (int m = 0; m < 6; ++m) {
-        MhdWave<R> q;
-        mhd_six_wave<R, false>(s, x, gg, m, q, dU);
-        for (int r = 0; r < 8; ++r) Rv[r][2 + m] = dU[r];
-        if (cluster) {   // the wave's coefficients in the y_a
-            for (int k = 0; k < 3; ++k) S[k][m] = (q.u[1 + k] - w[1 + k] * q.u[0]) * s.iW;
-            S[3][m] = q.p;
-            const R ga = -dU[5] * rcp<R>((R)1 - s.v1 * s.v1);
-            S[4][m] = dU[6] - ga * s.v1 * w[2];
-            S[5][m] = dU[7] - ga * s.v1 * w[3];
-        }
-    }
-    if (cluster) mhd_canonical<R>(gam, w, lam, S, Rv);
-}
 // the smallest and largest speed (the fast waves) at the rotated state w: the
 // CFL radius needs no vectors
 template <typename R>
@@ -726,7 +571,7 @@ static __device__ __noinline__ void mhd_speed_range(double gam, const R w[8], R 
     hi = s.v1 + tf * s.iW;
 }
 
-// The canonical basis (mhd_canonical) of a cluster of two waves a, b of one side, an
+// The canonical basis (see eigen_mhd_gram) of a cluster of two waves a, b of one side, an
 // Alfven and a magnetosonic one: they are orthogonal whatever their speeds (s is normal to
 // t, k and b), so a rotation of the two columns is all that is needed, and its first
 // vector is the first row (E[i][a], E[i][b]) of E = L^T S whose squared norm is at least
@@ -734,8 +579,8 @@ static __device__ __noinline__ void mhd_speed_range(double gam, const R w[8], R 
 // e_0 or e_1 (v_1, v_2) nearly always decides: e_{v_k} in closed form,
 //   du = (W u_k, e_k + u_k u) (times W), db from B = const,  dV = beta (0, du, -du^0, db),
 // with <e_i, a> = dV(e_i).R_a, and <e_i, e_j> from the bilinear form X^0.  Returns false
-// where neither row decides.  (~150 operations, against ~3,500 of eigen_mhd and the whole
-// Gram matrix: a rotor's ambient field along x_1 leaves clusters in half the interfaces
+// where neither row decides.  (~150 operations, against ~1,000 with the whole Gram
+// matrix: a rotor's ambient field along x_1 leaves clusters in half the interfaces
 // of that sweep.)  Rv: rows dU of the waves, rows 0 and 1 the entropy and divergence waves.
 template <typename R>
 __device__ __forceinline__ bool mhd_turn_pair(const MhdBase<R> &s, const R B[3], R Rv[8][8], int a)
@@ -798,6 +643,174 @@ __device__ __forceinline__ bool mhd_turn_pair(const MhdBase<R> &s, const R B[3],
     return true;
 }
 
+// The canonical basis of every cluster among the six waves (bit m of near: waves m and m + 1
+// are in one), whose rows dU of Rv it replaces: with the directions e_i = v_1, v_2, v_3 (times
+// 1/W), p, B_2, B_3 in closed form (as in mhd_turn_pair; p: du = db = 0, dV = -(beta/p)
+// (1 + 1/((Gamma-1) beta), u, -W, b); B_k: db = e_k/W + u_k (1, u/W), dV = beta (0, 0, 0, db)), their
+// Gram matrix G = L L^T off the entropy and divergence waves and S[i][m] the wave m's
+// coefficients in the e_i, the waves in C-space are E = L^T S; each cluster is orthonormalized there (twice: its waves
+// may be oblique at rounding level over their gap) and takes the Gram-Schmidt of the
+// unit vectors projected on its span, both as a matrix on its rows of Rv.  ~1,000
+// FP64 instructions, against ~3,500 with the images on dual numbers and the waves formed
+// anew; four waves of one speed are the rule where B_n = 0.  Measured: the untapered 512^2
+// rotor step 16.1 -> 13.4 ms, mixed 2.36 -> 1.94 ms, a 64^3 blast step at rest 29.4 -> 23.2 ms,
+// a 64^3 step of gas without a field 36.7 -> 27.6 ms.
+template <typename R>
+static __device__ __noinline__ void mhd_turn_clusters(const MhdBase<R> &s, R ig, const R B[3], R S[6][6], R Rv[8][8],
+                                                          int near)
+{
+    R du[3][4], db[5][4], P[5], f0[6], f1[6], G[6][6], E[6][6];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        if (k < 3) {
+            const R uk = s.u[1 + k];
+            du[k][0] = s.W * uk;
+#pragma unroll
+            for (int q = 1; q < 4; ++q) du[k][q] = (q == 1 + k ? (R)1 : (R)0) + s.u[q] * uk;
+            db[k][0] = du[k][1] * B[0] + du[k][2] * B[1] + du[k][3] * B[2];
+#pragma unroll
+            for (int q = 1; q < 4; ++q) db[k][q] = (db[k][0] * s.u[q] + s.b[0] * du[k][q] - s.b[q] * du[k][0]) * s.iW;
+        } else {   // B_2, B_3
+            const R uk = s.u[k - 1];
+            db[k][0] = uk;
+#pragma unroll
+            for (int q = 1; q < 4; ++q) db[k][q] = ((q == k - 1 ? (R)1 : (R)0) + uk * s.u[q]) * s.iW;
+        }
+        P[k] = mdot<R>(s.b, db[k]);
+    }
+    // <e_i, .> over beta with the entropy and the divergence wave (index of db: v 0..2, B 3,
+    // 4; of f0: v 0..2, p 3, B 4, 5)
+    const R cp = (R)1 + ig * rcp<R>(s.beta);
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+        const R *r = Rv[m];
+        R *f = m == 0 ? f0 : f1;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            R acc = db[k][1] * r[5] + db[k][2] * r[6] + db[k][3] * r[7];
+            if (k < 3) acc += du[k][1] * r[1] + du[k][2] * r[2] + du[k][3] * r[3] - du[k][0] * r[4];
+            f[k < 3 ? k : k + 1] = acc;
+        }
+        f[3] = -s.ip * (cp * r[0] + s.u[1] * r[1] + s.u[2] * r[2] + s.u[3] * r[3] - s.W * r[4] + s.b[1] * r[5] + s.b[2] * r[6] +
+                        s.b[3] * r[7]);
+    }
+    // Gram entries over beta, scaled to a unit diagonal (E is unchanged by that)
+#pragma unroll
+    for (int a = 0; a < 5; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b) {
+            R g = s.W * mdot<R>(db[a], db[b]);
+            if (a < 3) {
+                g += s.W * (s.e * mdot<R>(du[a], du[b])) + du[a][0] * P[b] + du[b][0] * P[a] -
+                     s.b[0] * (mdot<R>(db[a], du[b]) + mdot<R>(db[b], du[a]));
+            } else if (b < 3) {
+                g += du[b][0] * P[a] - s.b[0] * mdot<R>(db[a], du[b]);
+            }
+            G[a < 3 ? a : a + 1][b < 3 ? b : b + 1] = g;
+        }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        G[3][k] = du[k][0];
+        if (k < 2) G[4 + k][3] = (R)0;
+    }
+    G[3][3] = s.W * s.ip * ig;   // (Gamma/(Gamma-1) - 1 = 1/(Gamma-1))
+    R sc[6];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+#pragma unroll
+        for (int b = 0; b <= a; ++b) G[a][b] -= s.beta * (f0[a] * f0[b] + f1[a] * f1[b]);
+        sc[a] = rsq<R>(G[a][a]);
+    }
+#pragma unroll
+    for (int a = 0; a < 6; ++a)
+#pragma unroll
+        for (int b = 0; b <= a; ++b) G[a][b] *= sc[a] * sc[b];
+#pragma unroll 1
+    for (int j = 0; j < 6; ++j) {
+        R d = G[j][j];
+        for (int k = 0; k < j; ++k) d -= G[j][k] * G[j][k];
+        if constexpr (sizeof(R) == 4)
+            if (!(d > (R)1.0e-12)) d = (R)1.0e-12;   // FP32: keep the factor finite
+        const R idg = rsq<R>(d);
+        G[j][j] = d * idg;
+        for (int i = j + 1; i < 6; ++i) {
+            R t = G[i][j];
+            for (int k = 0; k < j; ++k) t -= G[i][k] * G[j][k];
+            G[i][j] = t * idg;
+        }
+        sc[j] = rcp<R>(sc[j]);
+        for (int m = 0; m < 6; ++m) S[j][m] *= sc[j];
+    }
+#pragma unroll 1
+    for (int i = 0; i < 6; ++i)   // E over sqrt(beta): its columns are normalized below
+        for (int m = 0; m < 6; ++m) {
+            R t = G[i][i] * S[i][m];
+            for (int j = i + 1; j < 6; ++j) t += G[j][i] * S[j][m];
+            E[i][m] = t;
+        }
+    const R isb = rsq<R>(s.beta);
+    int start = 0;
+#pragma unroll 1
+    while (start < 6) {
+        int end = start + 1;
+        while (end < 6 && (near >> (end - 1) & 1)) ++end;
+        const int k = end - start;
+        if (k > 1) {
+            R M[6][6], basis[6][6], z[6][6];   // M: the orthonormal members (columns) from the waves
+            for (int c = 0; c < k; ++c) {
+                for (int q = 0; q < k; ++q) M[q][c] = q == c ? isb : (R)0;
+                for (int pass = 0; pass < 2; ++pass)
+                    for (int b = 0; b < c; ++b) {
+                        R pr = (R)0;
+                        for (int i = 0; i < 6; ++i) pr += E[i][start + b] * E[i][start + c];
+                        for (int i = 0; i < 6; ++i) E[i][start + c] -= pr * E[i][start + b];
+                        for (int q = 0; q < k; ++q) M[q][c] -= pr * M[q][b];
+                    }
+                R n2 = (R)0;
+                for (int i = 0; i < 6; ++i) n2 += E[i][start + c] * E[i][start + c];
+                const R inr = rsq<R>(n2);
+                for (int i = 0; i < 6; ++i) E[i][start + c] *= inr;
+                for (int q = 0; q < k; ++q) M[q][c] *= inr;
+            }
+            for (int i = 0; i < 6; ++i)
+                for (int c = 0; c < k; ++c) z[i][c] = E[i][start + c];
+            int nt = 0;
+            for (int i = 0; i < 6 && nt < k; ++i) {
+                R n2 = (R)0;
+                for (int c = 0; c < k; ++c) n2 += z[i][c] * z[i][c];
+                if (!(n2 >= (R)0.125)) continue;
+                const R inr = rsq<R>(n2);
+                for (int c = 0; c < k; ++c) basis[nt][c] = z[i][c] * inr;
+                for (int ii = i + 1; ii < 6; ++ii) {
+                    R pr = (R)0;
+                    for (int c = 0; c < k; ++c) pr += z[ii][c] * basis[nt][c];
+                    for (int c = 0; c < k; ++c) z[ii][c] -= pr * basis[nt][c];
+                }
+                ++nt;
+            }
+            if (nt == k) {   // (less: non-finite input)
+                R T[6][6];   // canonical member t = sum_q T[t][q] wave q
+                for (int t = 0; t < k; ++t)
+                    for (int q = 0; q < k; ++q) {
+                        R acc = (R)0;
+                        for (int c = 0; c < k; ++c) acc += M[q][c] * basis[t][c];
+                        T[t][q] = acc;
+                    }
+                for (int r = 0; r < 8; ++r) {
+                    R o[6];
+                    for (int t = 0; t < k; ++t) {
+                        R acc = (R)0;
+                        for (int q = 0; q < k; ++q) acc += T[t][q] * Rv[2 + start + q][r];
+                        o[t] = acc;
+                    }
+                    for (int t = 0; t < k; ++t) Rv[2 + start + t][r] = o[t];
+                }
+            }
+        }
+        start = end;
+    }
+}
+
 // The ES dissipation of one interface in its rotated frame (first axis along the
 // normal): with the interface state rho = {{rho}}^ln, u = {{u}}, p = 1/ip, B = {{B}}
 // and the scaled eigenvectors R, d = lambda^/2 R Y <<R^T V>>, lambda^ the largest |jt + Lk
@@ -805,8 +818,8 @@ __device__ __forceinline__ bool mhd_turn_pair(const MhdBase<R> &s, const R B[3],
 // stencil's node k.  The dissipation depends on differences of V alone, so those are
 // projected (w of them), and the wave's edge jump comes from them (weno5_jump); the
 // switch's tolerance, a threshold, is formed in FP32 from |R| and |V|.  Clusters of two
-// waves of one side are turned (mhd_turn_pair); interfaces with other clusters, or
-// outside the closed form's range, take their vectors from eigen_mhd.
+// waves of one side are turned by mhd_turn_pair, others by mhd_turn_clusters; states outside
+// the closed form's range take eigen_mhd_gram.
 template <typename R, int WW, typename ROTV>
 __device__ __forceinline__ void es_dissipation_mhd(const Phys &ph, R rho, R p, R ip, const R us[3], const R Bs[3], R Lk,
                                                    R jt, ROTV rotV, R d[8])
@@ -828,25 +841,35 @@ __device__ __forceinline__ void es_dissipation_mhd(const Phys &ph, R rho, R p, R
             int near = 0;   // bit m: waves m and m + 1 in one cluster
 #pragma unroll
             for (int m = 0; m < 5; ++m) near |= (int)mhd_close<R>(l6[m], l6[m + 1]) << m;
-            whole = (near & 4) != 0 || (near & (near >> 1)) != 0;   // slow waves of both sides, or three and more
-            if (!whole) {
-                mhd_entropy_dU<R>(s, (R)ph.igg, Rv[0]);
-                mhd_divergence_dU<R>(s, Rv[1]);
+            R S[6][6];
+            mhd_entropy_dU<R>(s, (R)ph.igg, Rv[0]);
+            mhd_divergence_dU<R>(s, Rv[1]);
 #pragma unroll 1
-                for (int m = 0; m < 6; ++m) {
-                    MhdWave<R> q;
-                    mhd_six_wave<R, false>(s, x, gg, m, q, Rv[2 + m]);
+            for (int m = 0; m < 6; ++m) {
+                MhdWave<R> q;
+                mhd_six_wave<R, false>(s, x, gg, m, q, Rv[2 + m]);
+                if (near) {
+                    const R *r = Rv[2 + m], ga = -s.v1 * r[5] * qrcp<R>((R)1 - s.v1 * s.v1) * s.iW, d0 = q.u[0] * s.iW;
+                    for (int k = 0; k < 3; ++k) S[k][m] = q.u[1 + k] - s.u[1 + k] * d0;
+                    S[3][m] = q.p;
+                    S[4][m] = r[6] - ga * s.u[2];
+                    S[5][m] = r[7] - ga * s.u[3];
                 }
-                if (near)
+            }
+            if (near) {
+                // slow waves of both sides, or three and more
+                bool more = (near & 4) != 0 || (near & (near >> 1)) != 0;
+                if (!more)
 #pragma unroll 1
                     for (int m = 0; m < 5; ++m)
-                        if (near >> m & 1) whole = !mhd_turn_pair<R>(s, Bs, Rv, 2 + m) || whole;
+                        if (near >> m & 1) more = !mhd_turn_pair<R>(s, Bs, Rv, 2 + m) || more;
+                if (more) mhd_turn_clusters<R>(s, (R)ph.gm1i, Bs, S, Rv, near);
             }
         }
         if (whole) {
             R lam[8], Rc[8][8];
             const R w[8] = {rho, us[0] * s.iW, us[1] * s.iW, us[2] * s.iW, p, Bs[0], Bs[1], Bs[2]};
-            eigen_mhd<R>(ph.gamma, w, lam, Rc);
+            eigen_mhd_gram<R>(ph.gamma, w, lam, Rc, true);
             lo = lam[2];
             hi = lam[7];
             for (int m = 0; m < 8; ++m)

@@ -269,7 +269,7 @@ __device__ __forceinline__ void mhd_UFV_grad(double gam, const T w[8], const dou
 }
 
 // Clustered speeds: the waves of each cluster orthonormalized (R, X and A, rows 2 + m),
-// the orthogonal matrix Th with canonical wave t = sum_i Th[i][t] wave i (mhd_canonical),
+// the orthogonal matrix Th with canonical wave t = sum_i Th[i][t] wave i (mhd_turn_clusters),
 // and what the canonical basis's derivative needs: with G_y = L L^T the Gram matrix of
 // the y_a and S the waves' coefficients in them, E = L^T S (E[i][m] = <q_i, a_m>, q_i the
 // Gram-Schmidt of the y_a; E of the waves, Ec of the canonical ones), rows 4 and 5 of L,
