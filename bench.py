@@ -73,14 +73,14 @@ FLOPS_PER_IFACE_F32 = None
 TRAFFIC_IFACE_F32 = None
 # The same for the RMHD interface kernels at p = 2, WENO5, on the 512^2 rotor, the
 # mean of the two sweeps (whose ambient field leaves other clusters of speeds in each):
-# FP64 5,064 and 9,228 flops per interface, 79 and 259 MB of DRAM traffic per launch;
-# FP32 6,100 and 9,991 FP32 flops besides 70 and 124 FP64 ones, 44 and 484 MB.  The 3D
+# FP64 5,180 and 6,634 flops per interface, 140 and 592 MB of DRAM traffic per launch;
+# FP32 6,212 and 7,027 FP32 flops besides 70 FP64 ones, 72 and 271 MB.  The 3D
 # kernel has not been recaptured since its waves came in closed form (the figures are of
 # the Gram form; its digest below is of those sources, so the bench reports none).
-FLOPS_PER_IFACE_MHD2 = 7146
-TRAFFIC_IFACE_MHD2 = 0.169e9
-FLOPS_PER_IFACE_MHD2_F32 = 8045
-TRAFFIC_IFACE_MHD2_F32 = 0.264e9
+FLOPS_PER_IFACE_MHD2 = 5907
+TRAFFIC_IFACE_MHD2 = 0.366e9
+FLOPS_PER_IFACE_MHD2_F32 = 6620
+TRAFFIC_IFACE_MHD2_F32 = 0.172e9
 FLOPS_PER_IFACE_MHD3 = 16265
 TRAFFIC_IFACE_MHD3 = 9.62e9
 # The fused sweep kernel (pair and interface fluxes in one launch) on the
@@ -101,7 +101,7 @@ COUNTER_SOURCES = {
     "mhd2": ("esmm_mhd.cuh", "esmm_mhd_waves.cuh", "esmm_device.cuh", "esmm_conv.h"),
     "mhd3": ("esmm_3d.cuh", "esmm_3d_iface.cu", "esmm_mhd.cuh", "esmm_mhd_waves.cuh", "esmm_device.cuh", "esmm_conv.h"),
 }
-COUNTER_DIGEST = {"sweep": "929ee2bdf445f782", "mhd2": "fc66711d106938ae", "mhd3": "dd8daf5262c5c5b3"}
+COUNTER_DIGEST = {"sweep": "929ee2bdf445f782", "mhd2": "53088b2c47c2d899", "mhd3": "dd8daf5262c5c5b3"}
 
 
 def source_digest(kind, csrc=None):
