@@ -385,30 +385,53 @@ template <> __device__ __forceinline__ float sub_<float>(float a, float b) { ret
 // second order in FP32).  In FP64 that is 3 and 5 FP64 instructions, against about 7
 // and 10 of the correctly rounded reciprocal and of rsqrt, whose special cases (zero,
 // infinite, subnormal arguments) these leave out: here they give a NaN.
-template <typename R> __device__ __forceinline__ R qrcp(R x) { return rcp<R>(x); }
-template <typename R> __device__ __forceinline__ R qrsq(R x) { return rsq<R>(x); }
+// (Compiled for the host, the approximations are IEEE quotients on the hardware's domain:
+// subnormal arguments and results count as zero.)
 #if defined(__CUDA_ARCH__)
-template <> __device__ __forceinline__ double qrcp<double>(double x)
+__device__ __forceinline__ double approx_rcp(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = __fma_rn(-x, r, 1.0);
+    return r;
+}
+__device__ __forceinline__ float approx_rcp(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ double approx_rsq(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+#else
+template <typename R> inline R ftz_(R x)
+{
+    const R tiny = sizeof(R) == 4 ? (R)1.17549435e-38f : (R)2.2250738585072014e-308;
+    return x < tiny && x > -tiny ? x * (R)0 : x;
+}
+template <typename R> inline R approx_rcp(R x) { return ftz_<R>((R)1 / ftz_<R>(x)); }
+inline double approx_rsq(double x) { return 1.0 / sqrt(ftz_<double>(x)); }
+#endif
+template <typename R> __device__ __forceinline__ R qrcp(R x) { return rcp<R>(x); }
+template <typename R> __device__ __forceinline__ R qrsq(R x) { return rsq<R>(x); }
+template <> __device__ __forceinline__ double qrcp<double>(double x)
+{
+    const double r = approx_rcp(x), e = __fma_rn(-x, r, 1.0);
     return __fma_rn(r, __fma_rn(e, e, e), r);
 }
 template <> __device__ __forceinline__ float qrcp<float>(float x)
 {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    const float r = approx_rcp(x);
     return __fmaf_rn(r, __fmaf_rn(-x, r, 1.0f), r);
 }
 template <> __device__ __forceinline__ double qrsq<double>(double x)
 {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+    const double y = approx_rsq(x), e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
     return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
 }
-#endif
 template <typename R> __device__ __forceinline__ R fab(R x);
 template <> __device__ __forceinline__ double fab<double>(double x) { return fabs(x); }
 template <> __device__ __forceinline__ float fab<float>(float x) { return fabsf(x); }

@@ -811,71 +811,80 @@ static __device__ __noinline__ void mhd_turn_clusters(const MhdBase<R> &s, R ig,
     }
 }
 
+// The scaled eigenvectors of one interface in its rotated frame (first axis along the
+// normal; rows of Rv, one per wave) at the interface state rho, p = 1/ip, spatial
+// 4-velocity us, field Bs, and the smallest and largest speed.  Clusters of two
+// waves of one side are turned by mhd_turn_pair, others by mhd_turn_clusters; states outside
+// the closed form's range take eigen_mhd_gram.
+template <typename R>
+__device__ __forceinline__ void mhd_scaled_waves(const Phys &ph, R rho, R p, R ip, const R us[3], const R Bs[3], R &lo, R &hi,
+                                                 R Rv[8][8])
+{
+    const R gg = (R)(ph.gamma * ph.gm1i);
+    MhdBase<R> s;
+    const R W2 = (R)1 + (us[0] * us[0] + us[1] * us[1] + us[2] * us[2]), iW = qrsq<R>(W2);
+    mhd_base_u<R>((R)ph.gamma, gg, rho, p, ip, W2 * iW, iW, us, Bs, s);
+    bool whole = !mhd_in_range<R>(s);
+    if (!whole) {
+        MhdSix<R> x;
+        R l6[6];
+        mhd_six<R>(s, x, l6);
+        lo = l6[0];
+        hi = l6[5];
+        int near = 0;   // bit m: waves m and m + 1 in one cluster
+#pragma unroll
+        for (int m = 0; m < 5; ++m) near |= (int)mhd_close<R>(l6[m], l6[m + 1]) << m;
+        R S[6][6];
+        mhd_entropy_dU<R>(s, (R)ph.igg, Rv[0]);
+        mhd_divergence_dU<R>(s, Rv[1]);
+#pragma unroll 1
+        for (int m = 0; m < 6; ++m) {
+            MhdWave<R> q;
+            mhd_six_wave<R, false>(s, x, gg, m, q, Rv[2 + m]);
+            if (near) {
+                const R *r = Rv[2 + m], ga = -s.v1 * r[5] * qrcp<R>((R)1 - s.v1 * s.v1) * s.iW, d0 = q.u[0] * s.iW;
+                for (int k = 0; k < 3; ++k) S[k][m] = q.u[1 + k] - s.u[1 + k] * d0;
+                S[3][m] = q.p;
+                S[4][m] = r[6] - ga * s.u[2];
+                S[5][m] = r[7] - ga * s.u[3];
+            }
+        }
+        if (near) {
+            // pairs of one side (not the slow waves of both, nor three and more); a pair turned
+            // here is done: S describes the waves before it
+            int left = near;
+            if ((near & 4) == 0 && (near & (near >> 1)) == 0)
+#pragma unroll 1
+                for (int m = 0; m < 5; ++m)
+                    if ((near >> m & 1) && mhd_turn_pair<R>(s, Bs, Rv, 2 + m)) left &= ~(1 << m);
+            if (left) mhd_turn_clusters<R>(s, (R)ph.gm1i, Bs, S, Rv, left);
+        }
+    }
+    if (whole) {
+        R lam[8], Rc[8][8];
+        const R w[8] = {rho, us[0] * s.iW, us[1] * s.iW, us[2] * s.iW, p, Bs[0], Bs[1], Bs[2]};
+        eigen_mhd_gram<R>(ph.gamma, w, lam, Rc, true);
+        lo = lam[2];
+        hi = lam[7];
+        for (int m = 0; m < 8; ++m)
+            for (int r = 0; r < 8; ++r) Rv[m][r] = Rc[r][m];
+    }
+}
+
 // The ES dissipation of one interface in its rotated frame (first axis along the
 // normal): with the interface state rho = {{rho}}^ln, u = {{u}}, p = 1/ip, B = {{B}}
 // and the scaled eigenvectors R, d = lambda^/2 R Y <<R^T V>>, lambda^ the largest |jt + Lk
 // lambda_m| (reached by a fast wave).  rotV(k, V) gives the rotated entropy variables of the
 // stencil's node k.  The dissipation depends on differences of V alone, so those are
 // projected (w of them), and the wave's edge jump comes from them (weno5_jump); the
-// switch's tolerance, a threshold, is formed in FP32 from |R| and |V|.  Clusters of two
-// waves of one side are turned by mhd_turn_pair, others by mhd_turn_clusters; states outside
-// the closed form's range take eigen_mhd_gram.
+// switch's tolerance, a threshold, is formed in FP32 from |R| and |V|.
 template <typename R, int WW, typename ROTV>
 __device__ __forceinline__ void es_dissipation_mhd(const Phys &ph, R rho, R p, R ip, const R us[3], const R Bs[3], R Lk,
                                                    R jt, ROTV rotV, R d[8])
 {
     constexpr int OFF = (WW - 1) / 2;
-    const R gg = (R)(ph.gamma * ph.gm1i);
     R lo, hi, Rv[8][8];   // (a row per wave)
-    {
-        MhdBase<R> s;
-        const R W2 = (R)1 + (us[0] * us[0] + us[1] * us[1] + us[2] * us[2]), iW = qrsq<R>(W2);
-        mhd_base_u<R>((R)ph.gamma, gg, rho, p, ip, W2 * iW, iW, us, Bs, s);
-        bool whole = !mhd_in_range<R>(s);
-        if (!whole) {
-            MhdSix<R> x;
-            R l6[6];
-            mhd_six<R>(s, x, l6);
-            lo = l6[0];
-            hi = l6[5];
-            int near = 0;   // bit m: waves m and m + 1 in one cluster
-#pragma unroll
-            for (int m = 0; m < 5; ++m) near |= (int)mhd_close<R>(l6[m], l6[m + 1]) << m;
-            R S[6][6];
-            mhd_entropy_dU<R>(s, (R)ph.igg, Rv[0]);
-            mhd_divergence_dU<R>(s, Rv[1]);
-#pragma unroll 1
-            for (int m = 0; m < 6; ++m) {
-                MhdWave<R> q;
-                mhd_six_wave<R, false>(s, x, gg, m, q, Rv[2 + m]);
-                if (near) {
-                    const R *r = Rv[2 + m], ga = -s.v1 * r[5] * qrcp<R>((R)1 - s.v1 * s.v1) * s.iW, d0 = q.u[0] * s.iW;
-                    for (int k = 0; k < 3; ++k) S[k][m] = q.u[1 + k] - s.u[1 + k] * d0;
-                    S[3][m] = q.p;
-                    S[4][m] = r[6] - ga * s.u[2];
-                    S[5][m] = r[7] - ga * s.u[3];
-                }
-            }
-            if (near) {
-                // slow waves of both sides, or three and more
-                bool more = (near & 4) != 0 || (near & (near >> 1)) != 0;
-                if (!more)
-#pragma unroll 1
-                    for (int m = 0; m < 5; ++m)
-                        if (near >> m & 1) more = !mhd_turn_pair<R>(s, Bs, Rv, 2 + m) || more;
-                if (more) mhd_turn_clusters<R>(s, (R)ph.gm1i, Bs, S, Rv, near);
-            }
-        }
-        if (whole) {
-            R lam[8], Rc[8][8];
-            const R w[8] = {rho, us[0] * s.iW, us[1] * s.iW, us[2] * s.iW, p, Bs[0], Bs[1], Bs[2]};
-            eigen_mhd_gram<R>(ph.gamma, w, lam, Rc, true);
-            lo = lam[2];
-            hi = lam[7];
-            for (int m = 0; m < 8; ++m)
-                for (int r = 0; r < 8; ++r) Rv[m][r] = Rc[r][m];
-        }
-    }
+    mhd_scaled_waves<R>(ph, rho, p, ip, us, Bs, lo, hi, Rv);
     R D[WW][8];
     float aT[8];
     {
@@ -1397,6 +1406,7 @@ __global__ void k_update_mhd(ProbArg pa, const double *__restrict__ q, const R *
 }
 
 
+#if defined(__CUDACC__)
 template <typename R, int P>
 static void launch_iface_mhd_p(const LaunchDom &L, const Phys &ph, const double *q, const R *qr, R *iflux, int dir,
                                cudaStream_t st)
@@ -1430,5 +1440,6 @@ static void launch_update_mhd_t(const LaunchDom &L, const double *q, const void 
     k_update_mhd<R><<<L.nblk, L.bs, 0, st>>>(L.pa, q, (const R *)fl, dcons, dJ, cn, Jn, xn, cs, Js, xs, xdot, A, B,
                                              dt_dev, co, Jo, xo);
 }
+#endif
 
 }  // namespace esmm
