@@ -332,7 +332,8 @@ __device__ __forceinline__ void mhd_still_wave(const MhdBase<R> &s, bool along_u
 }
 
 // The wave of kind 0 (fast), 1 (Alfven), 2 (slow) on the side sg, given its |a| = t; c
-// spans with u and xi the wave's plane (b, or a coordinate axis where b lies along k).
+// spans with u and xi the wave's plane (b's direction, of size 1 so that s^2 and t^2 are
+// normal numbers under any field, or a coordinate axis where b lies along k).
 // With k^2 = 1 - lambda^2 + a^2, s normal to u, xi and c, t normal to u, xi and s
 // (t^2 = s^2 k^2), every wave has
 //   du = y = y_t t + y_k k (Alfven: s),  d p = Gamma p pk,  d rho = rho pk,
@@ -425,10 +426,37 @@ __device__ __forceinline__ void mhd_wave(const MhdBase<R> &s, R sqe, R gg, int k
     }
 }
 
+// The power of two that brings the largest |b_i| into [1, 2); 0 where all are zero or
+// subnormal.  (By their bits, off the FP64 pipe.)
+template <typename R> __device__ __forceinline__ R inv_binade(const R b[3]);
+template <> __device__ __forceinline__ double inv_binade<double>(const double b[3])
+{
+    uint32_t e = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const uint32_t h = (uint32_t)(conv_bits64(b[k]) >> 32) & 0x7fffffffu;
+        e = h > e ? h : e;
+    }
+    e >>= 20;
+    return e == 0 ? 0.0 : conv_double((uint64_t)(2046u - e) << 52);
+}
+template <> __device__ __forceinline__ float inv_binade<float>(const float b[3])
+{
+    uint32_t e = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const uint32_t h = conv_bits32(b[k]) & 0x7fffffffu;
+        e = h > e ? h : e;
+    }
+    e >>= 23;
+    return e == 0 ? 0.0f : conv_float((254u - e) << 23);
+}
+
 // The six waves' |a| and the frame data shared by their vectors.
 template <typename R>
 struct MhdSix {
     R t[6], sqe;
+    R c[4];          // b by a power of two, of size 1 (0 where there is no field)
     bool alf[2];     // per side: the fast wave is the Alfven-like one
     bool axis[2];    // b along k (|b_t| at rounding level) or no field: c a coordinate axis
 };
@@ -439,6 +467,9 @@ __device__ __forceinline__ void mhd_six(const MhdBase<R> &s, MhdSix<R> &x, R lam
     MhdCoef<R> kc;
     mhd_coef<R>(s, kc);
     x.sqe = kc.sqe;
+    const R cs = inv_binade<R>(s.b + 1);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) x.c[m] = s.b[m] * cs;
     const float irh = __frcp_rn(to_f32(s.rh)), gp = to_f32(s.gp) * irh;
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
@@ -454,8 +485,8 @@ __device__ __forceinline__ void mhd_six(const MhdBase<R> &s, MhdSix<R> &x, R lam
         x.alf[side] = af * af > gp * ((1.0f - lf) * (1.0f + lf) + af * af);
         const R la = s.v1 - (R)sg * tA * s.iW;
         R sv[4];
-        mcross<R>(s.u, la, s.b, sv);
-        const R A = s.u[0] - la * s.u[1], q = (R)(sizeof(R) == 4 ? 1.0e-10 : 1.0e-22) * s.b2 * A * A;
+        mcross<R>(s.u, la, x.c, sv);
+        const R A = s.u[0] - la * s.u[1], q = (R)(sizeof(R) == 4 ? 1.0e-10 : 1.0e-22) * mdot<R>(x.c, x.c) * A * A;
         x.axis[side] = !(sgn_d(mdot<R>(sv, sv) - q) > 0);
     }
 #pragma unroll
@@ -467,7 +498,7 @@ __device__ __forceinline__ void mhd_six_wave(const MhdBase<R> &s, const MhdSix<R
 {
     const int side = m < 3 ? 0 : 1, kind = m < 3 ? m : 5 - m;   // 0 fast, 1 Alfven, 2 slow
     const bool alf = side == 0 ? x.alf[0] : x.alf[1], axis = side == 0 ? x.axis[0] : x.axis[1];
-    const R c[4] = {axis ? (R)0 : s.b[0], axis ? (R)0 : s.b[1], axis ? (R)1 : s.b[2], axis ? (R)0 : s.b[3]};
+    const R c[4] = {axis ? (R)0 : x.c[0], axis ? (R)0 : x.c[1], axis ? (R)1 : x.c[2], axis ? (R)0 : x.c[3]};
     mhd_wave<R, FULL>(s, x.sqe, gg, kind, side == 0 ? 1 : -1, x.t[m], kind == 0 ? alf : !alf, c, q, dU);
 }
 
