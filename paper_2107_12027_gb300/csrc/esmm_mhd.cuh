@@ -815,7 +815,7 @@ static __device__ __noinline__ void mhd_turn_clusters(const MhdBase<R> &s, R ig,
 // normal; rows of Rv, one per wave) at the interface state rho, p = 1/ip, spatial
 // 4-velocity us, field Bs, and the smallest and largest speed.  Clusters of two
 // waves of one side are turned by mhd_turn_pair, others by mhd_turn_clusters; states outside
-// the closed form's range take eigen_mhd_gram.
+// the closed form's range, and where it finds no positive norm, take eigen_mhd_gram.
 template <typename R>
 __device__ __forceinline__ void mhd_scaled_waves(const Phys &ph, R rho, R p, R ip, const R us[3], const R Bs[3], R &lo, R &hi,
                                                  R Rv[8][8])
@@ -840,7 +840,7 @@ __device__ __forceinline__ void mhd_scaled_waves(const Phys &ph, R rho, R p, R i
 #pragma unroll 1
         for (int m = 0; m < 6; ++m) {
             MhdWave<R> q;
-            mhd_six_wave<R, false>(s, x, gg, m, q, Rv[2 + m]);
+            whole = !mhd_six_wave<R, false>(s, x, gg, m, q, Rv[2 + m]) || whole;
             if (near) {
                 const R *r = Rv[2 + m], ga = -s.v1 * r[5] * qrcp<R>((R)1 - s.v1 * s.v1) * s.iW, d0 = q.u[0] * s.iW;
                 for (int k = 0; k < 3; ++k) S[k][m] = q.u[1 + k] - s.u[1 + k] * d0;

@@ -150,6 +150,9 @@ template <typename R> __device__ __forceinline__ bool is_zero(R x) { return x ==
 template <> __device__ __forceinline__ bool is_neg<double>(double x) { return (conv_bits64(x) >> 63) != 0; }
 template <> __device__ __forceinline__ bool is_zero<double>(double x) { return (conv_bits64(x) << 1) == 0; }
 
+__device__ __forceinline__ bool positive_finite(float x) { return x > 0.0f && x < __FLT_MAX__; }
+__device__ __forceinline__ bool positive_finite(double x) { return conv_bits64(x) - 1ull < 0x7fefffffffffffffull; }
+
 // the smaller and larger of two numbers, b >= 0: in FP64 by their bits (non-negative
 // numbers order like them and a negative one lies below; FP64 compares cost FP64-pipe slots)
 __device__ __forceinline__ float lesser_nn(float a, float b) { return fminf(a, b); }
@@ -307,20 +310,19 @@ __device__ __forceinline__ void mhd_wave_dU(const MhdBase<R> &s, R gg, const Mhd
 }
 
 // One of the four waves of speed v_1 at B_1 = 0, spanned by du or db along s or t
-// with P = 0
+// with P = 0; du.db = 0, and m du^2 is e du^2 - (b.du)^2: m = e along s, rho h along t
 template <typename R>
-__device__ __forceinline__ void mhd_still_wave(const MhdBase<R> &s, bool along_u, const R d[4], MhdWave<R> &q)
+__device__ __forceinline__ void mhd_still_wave(const MhdBase<R> &s, bool along_u, R m, const R d[4], MhdWave<R> &q)
 {
     const R bd = mdot<R>(s.b, d);
     q.p = along_u ? (R)0 : -bd;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        q.u[m] = along_u ? d[m] : (R)0;
-        q.b[m] = along_u ? bd * s.u[m] : d[m];   // (db = (b.du) u)
+    for (int i = 0; i < 4; ++i) {
+        q.u[i] = along_u ? d[i] : (R)0;
+        q.b[i] = along_u ? bd * s.u[i] : d[i];   // (db = (b.du) u)
     }
-    const R P = q.p + mdot<R>(s.b, q.b);
-    const R n2 = s.beta * (s.W * (q.p * q.p * rcp<R>(s.gp) + s.e * mdot<R>(q.u, q.u) + mdot<R>(q.b, q.b)) +
-                           (R)2 * (q.u[0] * P - s.b[0] * mdot<R>(q.b, q.u)));
+    const R d2 = mdot<R>(d, d);
+    const R n2 = s.beta * s.W * (along_u ? m * d2 : d2 + bd * bd * rcp<R>(s.gp));
     const R sc = rsq<R>(n2);
     q.p *= sc;
 #pragma unroll
@@ -338,13 +340,18 @@ __device__ __forceinline__ void mhd_still_wave(const MhdBase<R> &s, bool along_u
 // (t^2 = s^2 k^2), every wave has
 //   du = y = y_t t + y_k k (Alfven: s),  d p = Gamma p pk,  d rho = rho pk,
 //   db = r y + pk b + (b.y) u,  r = B/a,
-// so that the norm and dU take the scalars y^2, b.y, db.y = r y^2 + pk b.y, b.db = r b.y + pk
-// b^2 and db^2 = r db.y + pk b.db - (b.y)^2 (u is normal to b and y) instead of 4-vector
-// products (~30 operations fewer per wave, and one code path for the two magnetosonic
-// forms, which differ between the lanes of a warp).  out: dU, and the du (4-vector)
-// and dp it belongs to; FULL: the perturbations q instead of dU.
+// so that the norm and dU take scalars instead of 4-vector products, and one code path for the
+// two magnetosonic forms, which differ between the lanes of a warp.  The norm is
+//   X^0(q, q) = beta { E W (1 - v_1 lambda)/k^2 + 2 t^0 y_t dp },
+//   E = dp pk + rho h y^2 + z^2 t^2 (1 + a^2/k^2),  z = r y_t + pk (b.t)/t^2,  t^2 = s^2 k^2
+// (the parts of X^mu along k follow from xi.X = 0 and along t all but one cancel; the Alfven
+// waves': 2 beta y^2 (W e - b^0 r)): E is a sum of squares, where the energy's own terms
+// W (e y^2 + db^2) + 2 (y^0 P - b^0 db.y) cancel to 1/W^2 of their size under strong fields
+// (FP32 norms at W = 10 .. 20, b^2 > rho h were off by 8% in the median, 6% of them negative; now
+// 6e-4).  out: dU, and the du (4-vector) and dp it belongs to; FULL: the perturbations q
+// instead of dU; false where rounding leaves no positive norm (FP32 above W ~ 200).
 template <typename R, bool FULL>
-__device__ __forceinline__ void mhd_wave(const MhdBase<R> &s, R sqe, R gg, int kind, int sg, R tw, bool alf_like,
+__device__ __forceinline__ bool mhd_wave(const MhdBase<R> &s, R sqe, R gg, int kind, int sg, R tw, bool alf_like,
                                          const R c[4], MhdWave<R> &q, R dU[8])
 {
     const R a = (R)sg * tw, lam = s.v1 - a * s.iW;
@@ -352,11 +359,11 @@ __device__ __forceinline__ void mhd_wave(const MhdBase<R> &s, R sqe, R gg, int k
     mcross<R>(s.u, lam, c, sv);
     mcross<R>(s.u, lam, sv, tv);
     if (kind != 0 && is_zero(tw)) {
-        mhd_still_wave<R>(s, sg > 0, kind == 1 ? sv : tv, q);
+        mhd_still_wave<R>(s, sg > 0, kind == 1 ? s.e : s.rh, kind == 1 ? sv : tv, q);
         if constexpr (!FULL) mhd_wave_dU<R>(s, gg, q, dU);
-        return;
+        return true;
     }
-    R y[4], y2, by, r, pk;
+    R y[4], by, r, pk, n2;
     if (kind == 1) {
         R s2[4];
         mcross<R>(s.u, lam, tv, s2);   // (normal to u and xi at rounding)
@@ -364,39 +371,32 @@ __device__ __forceinline__ void mhd_wave(const MhdBase<R> &s, R sqe, R gg, int k
         for (int m = 0; m < 4; ++m) y[m] = s2[m];
         r = is_neg(s.B1) ? (R)-sg * sqe : (R)sg * sqe;
         pk = (R)0;
-        y2 = mdot<R>(y, y);
         by = mdot<R>(s.b, y);
+        n2 = (R)2 * mdot<R>(y, y) * (s.W * s.e - s.b[0] * r);
     } else {
-        const R k2 = ((R)1 - lam) * ((R)1 + lam) + a * a, Bx = (s.B1 + a * s.b[0]) * s.iW;
-        const R bt = mdot<R>(s.b, tv), s2 = mdot<R>(sv, sv), t2 = s2 * k2;
-        R yt, yk;
+        const R a2 = a * a, k2 = ((R)1 - lam) * ((R)1 + lam) + a2, Bx = (s.B1 + a * s.b[0]) * s.iW;
+        const R bt = mdot<R>(s.b, tv), s2 = mdot<R>(sv, sv), ra2 = s.rh * a2, gk2 = s.gp * k2;
         r = Bx * qrcp<R>(a);
         // alf_like: y = r t - (rho h a (b.t)/Sf) k; else y = a (B (rho h - Gamma p) (b.t)/(rho h
-        // De s^2) t - k)
-        const R den = alf_like ? s.rh * a * a - s.gp * k2 : s.rh * (s.e * a * a - Bx * Bx) * s2;
-        const R num = (alf_like ? s.rh : Bx * (s.rh - s.gp)) * bt;
-        const R cf = is_zero(bt) ? (R)0 : num * qrcp<R>(den);
-        if (alf_like) {
-            yt = r;
-            yk = -cf * a;
-            pk = cf * k2;
-        } else {
-            yt = a * cf;
-            yk = -a;
-            pk = k2;
-        }
+        // De s^2) t - k); one reciprocal for 1/k^2, 1/s^2 and the wave's own quotient
+        const bool none = is_zero(bt);
+        const R den = none ? (R)1 : (alf_like ? ra2 - gk2 : s.rh * (s.e * a2 - Bx * Bx));
+        const R iq = qrcp<R>(k2 * s2 * den), qd = iq * den, ik2 = s2 * qd, is2 = k2 * qd;
+        const R cf = (alf_like ? s.rh * s2 : Bx * (s.rh - s.gp)) * (bt * (k2 * iq));
+        const R yt = alf_like ? r : a * cf, h = alf_like ? cf : (R)1, yk = -h * a;
+        pk = h * k2;
         const R ka = yk * a;   // k = xi + a u
         y[0] = yt * tv[0] + (yk * lam + ka * s.u[0]);
         y[1] = yt * tv[1] + (yk + ka * s.u[1]);
         y[2] = yt * tv[2] + ka * s.u[2];
         y[3] = yt * tv[3] + ka * s.u[3];
-        y2 = yt * yt * t2 + yk * yk * k2;
         by = yt * bt + yk * Bx;
+        const R z = r * yt + h * bt * is2;
+        n2 = (h * h * (ra2 + gk2) + s2 * (s.rh * yt * yt + z * z * ((R)1 + a2 * ik2))) * (s.W * ((R)1 - s.v1 * lam)) +
+             (R)2 * tv[0] * (yt * (h * gk2));
     }
     R bz = r * by + pk * s.b2;
-    const R zy = r * y2 + pk * by, db2 = r * zy + (pk * bz - by * by);
-    const R n2 = s.beta * (s.W * (s.gp * pk * pk + (s.e * y2 + db2)) + (R)2 * (y[0] * (s.gp * pk + bz) - s.b[0] * zy));
-    const R sc = qrsq<R>(n2);
+    const R sc = qrsq<R>(s.beta * n2);
 #pragma unroll
     for (int m = 0; m < 4; ++m) y[m] *= sc;
     pk *= sc;
@@ -424,6 +424,7 @@ __device__ __forceinline__ void mhd_wave(const MhdBase<R> &s, R sqe, R gg, int k
         }
         dU[4] = de * (s.W * s.W) + (R)2 * (c1 * y[0] - s.b[0] * db0) - (p + bz);
     }
+    return positive_finite(n2);
 }
 
 // The power of two that brings the largest |b_i| into [1, 2); 0 where all are zero or
@@ -494,12 +495,12 @@ __device__ __forceinline__ void mhd_six(const MhdBase<R> &s, MhdSix<R> &x, R lam
 }
 
 template <typename R, bool FULL>
-__device__ __forceinline__ void mhd_six_wave(const MhdBase<R> &s, const MhdSix<R> &x, R gg, int m, MhdWave<R> &q, R dU[8])
+__device__ __forceinline__ bool mhd_six_wave(const MhdBase<R> &s, const MhdSix<R> &x, R gg, int m, MhdWave<R> &q, R dU[8])
 {
     const int side = m < 3 ? 0 : 1, kind = m < 3 ? m : 5 - m;   // 0 fast, 1 Alfven, 2 slow
     const bool alf = side == 0 ? x.alf[0] : x.alf[1], axis = side == 0 ? x.axis[0] : x.axis[1];
     const R c[4] = {axis ? (R)0 : x.c[0], axis ? (R)0 : x.c[1], axis ? (R)1 : x.c[2], axis ? (R)0 : x.c[3]};
-    mhd_wave<R, FULL>(s, x.sqe, gg, kind, side == 0 ? 1 : -1, x.t[m], kind == 0 ? alf : !alf, c, q, dU);
+    return mhd_wave<R, FULL>(s, x.sqe, gg, kind, side == 0 ? 1 : -1, x.t[m], kind == 0 ? alf : !alf, c, q, dU);
 }
 
 // The entropy wave (d rho = 1; its dU[5..7] = 0) and the divergence wave dB = e_1 -

@@ -101,3 +101,26 @@ def test_columns_of_weak_fields(dev, prec, along):
             ref = oracle.mhd_eigen(GAMMA, w)[1]
             R = production(dev, prec, w)[1]
             assert worst(R, ref.T) <= BOUND[prec], (w, worst(R, ref.T))
+
+
+@pytest.mark.parametrize("prec", ["64", "32"])
+@pytest.mark.parametrize("wlo,whi,cold,b2", [(10, 20, (1e-4, 1e-3), (1, 30)), (10, 20, (1e-4, 1), (0.01, 10)), (1, 60, (1e-6, 1), (0.01, 100))])
+def test_columns_of_fast_magnetized_gas(dev, prec, wlo, whi, cold, b2):
+    """Norms of fast, cold, strongly magnetized states: positive, and in FP32 the columns'
+    median error, W^2 eps ~ 1e-5 over the p/(rho h) that the sound speed resolves, below 5e-3 up to
+    W = 20 (FP64 1e-6, which is the oracle's own at these)."""
+    r = np.random.default_rng(991)
+    err = []
+    for _ in range(600):
+        W, d, n = r.uniform(wlo, whi), r.standard_normal(3), r.standard_normal(3)
+        v = d / np.linalg.norm(d) * np.sqrt(1.0 - 1.0 / W ** 2)
+        rho = np.exp(r.uniform(-1, 1))
+        p = rho * np.exp(r.uniform(*np.log(cold)))
+        n /= np.linalg.norm(n)
+        b = np.sqrt((rho + 2.5 * p) * np.exp(r.uniform(*np.log(b2))) / (1.0 / W ** 2 + (v @ n) ** 2))
+        w = state(rho, v, p, b * n)
+        lohi, R = production(dev, prec, w)
+        assert np.isfinite(lohi).all() and np.isfinite(R).all(), w
+        err.append(worst(R, oracle.mhd_eigen(GAMMA, w)[1].T))
+    if whi <= 20:
+        assert np.median(err) <= (5e-3 if prec == "32" else 1e-6)
