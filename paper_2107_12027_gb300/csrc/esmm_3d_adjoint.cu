@@ -132,8 +132,9 @@ __device__ __forceinline__ void dphi8(const double r[8], double d[8])
     d[4] = 0.0; d[5] = 0.0; d[6] = r[7]; d[7] = -r[6];
 }
 
+// (three blocks an SM: 168 registers; the Gram form's tangents, seldom called, would take 255)
 template <int WW>
-__global__ void __launch_bounds__(128) k3_iface_vjp(Geom3 g, Phys ph, const double *__restrict__ q,
+__global__ void __launch_bounds__(128, 3) k3_iface_vjp(Geom3 g, Phys ph, const double *__restrict__ q,
                                                     const double *__restrict__ mu, double *__restrict__ lamq, int dir)
 {
     constexpr int NS = WW + 1, OFF = (WW - 1) / 2;

@@ -419,6 +419,72 @@ static __device__ __noinline__ void mhd_turn(const MhdClusters &c, double M[8][8
     }
 }
 
+// mhd_diss_vjp by the Gram form and its tangent along each direction of the state, for what
+// the closed form leaves to it (as in mhd_scaled_waves).
+template <int WW>
+static __device__ __noinline__ void mhd_diss_vjp_gram(const Phys &ph, const double wrot[8], double Lk, double jt,
+                                                      const double lrot[8], const double TV[][8], double gTV[][8],
+                                                      double gw[8], double Rz[8], double &hl)
+{
+    constexpr int NS = WW + 1, OFF = (WW - 1) / 2;
+    double lam[8], R[8][8];   // (a column per wave)
+    eigen_mhd_gram<double>(ph.gamma, wrot, lam, R, true);
+    double lhat = 0.0;
+    int msel = 0;
+    for (int m = 0; m < 8; ++m) {
+        const double v = fabs(jt + Lk * lam[m]);
+        if (v > lhat) { lhat = v; msel = m; }
+    }
+    const double sg = (jt + Lk * lam[msel]) >= 0.0 ? 1.0 : -1.0;
+    hl = 0.5 * lhat;
+    for (int k = 0; k < NS; ++k)
+        for (int b = 0; b < 8; ++b) gTV[k][b] = 0.0;
+    for (int b = 0; b < 8; ++b) Rz[b] = 0.0;
+    double Rb[8][8], zeta = 0.0;
+#pragma unroll 1
+    for (int m = 0; m < 8; ++m) {
+        double Vt[NS], gVt[NS], scale = 0.0, qm = 0.0;
+        for (int k = 0; k < NS; ++k) {
+            Vt[k] = 0.0;
+            for (int a = 0; a < 8; ++a) {
+                const double t = R[a][m] * TV[k][a];
+                Vt[k] += t;
+                if (k == OFF || k == OFF + 1) scale += fabs(t);
+            }
+        }
+        for (int b = 0; b < 8; ++b) qm += R[b][m] * lrot[b];
+        double vminus, vplus;
+        if constexpr (WW == 5) weno5_lr<double>(Vt[0], Vt[1], Vt[2], Vt[3], Vt[4], Vt[5], ph.eps, vminus, vplus);
+        else weno3_lr<double>(Vt[0], Vt[1], Vt[2], Vt[3], ph.eps, vminus, vplus);
+        const double jw = vplus - vminus, jump = Vt[OFF + 1] - Vt[OFF];
+        const int sj = fabs(jump) <= ph.sign_tol * scale ? 0 : sgn_d(jump);
+        const bool y = sgn_d(jw) == sj;
+        const double z = y ? jw : 0.0;
+        zeta += qm * z;
+        for (int b = 0; b < 8; ++b) {
+            Rz[b] += R[b][m] * z;
+            Rb[b][m] = -hl * lrot[b] * z;
+        }
+        if (!y) continue;
+        weno_jump_vjp<WW>(Vt, ph.eps, -hl * qm, gVt);
+        for (int k = 0; k < NS; ++k)
+            for (int b = 0; b < 8; ++b) {
+                gTV[k][b] += R[b][m] * gVt[k];
+                Rb[b][m] += gVt[k] * TV[k][b];
+            }
+    }
+#pragma unroll 1
+    for (int a = 0; a < 8; ++a) {
+        dual wd[8], ld[8], Rd[8][8];
+        for (int k = 0; k < 8; ++k) wd[k] = dual(wrot[k], k == a ? 1.0 : 0.0);
+        eigen_mhd_gram<dual>(ph.gamma, wd, ld, Rd, true);
+        double acc = -0.5 * sg * Lk * ld[msel].d * zeta;
+        for (int b = 0; b < 8; ++b)
+            for (int m = 0; m < 8; ++m) acc += Rb[b][m] * Rd[b][m].d;
+        gw[a] = acc;
+    }
+}
+
 // Reverse sweep of the ES dissipation at one interface (rotated frame):
 // lrot = T lambda_F, TV the stencil's rotated entropy variables, wrot the rotated
 // interface state.  gTV: adjoint of TV; gw: adjoint of wrot; Rz = R z and hl =
@@ -430,9 +496,10 @@ static __device__ __noinline__ void mhd_turn(const MhdClusters &c, double M[8][8
 // lower half of L^-1 G_y' L^-T and h_k = v_1 v_k/(1 - v_1^2) (from the divergence wave's
 // direction), sum_{s <= j} E[ii[j]][s] O_st equals minus the rest, a triangular system
 // whose adjoint adds to the coefficients of G', K' and of the divergence direction.
-// The speed lambda^ keeps its own resolved wave.
+// The speed lambda^ keeps its own resolved wave.  False where the closed form leaves the
+// interface to the Gram form.
 template <int WW>
-__device__ __noinline__ void mhd_diss_vjp(const Phys &ph, const double wrot[8], double Lk, double jt,
+__device__ __noinline__ bool mhd_diss_vjp_waves(const Phys &ph, const double wrot[8], double Lk, double jt,
                                           const double lrot[8], const double TV[][8], double gTV[][8], double gw[8],
                                           double Rz[8], double &hl)
 {
@@ -440,6 +507,7 @@ __device__ __noinline__ void mhd_diss_vjp(const Phys &ph, const double wrot[8], 
     const double gam = ph.gamma, gm1i = 1.0 / (gam - 1.0), gg = gam * gm1i;
     MhdBase<double> s;
     mhd_base<double>(gam, gg, wrot, s);
+    if (!mhd_in_range<double>(s)) return false;
     MhdSix<double> six;
     double lam[8];
     lam[0] = lam[1] = s.v1;
@@ -483,7 +551,7 @@ __device__ __noinline__ void mhd_diss_vjp(const Phys &ph, const double wrot[8], 
 #pragma unroll 1
     for (int m = 0; m < 6; ++m) {
         MhdWave<double> q;
-        mhd_six_wave<double, true>(s, six, gg, m, q, R[2 + m]);
+        if (!mhd_six_wave<double, true>(s, six, gg, m, q, R[2 + m])) return false;
         mhd_wave_dU<double>(s, gg, q, R[2 + m]);
         const double db = (q.rho - s.beta * q.p) * s.ip;
         double *x = X[2 + m], *a = A[2 + m];
@@ -719,6 +787,16 @@ __device__ __noinline__ void mhd_diss_vjp(const Phys &ph, const double wrot[8], 
         g[3] += eta[1] * v[0] * iv;
     }
     for (int k = 0; k < 8; ++k) gw[k] = g[k];
+    return true;
+}
+
+template <int WW>
+__device__ __forceinline__ void mhd_diss_vjp(const Phys &ph, const double wrot[8], double Lk, double jt,
+                                             const double lrot[8], const double TV[][8], double gTV[][8], double gw[8],
+                                             double Rz[8], double &hl)
+{
+    if (!mhd_diss_vjp_waves<WW>(ph, wrot, Lk, jt, lrot, TV, gTV, gw, Rz, hl))
+        mhd_diss_vjp_gram<WW>(ph, wrot, Lk, jt, lrot, TV, gTV, gw, Rz, hl);
 }
 
 }  // namespace esmm
