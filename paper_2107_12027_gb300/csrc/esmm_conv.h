@@ -104,4 +104,39 @@ ESMM_CONV_HD double f2d_int(float x)
     return (double)x;
 }
 
+// d2f_int(x 2^-k) and f2d_int(x) 2^k without the product, where it is normal; a result
+// below the normal range is 0, one above it infinite
+ESMM_CONV_HD float d2f_scaled(double x, int k)
+{
+    const uint64_t b = conv_bits64(x);
+    const uint32_t hi = (uint32_t)(b >> 32);
+    const uint32_t sign = hi & 0x80000000u;
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    const int es = (int)e - k - 896;
+    if (e - 1u < 2046u && (uint32_t)(es - 1) <= 253u) {
+        const uint64_t m = b & 0x000fffffffffffffull;
+        uint32_t r = ((uint32_t)es << 23) | (uint32_t)(m >> 29);
+        const uint32_t rem = (uint32_t)m & 0x1fffffffu;
+        r += (uint32_t)(rem > 0x10000000u) | ((uint32_t)(rem == 0x10000000u) & (r & 1u));
+        return conv_float(r | sign);
+    }
+    if (e == 0x7ffu) return (float)x;
+    return conv_float(sign | (e != 0u && es > 254 ? 0x7f800000u : 0u));
+}
+
+ESMM_CONV_HD double f2d_scaled(float x, int k)
+{
+    const uint32_t u = conv_bits32(x);
+    const uint32_t e = (u >> 23) & 0xffu;
+    const uint64_t sign = (uint64_t)(u & 0x80000000u) << 32;
+    const int ed = (int)e + 896 + k;
+    if (e - 1u < 254u && (uint32_t)(ed - 1) < 2046u)
+        return conv_double(sign | ((uint64_t)(uint32_t)ed << 52) | ((uint64_t)(u & 0x7fffffu) << 29));
+    if (e == 0xffu) return (double)x;
+    return conv_double(sign | (e != 0u && ed > 2046 ? 0x7ff0000000000000ull : 0ull));
+}
+
+// k of 2^k <= |x| < 2^(k+1)
+ESMM_CONV_HD int binade(double x) { return (int)((conv_bits64(x) >> 52) & 0x7ffu) - 1023; }
+
 }  // namespace esmm

@@ -468,7 +468,7 @@ __device__ __forceinline__ void logmean(T a, T b, T la, T lb, double thr, R &mea
 //   f(p) = (G-1)/G ((E+p)(1-v^2) - D sqrt(1-v^2)) - p,  v = |m|/(E+p).
 // An FP32 Newton iteration (c2p_estimate, off the FP64 pipe) gives p to about 1e-7 (E + p);
 // one FP64 step of third order (Halley's; the curvature in FP32) then lands on the root
-// to rounding: it is the last where it is below 3e-6 of E + p - |m|, the length on
+// to rounding, in any units (the FP32 parts work over the power of two below E): it is the last where it is below 3e-6 of E + p - |m|, the length on
 // which f bends, and its second-order part below 3e-6 of it, which leaves the next
 // term under 1e-11 of the step.  Where that fails three times (an estimate that failed,
 // states at the edge of the admissible set) c2p_loop starts over: FP64 Newton safeguarded by bisection on [0, (G-1)E],
@@ -542,9 +542,10 @@ __device__ __forceinline__ int cons2prim_gg(double gam, double gg, double D, dou
     }
     const double hi = (gam - 1.0) * E, EmS = E - S;
     const double pw = (p0 > 0.0 && p0 < hi) ? p0 : 0.5 * hi;
-    const float ggf = d2f_int(gg), Df = d2f_int(D), EmSf = d2f_int(EmS);
-    const float pf = c2p_estimate(ggf, Df, d2f_int(S2), d2f_int(S), EmSf, d2f_int(E), d2f_int(hi), d2f_int(pw));
-    double pc = f2d_int(pf);
+    const int k = binade(E);   // the FP32 parts take every quantity over 2^k
+    const float ggf = d2f_int(gg), Df = d2f_scaled(D, k), EmSf = d2f_scaled(EmS, k), Sf = d2f_scaled(S, k);
+    const float pf = c2p_estimate(ggf, Df, Sf * Sf, Sf, EmSf, d2f_scaled(E, k), d2f_scaled(hi, k), d2f_scaled(pw, k));
+    double pc = f2d_scaled(pf, k);
     int st = 0;
     bool ok = false;
 #pragma unroll 1
@@ -553,12 +554,12 @@ __device__ __forceinline__ int cons2prim_gg(double gam, double gg, double D, dou
         const double v2 = S2 * (r * r), Dw = D * rs;
         const double f = gg * (Ep * iW2 - Dw * iW2) - pc, df = gg * (1.0 + v2 - Dw * (v2 * r)) - 1.0;
         const double dp = f * qrcp<double>(df);
-        const float rf = d2f_int(r), vf = d2f_int(v2), sf = d2f_int(rs), dpf = d2f_int(dp);
+        const float rf = d2f_scaled(r, -k), vf = d2f_int(v2), sf = d2f_int(rs), dpf = d2f_scaled(dp, k);
         const float a = vf * rf, f2 = ggf * (Df * sf * (3.0f * a * rf + a * a * (sf * sf)) - 2.0f * a);
         const float eta = 0.5f * f2 * dpf * __frcp_rn(d2f_int(df));
-        ok = fabsf(dpf) <= 3.0e-6f * (EmSf + d2f_int(pc)) && fabsf(eta) <= 3.0e-6f;
-        const double pn = pc - (dp + f2d_int(dpf * eta));
-        if (!(d2f_int(pn) > 0.0f) || !(fabsf(eta) <= 0.1f)) {
+        ok = fabsf(dpf) <= 3.0e-6f * (EmSf + d2f_scaled(pc, k)) && fabsf(eta) <= 3.0e-6f;
+        const double pn = pc - __fma_rn(dp, f2d_int(eta), dp);
+        if (!(d2f_scaled(pn, k) > 0.0f) || !(fabsf(eta) <= 0.1f)) {
             ok = false;
             break;
         }

@@ -38,7 +38,8 @@ constexpr int NFM = 10;                          // interface values per directi
 // its second-order part below 3e-6 of it), and where that fails three times c2p_loop_mhd, FP64 Newton with
 // bisection on [0, Gamma E], which stops when a step moves Z by at most 1e-15 (E + Z), or
 // where |f| <= 2e-15 (E + Z), f's rounding level (a root, whose tiny steps the open
-// bracket would otherwise reject).  The FP32 iteration works in units of E.
+// bracket would otherwise reject).  The FP32 parts work in units of E (converted over powers of
+// two, so that E^2 and E^3 stay in FP32's range).
 // Z0: warm start (ignored outside the bracket).  Measured: the node pass of 512^2 nodes 214 ->
 // 146 us, mixed rotor steps 3.71 -> 3.05 ms (with the speeds' pass in 80 registers).
 // Returns 0, 1 (non-admissible) or 2 (iteration cap).
@@ -114,10 +115,11 @@ __device__ __forceinline__ int cons2prim_mhd(double gam, const double U[8], doub
     if (!(D > 0.0) || !(E > 0.0)) return 1;
     const double hi = gam * E;
     const double Zw = (Z0 > 0.0 && Z0 < hi) ? Z0 : 0.5 * hi;
-    const float Ef = d2f_int(E), iE = __frcp_rn(Ef), gf = d2f_int(g), Df = d2f_int(D) * iE, B2f = d2f_int(B2) * iE;
-    const float m2f = d2f_int(m2) * iE * iE, S2f = d2f_int(S2) * iE * iE * iE;
-    const float Zf = c2p_estimate_mhd(gf, d2f_int(gam), Df, m2f, B2f, S2f, d2f_int(Zw) * iE);
-    double Z = f2d_int(Zf * Ef);
+    const int k = binade(E);
+    const float Ef = d2f_scaled(E, k), iE = __frcp_rn(Ef), gf = d2f_int(g), Df = d2f_scaled(D, k) * iE;
+    const float B2f = d2f_scaled(B2, k) * iE, m2f = d2f_scaled(m2, 2 * k) * iE * iE, S2f = d2f_scaled(S2, 3 * k) * iE * iE * iE;
+    const float Zf = c2p_estimate_mhd(gf, d2f_int(gam), Df, m2f, B2f, S2f, d2f_scaled(Zw, k) * iE);
+    double Z = f2d_scaled(Zf * Ef, k);
     int st = 0;
     bool ok = false;
 #pragma unroll 1
@@ -129,15 +131,15 @@ __device__ __forceinline__ int cons2prim_mhd(double gam, const double U[8], doub
         const double df = 1.0 - g * (iW2 - dv2 * (Z - 0.5 * Dw)) + 0.5 * B2 * dv2 + t * iZ;
         const double dZ = f * qrcp<double>(df);
         // f'' in units of E (Z = z E): v2'' = N'' q^2 - 4 N' q^3 + 6 N q^4
-        const float z = d2f_int(Z) * iE, iz = __frcp_rn(z), q = __frcp_rn(z + B2f), tf = S2f * iz * iz, Nf = m2f + (2.0f * z + B2f) * tf;
+        const float z = d2f_scaled(Z, k) * iE, iz = __frcp_rn(z), q = __frcp_rn(z + B2f), tf = S2f * iz * iz, Nf = m2f + (2.0f * z + B2f) * tf;
         const float N1 = -2.0f * tf * (1.0f + B2f * iz), N2 = tf * iz * (4.0f + 6.0f * B2f * iz), qq = q * q;
         const float v1 = (N1 - 2.0f * Nf * q) * qq, v22 = (N2 - 4.0f * N1 * q + 6.0f * Nf * qq) * qq, sf = d2f_int(rs);
         const float p2 = gf * (-2.0f * v1 - z * v22 + 0.5f * Df * sf * (v22 + 0.5f * v1 * v1 * (sf * sf)));
         const float f2 = -p2 + 0.5f * B2f * v22 - 3.0f * tf * (iz * iz);
-        const float dz = d2f_int(dZ) * iE, eta = 0.5f * f2 * dz * __frcp_rn(d2f_int(df));
+        const float dz = d2f_scaled(dZ, k) * iE, eta = 0.5f * f2 * dz * __frcp_rn(d2f_int(df));
         ok = fabsf(dz) <= 3.0e-6f * z * d2f_int(iW2) && fabsf(eta) <= 3.0e-6f;
-        const double Zn = Z - (dZ + f2d_int(dz * eta * Ef));
-        if (!(d2f_int(Zn) > 0.0f) || !(fabsf(eta) <= 0.1f)) {
+        const double Zn = Z - __fma_rn(dZ, f2d_int(eta), dZ);
+        if (!(d2f_scaled(Zn, k) > 0.0f) || !(fabsf(eta) <= 0.1f)) {
             ok = false;
             break;
         }
