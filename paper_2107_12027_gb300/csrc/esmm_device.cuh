@@ -699,6 +699,18 @@ __device__ __forceinline__ void ec_pair(const NodeV<R> &l, const NodeV<R> &r, R 
 // 1.25 -> 1.22 ms, one 64^2 right-hand side 44 -> 37 us).  Everything is scaled by 4 (eps4 = 4 eps, b_k of doubled
 // first-derivative terms).  Sums of two products are written as the fused operation, so
 // that every kernel that inlines this rounds them alike.
+// FP32: the products of four e (up to 33 D^2 each, down to 4 eps) and a difference would leave the
+// range from D ~ 2,600 up, and for eps below ~1e-10.  A side's e count by their ratios alone, so they
+// are taken to 2^24 and below by the power of two: in range up to D ~ 1e7 and eps down to 1e-30
+// (400^2 mixed step 1.112 -> 1.120 ms).
+template <typename R> __device__ __forceinline__ void weno5_scale(R &, R &, R &) {}
+template <> __device__ __forceinline__ void weno5_scale<float>(float &e0, float &e1, float &e2)
+{
+    const float sc = conv_float((278u << 23) - (conv_bits32(fmaxf(fmaxf(e0, e1), e2)) & 0x7f800000u));
+    e0 *= sc;
+    e1 *= sc;
+    e2 *= sc;
+}
 template <typename R>
 __device__ __forceinline__ R weno5_jump(R D0, R D1, R D2, R D3, R D4, R eps4)
 {
@@ -711,6 +723,7 @@ __device__ __forceinline__ R weno5_jump(R D0, R D1, R D2, R D3, R D4, R eps4)
     {
         const R r0 = t0 + two * D1, r1 = D1 + D2, r2 = tb - two * D2;
         R e0 = fma_<R>(r0, r0, S0), e1 = fma_<R>(r1, r1, Sa), e2 = fma_<R>(r2, r2, Sb);
+        weno5_scale<R>(e0, e1, e2);
         e0 *= e0; e1 *= e1; e2 *= e2;
         nl = e1 * fma_<R>(three, e0 * d1, two * (e2 * d0));
         ql = qrcp<R>(fma_<R>(e2, fma_<R>(six, e0, e1), three * (e0 * e1)));
@@ -718,6 +731,7 @@ __device__ __forceinline__ R weno5_jump(R D0, R D1, R D2, R D3, R D4, R eps4)
     {
         const R r0 = t5 - two * D3, r1 = D2 + D3, r2 = ta + two * D2;
         R e0 = fma_<R>(r0, r0, S5), e1 = fma_<R>(r1, r1, Sb), e2 = fma_<R>(r2, r2, Sa);
+        weno5_scale<R>(e0, e1, e2);
         e0 *= e0; e1 *= e1; e2 *= e2;
         nr = e1 * fma_<R>(three, e0 * d1, two * (e2 * d2));
         qr = qrcp<R>(fma_<R>(e2, fma_<R>(six, e0, e1), three * (e0 * e1)));
