@@ -41,18 +41,6 @@ __device__ __forceinline__ NodeV<R> load_node(const Geom &g, const double *__res
     return v;
 }
 
-// The ES dissipation 1/2 lambda^ T^-1 R Y <<V~>> of eq. ESFlux_HO at one
-// interface, subtracted from the EC flux F.  nvx, nvy, jt: the interface
-// metrics (mean of the two nodes); rho0/1: the density at the two interface nodes
-// (log-mean arguments); st: the w + 1 stencil nodes, the interface nodes at
-// k = (w-1)/2 and (w+1)/2, with state (beta, u_x, u_y), differences dV(k) = V_{k+1} -
-// V_k of the entropy variables, and V32 their FP32 values (for the switch's
-// tolerance).  The eigen-system is taken at rho = {{rho}}^ln,
-// u = {{u}}, p = {{rho}}/{{beta}}; Y has sign 0 for jumps at rounding level.
-// Sums of two products are written as the fused operation, so that the kernels that
-// inline this round them alike.
-// The dissipation depends on differences of V alone, so they are projected (w of
-// them) rather than the w + 1 values.
 // The entropy variables (V_1, V_x, V_y, V_E) of one node (Sec. 2, B = 0)
 // from beta, u, W, ln rho, ln beta: V_1 = Gamma/(Gamma-1) + ln rho +
 // ln beta/(Gamma-1) + beta, (V_x, V_y) = beta u, V_E = -beta W.  Every
@@ -162,6 +150,33 @@ struct ArrGet {
     __device__ __forceinline__ R operator()(int k, int j) const { return a[k][j]; }
 };
 
+// jump_sign64 of a jump against its FP64 terms, e the wave's row
+template <typename ST>
+static __device__ __noinline__ int jump_sign_node64(ST st, int k, double c1g, double ig, double nx, double ny, double e0,
+                                                    double e1, double e2, double e3, double jump, double sign_tol)
+{
+    double scale = 0.0;
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+        double V[4];
+        st.V(k + side, c1g, ig, V);
+        scale += fabs(e0 * V[0]) + fabs(e1 * (nx * V[1] + ny * V[2])) + fabs(e2 * (nx * V[2] - ny * V[1])) + fabs(e3 * V[3]);
+    }
+    return jump_sign64(jump, sign_tol, scale);
+}
+
+// The ES dissipation 1/2 lambda^ T^-1 R Y <<V~>> of eq. ESFlux_HO at one
+// interface, subtracted from the EC flux F.  nvx, nvy, jt: the interface
+// metrics (mean of the two nodes); rho0/1: the density at the two interface nodes
+// (log-mean arguments); st: the w + 1 stencil nodes, the interface nodes at
+// k = (w-1)/2 and (w+1)/2, with state (beta, u_x, u_y), differences dV(k) = V_{k+1} -
+// V_k of the entropy variables, and V32 their FP32 values (for the switch's
+// tolerance).  The eigen-system is taken at rho = {{rho}}^ln,
+// u = {{u}}, p = {{rho}}/{{beta}}; Y has sign 0 for jumps at rounding level.
+// Sums of two products are written as the fused operation, so that the kernels that
+// inline this round them alike.
+// The dissipation depends on differences of V alone, so they are projected (w of
+// them) rather than the w + 1 values.
 template <typename R, int WW, typename ST>
 __device__ __forceinline__ void es_dissipation(R nvx, R nvy, R jt, const LmV<R> &rho0, const LmV<R> &rho1,
                                                const ST &st, const Phys &ph, R F[4])
@@ -199,6 +214,7 @@ __device__ __forceinline__ void es_dissipation(R nvx, R nvy, R jt, const LmV<R> 
         aT[1] = fab<S>(nx_ * V0[1] + ny_ * V0[2]) + fab<S>(nx_ * V1[1] + ny_ * V1[2]);
         aT[2] = fab<S>(nx_ * V0[2] - ny_ * V0[1]) + fab<S>(nx_ * V1[2] - ny_ * V1[1]);
         aT[3] = fab<S>(V0[3]) + fab<S>(V1[3]);
+        if constexpr (std::is_same<S, float>::value) jump_terms<R, 4>(aT);
     }
     // projected differences, the rotation T folded into the projection rows once per
     // interface
@@ -221,7 +237,6 @@ __device__ __forceinline__ void es_dissipation(R nvx, R nvy, R jt, const LmV<R> 
                 Dt[k][m] = fma_<R>(Ar[m][3], D[3], fma_<R>(Ar[m][2], D[2], fma_<R>(Ar[m][1], D[1], Ar[m][0] * D[0])));
         }
     }
-    const S tol = (S)ph.sign_tol;
     R d[4] = {(R)0, (R)0, (R)0, (R)0};
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -235,7 +250,15 @@ __device__ __forceinline__ void es_dissipation(R nvx, R nvy, R jt, const LmV<R> 
         // interface nodes is rounding noise: its sign is 0 (so Y = 0)
         const S scale = fab<S>(to_tol(E[m][0])) * aT[0] + fab<S>(to_tol(E[m][1])) * aT[1] +
                         fab<S>(to_tol(E[m][2])) * aT[2] + fab<S>(to_tol(E[m][3])) * aT[3];
-        const int sj = le(fab<S>(to_tol(jump)), tol * scale) ? 0 : sgn_d(jump);
+        int sj;
+        if constexpr (std::is_same<S, float>::value) {
+            sj = jump_sign(jump, ph.sign_tol, scale);
+            if constexpr (std::is_same<R, double>::value)
+                if (sj == JUMP_UNSURE)
+                    sj = jump_sign_node64(st, OFF, c1g, ig, nx, ny, E[m][0], E[m][1], E[m][2], E[m][3], jump, ph.sign_tol);
+        } else {
+            sj = le(fab<S>(jump), (S)ph.sign_tol * scale) ? 0 : sgn_d(jump);
+        }
         const R z = (sgn_d(jw) == sj) ? jw : (R)0;
 #pragma unroll
         for (int a = 0; a < 4; ++a) d[a] = fma_<R>(E[m][a], z, d[a]);
@@ -394,6 +417,7 @@ __global__ void __launch_bounds__(128) k_iface(ProbArg pa, Phys ph, const double
 
 inline long long tiles_of(const LaunchDom &L) { return L.ntiles < 0 ? (long long)L.nblk : L.ntiles; }
 
+#if defined(__CUDACC__)
 template <typename R, int P>
 static void launch_pairs_p(const LaunchDom &L, const Phys &ph, const double *q, const float *q32, R *pairs, int dir,
                            cudaStream_t st)
@@ -462,5 +486,6 @@ void launch_iface_t(const LaunchDom &L, const Phys &ph, const double *q, const f
     default: launch_iface_p<R, 3>(L, ph, q, q32, pr, fl, dir, st); break;
     }
 }
+#endif
 
 }  // namespace esmm

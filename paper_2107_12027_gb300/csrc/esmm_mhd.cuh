@@ -879,7 +879,7 @@ __device__ __forceinline__ void mhd_scaled_waves(const Phys &ph, R rho, R p, R i
 // lambda_m| (reached by a fast wave).  rotV(k, V) gives the rotated entropy variables of the
 // stencil's node k.  The dissipation depends on differences of V alone, so those are
 // projected (w of them), and the wave's edge jump comes from them (weno5_jump); the
-// switch's tolerance, a threshold, is formed in FP32 from |R| and |V|.
+// switch's tolerance is formed in FP32 from |R| and |V| (jump_sign).
 template <typename R, int WW, typename ROTV>
 __device__ __forceinline__ void es_dissipation_mhd(const Phys &ph, R rho, R p, R ip, const R us[3], const R Bs[3], R Lk,
                                                    R jt, ROTV rotV, R d[8])
@@ -887,7 +887,7 @@ __device__ __forceinline__ void es_dissipation_mhd(const Phys &ph, R rho, R p, R
     constexpr int OFF = (WW - 1) / 2;
     R lo, hi, Rv[8][8];   // (a row per wave)
     mhd_scaled_waves<R>(ph, rho, p, ip, us, Bs, lo, hi, Rv);
-    R D[WW][8];
+    R D[WW][8], Vo[8];   // (Vo: the left node's, for jumps that FP32 leaves open)
     float aT[8];
     {
         R V[2][8];
@@ -898,11 +898,15 @@ __device__ __forceinline__ void es_dissipation_mhd(const Phys &ph, R rho, R p, R
             rotV(k + 1, vb);
 #pragma unroll
             for (int a = 0; a < 8; ++a) {
-                if (k == OFF) aT[a] = fabsf(to_f32(va[a])) + fabsf(to_f32(vb[a]));
+                if (k == OFF) {
+                    aT[a] = fabsf(to_f32(va[a])) + fabsf(to_f32(vb[a]));
+                    Vo[a] = va[a];
+                }
                 D[k][a] = sub_<R>(vb[a], va[a]);
             }
         }
     }
+    jump_terms<R, 8>(aT);
 #pragma unroll
     for (int a = 0; a < 8; ++a) d[a] = (R)0;
 #pragma unroll 1
@@ -925,7 +929,14 @@ __device__ __forceinline__ void es_dissipation_mhd(const Phys &ph, R rho, R p, R
         if constexpr (WW == 5) jw = weno5_jump<R>(Dt[0], Dt[1], Dt[2], Dt[3], Dt[4], (R)(4.0 * ph.eps));
         else jw = weno3_jump<R>(Dt[0], Dt[1], Dt[2], (R)ph.eps);
         const R jump = Dt[OFF];
-        const int sj = fabsf(to_f32(jump)) <= (float)ph.sign_tol * scale ? 0 : sgn_d(jump);
+        int sj = jump_sign(jump, ph.sign_tol, scale);
+        if constexpr (std::is_same<R, double>::value)
+            if (sj == JUMP_UNSURE) {
+                double s64 = 0.0;
+#pragma unroll
+                for (int a = 0; a < 8; ++a) s64 += fabs(r[a]) * (fabs(Vo[a]) + fabs(Vo[a] + D[OFF][a]));
+                sj = jump_sign64(jump, ph.sign_tol, s64);
+            }
         const R z = sgn_d(jw) == sj ? jw : (R)0;
 #pragma unroll
         for (int a = 0; a < 8; ++a) d[a] += r[a] * z;

@@ -97,6 +97,11 @@ struct SmemStencil {
 #pragma unroll
         for (int a = 0; a < 4; ++a) v[a] = s.t[a * SW_NNP + base + k];
     }
+    __device__ __forceinline__ void V(int k, R c1g, R ig, R v[4]) const
+    {
+        const int e = base + k;
+        entropy_vars4<R>(s.at(1, e), s.at(4, e), s.at(5, e), s.at(6, e), s.at(2, e), s.at(3, e), c1g, ig, v);
+    }
 };
 
 // one node of global padded index c into staged slot e of a warp's arrays, with its
