@@ -432,6 +432,20 @@ template <> __device__ __forceinline__ double qrsq<double>(double x)
     const double y = approx_rsq(x), e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
     return __fma_rn(__dmul_rn(y, e), __fma_rn(0.375, e, 0.5), y);
 }
+// sqrt(x) as x qrsq(x) where that holds, sqrt's own value for 0, subnormal, infinite and
+// negative x
+__device__ __forceinline__ double qsqrt(double x)
+{
+    return (conv_bits64(x) >> 52) - 1ull < 0x7feull ? x * qrsq<double>(x) : sqrt(x);
+}
+// acoustic speeds along a normal with velocity vn; iden = 1/(1 - v^2 c^2) (their root is 0 where
+// rounding leaves v^2 = 1)
+__device__ __forceinline__ void rhd_speeds(double v2, double c2, double cs, double iden, double vn, double &lm, double &lp)
+{
+    const double disc = qsqrt((1.0 - v2) * (1.0 - v2 * c2 - vn * vn * (1.0 - c2)));
+    lm = (vn * (1.0 - c2) - cs * disc) * iden;
+    lp = (vn * (1.0 - c2) + cs * disc) * iden;
+}
 template <typename R> __device__ __forceinline__ R fab(R x);
 template <> __device__ __forceinline__ double fab<double>(double x) { return fabs(x); }
 template <> __device__ __forceinline__ float fab<float>(float x) { return fabsf(x); }

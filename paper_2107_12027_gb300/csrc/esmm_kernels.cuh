@@ -302,7 +302,7 @@ __global__ void k_cfl(ProbArg pa, double gam, double gg, const double *__restric
         double vx = q[Q_UX * g.P + c] * iW, vy = q[Q_UY * g.P + c] * iW;
         double v2 = vx * vx + vy * vy;
         double rh = rho + p * gg;
-        const double c2 = gam * p * qrcp<double>(rh), cs = c2 * qrsq<double>(c2);
+        const double c2 = gam * p * qrcp<double>(rh), cs = qsqrt(c2);
         double iJ = __drcp_rn(J[id]);
         const double iden = qrcp<double>(1.0 - v2 * c2);   // the same for both directions
 #pragma unroll
@@ -310,8 +310,8 @@ __global__ void k_cfl(ProbArg pa, double gam, double gg, const double *__restric
             double mx = q[(Q_M00 + 2 * k) * g.P + c], my = q[(Q_M01 + 2 * k) * g.P + c];
             const double n2 = mx * mx + my * my, iL = qrsq<double>(n2), Lk = n2 * iL;
             double vn = (mx * vx + my * vy) * iL;
-            const double d2 = (1.0 - v2) * (1.0 - v2 * c2 - vn * vn * (1.0 - c2)), disc = d2 * qrsq<double>(d2);
-            double lm = (vn * (1.0 - c2) - cs * disc) * iden, lp = (vn * (1.0 - c2) + cs * disc) * iden;
+            double lm, lp;
+            rhd_speeds(v2, c2, cs, iden, vn, lm, lp);
             r[k] = owned_row(g, j) ? Lk * fmax(fabs(lm), fabs(lp)) * iJ : 0.0;
             if (cflb) {
                 cflb[(2 + k) * g.N + id] = Lk * lm * iJ;
