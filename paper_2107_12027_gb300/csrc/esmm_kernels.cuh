@@ -302,7 +302,7 @@ __global__ void k_cfl(ProbArg pa, double gam, double gg, const double *__restric
         double vx = q[Q_UX * g.P + c] * iW, vy = q[Q_UY * g.P + c] * iW;
         double v2 = vx * vx + vy * vy;
         double rh = rho + p * gg;
-        const double c2 = gam * p * qrcp<double>(rh), cs = qsqrt(c2);
+        const double c2 = gam * p * qrcp<double>(rh), cs = c2 * qrsq<double>(c2);
         double iJ = __drcp_rn(J[id]);
         const double iden = qrcp<double>(1.0 - v2 * c2);   // the same for both directions
 #pragma unroll
