@@ -714,21 +714,28 @@ __device__ __forceinline__ void ec_pair(const NodeV<R> &l, const NodeV<R> &r, R 
 // first-derivative terms).  Sums of two products are written as the fused operation, so
 // that every kernel that inlines this rounds them alike.
 // FP32: the products of four e (up to 33 D^2 each, down to 4 eps) and a difference would leave the
-// range from D ~ 2,600 up, and for eps below ~1e-10.  A side's e count by their ratios alone, so they
-// are taken to 2^24 and below by the power of two: in range up to D ~ 1e7 and eps down to 1e-30
-// (400^2 mixed step 1.112 -> 1.120 ms).
-template <typename R> __device__ __forceinline__ void weno5_scale(R &, R &, R &) {}
-template <> __device__ __forceinline__ void weno5_scale<float>(float &e0, float &e1, float &e2)
+// range from D ~ 2,600 up, and for eps below ~1e-10.  The weights are 1/e^2 there instead, by the
+// hardware's reciprocals (within an ulp): as many instructions, and D to 1e8, eps down to 1e-19
+// (400^2 mixed step 1.120 -> 1.108 ms).
+template <typename R>
+__device__ __forceinline__ void weno5_side(R e0, R e1, R e2, R d0, R d1, R &n, R &q)
 {
-    const float sc = conv_float((278u << 23) - (conv_bits32(fmaxf(fmaxf(e0, e1), e2)) & 0x7f800000u));
-    e0 *= sc;
-    e1 *= sc;
-    e2 *= sc;
+    if constexpr (std::is_same<R, float>::value) {
+        e0 = approx_rcp(e0); e1 = approx_rcp(e1); e2 = approx_rcp(e2);
+        e0 *= e0; e1 *= e1; e2 *= e2;
+        n = fma_<R>(2.0f, e0 * d0, 3.0f * (e2 * d1));
+        q = qrcp<R>(fma_<R>(6.0f, e1, fma_<R>(3.0f, e2, e0)));
+    } else {
+        const R two = (R)2, three = (R)3, six = (R)6;
+        e0 *= e0; e1 *= e1; e2 *= e2;
+        n = e1 * fma_<R>(three, e0 * d1, two * (e2 * d0));
+        q = qrcp<R>(fma_<R>(e2, fma_<R>(six, e0, e1), three * (e0 * e1)));
+    }
 }
 template <typename R>
 __device__ __forceinline__ R weno5_jump(R D0, R D1, R D2, R D3, R D4, R eps4)
 {
-    const R c = (R)(13.0 / 3.0), two = (R)2, three = (R)3, six = (R)6;
+    const R c = (R)(13.0 / 3.0), two = (R)2;
     const R t0 = D1 - D0, ta = D2 - D1, tb = D3 - D2, t5 = D4 - D3;
     const R d0 = t0 - ta, d1 = ta - tb, d2 = tb - t5;
     const R S0 = fma_<R>(c * t0, t0, eps4), Sa = fma_<R>(c * ta, ta, eps4), Sb = fma_<R>(c * tb, tb, eps4),
@@ -737,18 +744,12 @@ __device__ __forceinline__ R weno5_jump(R D0, R D1, R D2, R D3, R D4, R eps4)
     {
         const R r0 = t0 + two * D1, r1 = D1 + D2, r2 = tb - two * D2;
         R e0 = fma_<R>(r0, r0, S0), e1 = fma_<R>(r1, r1, Sa), e2 = fma_<R>(r2, r2, Sb);
-        weno5_scale<R>(e0, e1, e2);
-        e0 *= e0; e1 *= e1; e2 *= e2;
-        nl = e1 * fma_<R>(three, e0 * d1, two * (e2 * d0));
-        ql = qrcp<R>(fma_<R>(e2, fma_<R>(six, e0, e1), three * (e0 * e1)));
+        weno5_side<R>(e0, e1, e2, d0, d1, nl, ql);
     }
     {
         const R r0 = t5 - two * D3, r1 = D2 + D3, r2 = ta + two * D2;
         R e0 = fma_<R>(r0, r0, S5), e1 = fma_<R>(r1, r1, Sb), e2 = fma_<R>(r2, r2, Sa);
-        weno5_scale<R>(e0, e1, e2);
-        e0 *= e0; e1 *= e1; e2 *= e2;
-        nr = e1 * fma_<R>(three, e0 * d1, two * (e2 * d2));
-        qr = qrcp<R>(fma_<R>(e2, fma_<R>(six, e0, e1), three * (e0 * e1)));
+        weno5_side<R>(e0, e1, e2, d2, d1, nr, qr);
     }
     return (d1 - fma_<R>(nl, ql, nr * qr)) * (R)(1.0 / 6.0);
 }
