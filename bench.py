@@ -73,24 +73,24 @@ FLOPS_PER_IFACE_F32 = None
 TRAFFIC_IFACE_F32 = None
 # The same for the RMHD interface kernels at p = 2, WENO5, on the 512^2 rotor, the
 # mean of the two sweeps (whose ambient field leaves other clusters of speeds in each):
-# FP64 5,180 and 6,634 flops per interface, 140 and 592 MB of DRAM traffic per launch;
-# FP32 6,212 and 7,027 FP32 flops besides 70 FP64 ones, 72 and 271 MB.  The 3D
-# kernel has not been recaptured since its waves came in closed form (the figures are of
-# the Gram form; its digest below is of those sources, so the bench reports none).
-FLOPS_PER_IFACE_MHD2 = 5907
-TRAFFIC_IFACE_MHD2 = 0.366e9
-FLOPS_PER_IFACE_MHD2_F32 = 6620
-TRAFFIC_IFACE_MHD2_F32 = 0.172e9
-FLOPS_PER_IFACE_MHD3 = 16265
-TRAFFIC_IFACE_MHD3 = 9.62e9
+# FP64 5,214 and 6,556 flops per interface, 154 and 610 MB of DRAM traffic per launch;
+# FP32 6,291 and 6,919 FP32 flops besides 70 FP64 ones, 73 and 268 MB.  The 3D
+# kernel on the 64^3 blast, the mean of its three sweeps (5,520, 6,903 and 7,032 flops, 434,
+# 982 and 986 MB), the traffic times 7.94 for a 128^3 launch's interfaces.
+FLOPS_PER_IFACE_MHD2 = 5885
+TRAFFIC_IFACE_MHD2 = 0.382e9
+FLOPS_PER_IFACE_MHD2_F32 = 6605
+TRAFFIC_IFACE_MHD2_F32 = 0.170e9
+FLOPS_PER_IFACE_MHD3 = 6485
+TRAFFIC_IFACE_MHD3 = 6.36e9
 # The fused sweep kernel (pair and interface fluxes in one launch) on the
 # same workload, from one capture of each form: executed flops per interface
 # (its pair fluxes included: 32 anchors per 31 interfaces) and DRAM bytes
 # per launch; None whenever the kernel has changed since.
 FLOPS_PER_SWEEP_F64 = 1117
-TRAFFIC_SWEEP_F64 = 13.18e6
-FLOPS_PER_SWEEP_F32 = 1072
-TRAFFIC_SWEEP_F32 = 9.20e6
+TRAFFIC_SWEEP_F64 = 13.2e6
+FLOPS_PER_SWEEP_F32 = 1040
+TRAFFIC_SWEEP_F32 = 9.2e6
 # The counters above were captured on kernels built from these sources. The
 # bench reports a kernel's counters only while its sources still hash to the
 # digest recorded at that capture: an edit of any of them drops that
@@ -101,7 +101,7 @@ COUNTER_SOURCES = {
     "mhd2": ("esmm_mhd.cuh", "esmm_mhd_waves.cuh", "esmm_device.cuh", "esmm_conv.h"),
     "mhd3": ("esmm_3d.cuh", "esmm_3d_iface.cu", "esmm_mhd.cuh", "esmm_mhd_waves.cuh", "esmm_device.cuh", "esmm_conv.h"),
 }
-COUNTER_DIGEST = {"sweep": "929ee2bdf445f782", "mhd2": "53088b2c47c2d899", "mhd3": "dd8daf5262c5c5b3"}
+COUNTER_DIGEST = {"sweep": "5c0be8c7c4ecca2b", "mhd2": "4eacf2817fd4c409", "mhd3": "06745601692cedb2"}
 
 
 def source_digest(kind, csrc=None):

@@ -65,10 +65,12 @@ extern "C" {
 #define ESMM_MEM_HOST 0
 #define ESMM_MEM_DEVICE 1
 
-#define ESMM_FP64 0         /* every step in FP64                              */
+#define ESMM_FP64 0         /* every value in FP64; FP32 starts the root
+                               searches, steers their Newton steps and takes
+                               the decisions that are clear in it             */
 #define ESMM_MIXED 1        /* fluxes, WENO and metrics in FP32 (log means' jumps
-                               from FP64 values); FP64 for the primitive
-                               recovery, the state, and all totals              */
+                               from 48 bits of the FP64 values); FP64 for the
+                               primitive recovery, the state, and all totals  */
 
 #define ESMM_MONITOR_RHO 0  /* monitor variable sigma = rho                    */
 #define ESMM_MONITOR_LNRHO 1/* monitor variable sigma = ln rho                 */
